@@ -29,8 +29,8 @@
 //               tile, ahead of the epilogue
 //   warps 4-11  epilogue: tcgen05.ld, int32 accumulation across chunks, dequantizing
 //               multiply, TMA stores of 32 x 32 boxes (or int32 TMA reductions into a
-//               split-K workspace; plain stores where the output rows are not 16-byte
-//               aligned)
+//               split-K workspace; direct 32-byte stores on pair tiles; plain stores where
+//               the output rows are not 16-byte aligned)
 // Work units reach the roles through a small shared-memory ring that the producer of the
 // CTA (a pair's leader) fills: with a scheduling counter it takes each next unit from it
 // (units are handed out in list order as CTAs free up), without one it strides over the
@@ -106,6 +106,7 @@ struct GemmParams {
   int mode;  // 0: per-column scale (forward, loss propagation); 1: row/column shifts (wgrad)
   int G;
   int vec_y;  // output rows 16-byte aligned: 16-byte stores
+  int vec_y32;  // ... 32-byte aligned
   const float* a_scale;
   const float* b_scale;
   const uint8_t* row_exp;
@@ -215,11 +216,39 @@ __device__ __noinline__ void write_acc_box(long long* acc, int64_t ld_acc, int64
 // as int32 partial sums through a TMA reduce-add into the split-K workspace, or -- past the
 // int32 range -- as int64 additions (64-bit atomics, a row of 32 columns per instruction)
 // into the int64 workspace.  The exactness-check integers are written when asked.
+// kDirect (pair tiles): a plain fp32 box whose rows are 32-byte aligned skips the staging --
+// each lane stores its row's 32 columns as four 32-byte sectors.  In a pair the tensor core
+// takes most of the shared-memory bandwidth, and a box's staging writes, its TMA reads and
+// the wait for them cost the MMAs more than the sector-wise stores cost L2: layer launches
+// of 12608 x 768 x 3072 (6-bit) 165.4 -> 155.7 us, 4096 x 11008 x 4096 (8-bit) 715 -> 703 us,
+// 16384 x 4096 x 11008 (6-bit) 2139 -> 2125 us.  Single tiles keep the staged TMA stores:
+// their launches are bound by the output stream, which full 128-byte lines serve better
+// (12544 x 2304 x 256, 4-bit: 57.9 us staged, 64.6 us direct; every second box direct 62.1).
+template <bool kDirect>
 __device__ __forceinline__ void emit_box(const GemmParams& p, const CUtensorMap* tma_y,
                                          const CUtensorMap* tma_ws, const uint32_t (&vals)[32],
                                          bool as_float, uint32_t fac, float rfac, uint32_t buf,
                                          int64_t row0, int64_t col0, int lane) {
   const bool tma_out = p.ws != nullptr ? !p.wide : p.vec_y != 0;
+  if (kDirect && p.vec_y32 && p.ws == nullptr && p.acc == nullptr && p.colmax == nullptr &&
+      col0 + kOutBox <= p.N) {
+    float* dst = p.y + (row0 + lane) * p.ldy + col0;
+    const bool in = row0 + lane < p.M;
+#pragma unroll
+    for (int k = 0; k < kOutBox / 8; ++k) {
+      const float4 fa = ld_shared_v4_f32(fac + k * 32), fb = ld_shared_v4_f32(fac + k * 32 + 16);
+      const float f[8] = {fa.x, fa.y, fa.z, fa.w, fb.x, fb.y, fb.z, fb.w};
+      float o[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const uint32_t a = vals[k * 8 + e];
+        const float val = as_float ? __uint_as_float(a) : __int2float_rn(static_cast<int32_t>(a));
+        o[e] = __fmul_rn(p.mode == 1 ? __fmul_rn(val, rfac) : val, f[e]);
+      }
+      if (in) st_global_v8(dst + k * 8, o);
+    }
+    return;
+  }
   if (lane == 0) {
     // the last TMA store has read the box (it may belong to another GEMM of the launch,
     // whatever this box's own way out)
@@ -1006,7 +1035,7 @@ __global__ void __launch_bounds__(kThreads, 1) shiftmm_kernel(const __grid_const
           const int64_t col0 = n0 + h * 128 + s * 32;
           if (row0 >= p.M || col0 >= p.N) continue;  // warp-uniform: nothing of this box exists
           const uint32_t buf = stage_out0;
-          emit_box(p, tma_y, tma_ws, v, true, smem_u32(fac + h * 128 + s * 32), rfac, buf, row0,
+          emit_box<kPair>(p, tma_y, tma_ws, v, true, smem_u32(fac + h * 128 + s * 32), rfac, buf, row0,
                            col0, lane);
         }
         __syncwarp();
@@ -1079,7 +1108,7 @@ __global__ void __launch_bounds__(kThreads, 1) shiftmm_kernel(const __grid_const
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[i] = acc[s * 32 + i];
           const uint32_t buf = stage_out0;
-          emit_box(p, tma_y, tma_ws, v, false, smem_u32(fac + h * 128 + s * 32), rfac, buf, row0,
+          emit_box<kPair>(p, tma_y, tma_ws, v, false, smem_u32(fac + h * 128 + s * 32), rfac, buf, row0,
                            col0, lane);
         }
         __syncwarp();
@@ -1577,6 +1606,7 @@ static int prepare_job(const GemmJob& j, const Plan* pl, int bits, int G, int32_
   p.mode = j.which == 2 ? 1 : 0;
   p.G = G;
   p.vec_y = (j.ldy % 4 == 0) && aligned16(j.y);
+  p.vec_y32 = (j.ldy % 8 == 0) && (reinterpret_cast<uintptr_t>(j.y) & 31u) == 0;
   p.a_scale = j.a_scale;
   p.b_scale = j.b_scale;
   p.row_exp = j.row_exp;
