@@ -48,6 +48,21 @@ __device__ __forceinline__ float4 ld_nc_v4(const float* p) {
   return v;
 }
 
+// ------------------------------------------------------------------ asynchronous copies
+// 16 bytes (bypassing L1), or 4 bytes, of global memory into shared memory; zeros when !in
+// (src is not read then, but must be a valid address)
+__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, bool in) {
+  asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+               "r"(in ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_4(uint32_t dst, const void* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
 // ----------------------------------------------------- programmatic dependent launch
 // Wait until the preceding kernel of the stream has completed and its writes are visible
 // (a no-op for a kernel launched without programmatic stream serialization).
@@ -269,6 +284,45 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c),
                "r"(d)
                : "memory");
+}
+
+__device__ __forceinline__ uint4 ld_shared_v4_u32(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ uint2 ld_shared_v2_u32(uint32_t addr) {
+  uint2 v;
+  asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_shared_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t a) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(a) : "memory");
+}
+// one code (1 or 2 bytes)
+template <typename CodeT>
+__device__ __forceinline__ CodeT ld_shared_code(uint32_t addr) {
+  uint16_t v;
+  if constexpr (sizeof(CodeT) == 2) {
+    asm volatile("ld.shared.b16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
+  } else {
+    asm volatile("{\n\t.reg .b32 t;\n\tld.shared.u8 t, [%1];\n\tcvt.u16.u32 %0, t;\n\t}"
+                 : "=h"(v)
+                 : "r"(addr)
+                 : "memory");
+  }
+  return static_cast<CodeT>(v);
 }
 
 // one 32-byte sector: dst 32-byte aligned

@@ -43,6 +43,7 @@
 
 #include <cstring>
 #include <mutex>
+#include <new>
 
 #include "sq_device.cuh"
 #include "sq_host.h"
@@ -738,6 +739,10 @@ __global__ void __launch_bounds__(kThreads, 1) shiftmm_kernel(const __grid_const
   else
     __syncthreads();
   tc_fence_after();
+  // launched behind the preceding kernel (programmatic stream serialization): everything up to
+  // here runs beside its tail, nothing it wrote is read before it has completed
+  griddep_wait();
+  griddep_launch_dependents();
   const uint32_t tmem_base = *tmem_slot;
   const int units = bt.unit_end[bt.count - 1];
   constexpr int kBKElems = kF8 ? kBKBytes : kBKBytes / 2;
@@ -1139,6 +1144,7 @@ __global__ void __launch_bounds__(kThreads, 1) shiftmm_kernel(const __grid_const
 // split-K: turn the summed int32 partials into the outputs, four consecutive outputs of a
 // row per thread (a split GEMM has N % 4 == 0); every load of a thread leaves at once
 __global__ void __launch_bounds__(256) splitk_finalize_kernel(const GemmParams p) {
+  griddep_wait();
   const float a_fac = epilogue_a_factor(p);
   const int nq = p.N / 4;
   const int64_t quads = static_cast<int64_t>(p.M) * nq;
@@ -1176,6 +1182,7 @@ __global__ void __launch_bounds__(256) splitk_finalize_kernel(const GemmParams p
 // The same from int64 sums (a K loop beyond the int32 range), one output per thread: the one
 // dequantizing multiply of the epilogue with T converted to FP32 once (round to nearest).
 __global__ void __launch_bounds__(256) splitk_finalize_wide_kernel(const GemmParams p) {
+  griddep_wait();
   const float a_fac = epilogue_a_factor(p);
   const long long* ws = reinterpret_cast<const long long*>(p.ws);
   const int64_t n = static_cast<int64_t>(p.M) * p.N;
@@ -1632,26 +1639,22 @@ template <int kF8, bool kMulti, bool kPair, bool kMn>
 static int launch_kernel(const GemmBatch& bt, int grid, int dev, cudaStream_t s) {
   const int st = configure_kernel<kF8, kMulti, kPair, kMn>(dev);
   if (st != SQ_OK) return st;
-  cudaError_t err;
-  if constexpr (kPair) {
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = Smem<true>::bytes;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    err = cudaLaunchKernelEx(&cfg, shiftmm_kernel<kF8, kMulti, true, kMn>, bt);
-    if (err == cudaSuccess) err = cudaGetLastError();
-  } else {
-    shiftmm_kernel<kF8, kMulti, false, kMn><<<grid, kThreads, Smem<false>::bytes, s>>>(bt);
-    err = cudaGetLastError();
-  }
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 2;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = Smem<kPair>::bytes;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = kPair ? 2 : 1;
+  cudaError_t err = cudaLaunchKernelEx(&cfg, shiftmm_kernel<kF8, kMulti, kPair, kMn>, bt);
+  if (err == cudaSuccess) err = cudaGetLastError();
   return err == cudaSuccess ? SQ_OK : cuda_fail(err, "shiftmm_kernel launch");
 }
 
@@ -1665,14 +1668,26 @@ static int launch_variant(const GemmBatch& bt, int grid, int dev, cudaStream_t s
                : launch_kernel<kF8, false, false, kMn>(bt, grid, dev, s);
 }
 
-// Checks, plans and launches up to kMaxBatch GEMMs (all with the same bits / n_groups) as
-// one persistent kernel; split-K partial sums are zeroed before and finalized after it.
-// sched (may be null): a unit counter, zeroed here before the launch, through which the
+// A checked and planned launch: what issue_jobs needs.
+struct JobPlan {
+  GemmBatch bt;
+  int grid, dev, sms;
+  bool multi, pair, mn, partial;
+  int elem_bytes;
+  ZeroRegion zero[kMaxBatch + 1];   // to be zeroed before the launch (the counter, partial sums)
+  int nzero;
+};
+
+// Checks and plans up to kMaxBatch GEMMs (all with the same bits / n_groups) as one persistent
+// kernel; split-K partial sums are zeroed before and finalized after it.
+// sched (may be null): a unit counter, zero before the launch, through which the
 // CTAs take their units as they free up -- for batches whose units differ in length.
 // Without one each CTA strides over the unit list.
-static int run_jobs(GemmJob* jobs, int njobs, int bits, int G, int32_t* dev_status, void* stream,
-                    int* sched, int max_ctas = 0, bool no_copies = false) {
-  cudaStream_t s = as_stream(stream);
+// counter_zeroed: the caller clears the counter word itself, it is not among the regions.
+// *live is false when there is nothing to launch.
+static int plan_jobs(GemmJob* jobs, int njobs, int bits, int G, int32_t* dev_status, cudaStream_t s,
+                     int* sched, int max_ctas, bool no_copies, bool counter_zeroed, JobPlan* jp, bool* have) {
+  *have = false;
   int live[kMaxBatch];
   int nlive = 0;
   for (int i = 0; i < njobs; ++i)
@@ -1694,7 +1709,7 @@ static int run_jobs(GemmJob* jobs, int njobs, int bits, int G, int32_t* dev_stat
   int dev = 0;
   const int sms = device_sms(&dev);
   if (sms <= 0) return fail(SQ_ECUDA, "%s: no current CUDA device", job_name(jobs[live[0]].which));
-  GemmBatch bt;
+  GemmBatch& bt = jp->bt;
   memset(&bt, 0, sizeof(bt));
   Plan plans[kMaxBatch];
   GemmJob* lj[kMaxBatch];
@@ -1746,27 +1761,21 @@ static int run_jobs(GemmJob* jobs, int njobs, int bits, int G, int32_t* dev_stat
     bt.planned |= bt.k_exp[g] != nullptr || bt.seg[g] != nullptr;
     bt.segmented |= bt.seg[g] != nullptr;
   }
-  // zero the counter and the partial sums, with one memset for the regions that follow the
+  // the counter and the partial sums start at zero: one region for those that follow the
   // counter back to back
-  char* zero_from = reinterpret_cast<char*>(sched);
-  char* zero_end = sched ? zero_from + kSchedBytes : nullptr;
-  cudaError_t err;
+  jp->nzero = 0;
+  if (sched != nullptr && !counter_zeroed) jp->zero[jp->nzero++] = {sched, kSchedBytes};
   for (int g = 0; g < nlive; ++g) {
     if (!bt.p[g].ws) continue;
     char* w = reinterpret_cast<char*>(bt.p[g].ws);
     // a partial call's sums go to the caller's buffer of exactly M N words
     const size_t b = partial ? static_cast<size_t>(bt.p[g].M) * bt.p[g].N * sizeof(int)
                              : split_ws_bytes(bt.p[g].M, bt.p[g].N, bt.p[g].wide != 0);
-    if (zero_end != nullptr && w == zero_end) {
-      zero_end = w + b;
-      continue;
-    }
-    err = cudaMemsetAsync(w, 0, b, s);
-    if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync");
-  }
-  if (zero_from != nullptr) {
-    err = cudaMemsetAsync(zero_from, 0, static_cast<size_t>(zero_end - zero_from), s);
-    if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync");
+    ZeroRegion* last = jp->nzero > 0 ? &jp->zero[jp->nzero - 1] : nullptr;
+    if (last != nullptr && w == static_cast<char*>(last->p) + last->bytes)
+      last->bytes += b;
+    else
+      jp->zero[jp->nzero++] = {w, b};
   }
   // CTA groups (pairs, or single CTAs); a cap on the CTAs leaves at least one group
   const int cg = pair ? 2 : 1;
@@ -1785,26 +1794,63 @@ static int run_jobs(GemmJob* jobs, int njobs, int bits, int G, int32_t* dev_stat
   }
   bool mn = false;
   for (int g = 0; g < nlive; ++g) mn |= bt.mn[g] != 0;
-  if (plans[0].elem_bytes == 1)
-    st = mn ? launch_variant<1, true>(bt, grid, dev, s, multi, pair)
-            : launch_variant<1, false>(bt, grid, dev, s, multi, pair);
+  jp->grid = grid;
+  jp->dev = dev;
+  jp->sms = sms;
+  jp->multi = multi;
+  jp->pair = pair;
+  jp->mn = mn;
+  jp->partial = partial;
+  jp->elem_bytes = plans[0].elem_bytes;
+  *have = true;
+  return SQ_OK;
+}
+
+// Issues a planned launch and the output passes of its split GEMMs; the plan's regions are
+// zero when the stream gets there.
+static int issue_jobs(const JobPlan& jp, cudaStream_t s) {
+  int st;
+  if (jp.elem_bytes == 1)
+    st = jp.mn ? launch_variant<1, true>(jp.bt, jp.grid, jp.dev, s, jp.multi, jp.pair)
+               : launch_variant<1, false>(jp.bt, jp.grid, jp.dev, s, jp.multi, jp.pair);
   else
-    st = mn ? launch_variant<0, true>(bt, grid, dev, s, multi, pair)
-            : launch_variant<0, false>(bt, grid, dev, s, multi, pair);
+    st = jp.mn ? launch_variant<0, true>(jp.bt, jp.grid, jp.dev, s, jp.multi, jp.pair)
+               : launch_variant<0, false>(jp.bt, jp.grid, jp.dev, s, jp.multi, jp.pair);
   if (st != SQ_OK) return st;
-  for (int g = 0; g < nlive; ++g) {
-    if (!bt.p[g].ws || partial) continue;
-    const int64_t items = static_cast<int64_t>(bt.p[g].M) * (bt.p[g].wide ? bt.p[g].N : bt.p[g].N / 4);
+  for (int g = 0; g < jp.bt.count; ++g) {
+    const GemmParams& p = jp.bt.p[g];
+    if (!p.ws || jp.partial) continue;
+    const int64_t items = static_cast<int64_t>(p.M) * (p.wide ? p.N : p.N / 4);
     int64_t blocks = (items + 255) / 256;
-    if (blocks > static_cast<int64_t>(sms) * 16) blocks = static_cast<int64_t>(sms) * 16;
-    if (bt.p[g].wide)
-      splitk_finalize_wide_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(bt.p[g]);
-    else
-      splitk_finalize_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(bt.p[g]);
-    err = cudaGetLastError();
+    if (blocks > static_cast<int64_t>(jp.sms) * 16) blocks = static_cast<int64_t>(jp.sms) * 16;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaError_t err = cudaLaunchKernelEx(&cfg, p.wide ? splitk_finalize_wide_kernel : splitk_finalize_kernel, p);
+    if (err == cudaSuccess) err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_fail(err, "splitk_finalize_kernel launch");
   }
   return SQ_OK;
+}
+
+static int run_jobs(GemmJob* jobs, int njobs, int bits, int G, int32_t* dev_status, void* stream,
+                    int* sched, int max_ctas = 0, bool no_copies = false) {
+  cudaStream_t s = as_stream(stream);
+  JobPlan jp;
+  bool have = false;
+  const int st = plan_jobs(jobs, njobs, bits, G, dev_status, s, sched, max_ctas, no_copies, false, &jp, &have);
+  if (st != SQ_OK || !have) return st;
+  for (int k = 0; k < jp.nzero; ++k) {
+    const cudaError_t err = cudaMemsetAsync(jp.zero[k].p, 0, jp.zero[k].bytes, s);
+    if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync");
+  }
+  return issue_jobs(jp, s);
 }
 
 static int run_gemm(int which, const void* a_codes, int64_t lda, const void* b_codes, int64_t ldb,
@@ -2080,10 +2126,11 @@ extern "C" sq_status shiftquant_gemm_wgrad_static(
                   scratch ? kStaticScratchBytes : 0, dev_status, stream);
 }
 
-extern "C" sq_status shiftquant_gemm_layer(const sq_layer_gemms* args, void* workspace,
-                                           size_t workspace_bytes, int32_t* dev_status,
-                                           void* stream) {
-  fail(SQ_OK, "");
+namespace sq {
+
+// the argument checks of a layer launch and its jobs over the workspace
+static int prepare_layer(const sq_layer_gemms* args, void* workspace, size_t workspace_bytes, GemmJob jobs[3],
+                         int** sched) {
   if (args == nullptr) return fail(SQ_EINVAL, "gemm_layer: args is NULL");
   if (!bits_ok(args->bits) || !groups_ok(args->n_groups))
     return fail(SQ_EINVAL, "gemm_layer: bits must be in [2, 8] and n_groups in [1, 8]");
@@ -2094,12 +2141,45 @@ extern "C" sq_status shiftquant_gemm_layer(const sq_layer_gemms* args, void* wor
                 (args->gt_codes == nullptr && args->g_seg != nullptr)))
     return fail(SQ_EINVAL, "gemm_layer: a group-ordered operand needs its transposed copy "
                 "(xt_codes / gt_codes) for the weight gradient");
-  GemmJob jobs[3];
   layer_jobs(args, jobs, args->gemm_mask);
   const int sms = device_sms(nullptr);
   const int pairs = device_pairs(nullptr);
-  int* sched =
-      assign_layer_ws(jobs, args->bits, args->n_groups, sms, pairs, workspace, workspace_bytes);
+  *sched = assign_layer_ws(jobs, args->bits, args->n_groups, sms, pairs, workspace, workspace_bytes);
+  return SQ_OK;
+}
+
+static_assert(sizeof(JobPlan) + sizeof(bool) <= sizeof(LayerPlan), "LayerPlan holds a JobPlan");
+
+int plan_layer_gemms(const sq_layer_gemms* args, void* workspace, size_t workspace_bytes, int32_t* dev_status,
+                     LayerPlan* plan, ZeroRegion* zero, int* nzero) {
+  GemmJob jobs[3];
+  int* sched = nullptr;
+  int st = prepare_layer(args, workspace, workspace_bytes, jobs, &sched);
+  if (st != SQ_OK) return st;
+  JobPlan* jp = new (plan->bytes) JobPlan;
+  bool have = false;
+  st = plan_jobs(jobs, 3, args->bits, args->n_groups, dev_status, nullptr, sched, args->max_ctas, false, true, jp, &have);
+  if (st != SQ_OK) return st;
+  if (!have) return fail(SQ_EINVAL, "gemm_layer: nothing to launch");
+  *nzero = jp->nzero;
+  for (int k = 0; k < jp->nzero; ++k) zero[k] = jp->zero[k];
+  return SQ_OK;
+}
+
+int issue_layer_gemms(const LayerPlan* plan, cudaStream_t s) {
+  return issue_jobs(*reinterpret_cast<const JobPlan*>(plan->bytes), s);
+}
+
+}  // namespace sq
+
+extern "C" sq_status shiftquant_gemm_layer(const sq_layer_gemms* args, void* workspace,
+                                           size_t workspace_bytes, int32_t* dev_status,
+                                           void* stream) {
+  fail(SQ_OK, "");
+  GemmJob jobs[3];
+  int* sched = nullptr;
+  const int st = prepare_layer(args, workspace, workspace_bytes, jobs, &sched);
+  if (st != SQ_OK) return st;
   return run_jobs(jobs, 3, args->bits, args->n_groups, dev_status, stream, sched, args->max_ctas);
 }
 

@@ -37,4 +37,31 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 inline cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 
+// ------------------------------------------------------------ one layer step's parts
+// device memory a launch wants zeroed before it (16-byte aligned, a multiple of 16 bytes)
+struct ZeroRegion {
+  void* p;
+  size_t bytes;
+};
+
+// The quantizer's argument checks of a layer step (non-empty, required pointers checked).
+int check_layer_quant(const sq_layer_step* L);
+// whether the passes of quantize_layer can index the layer's tiles
+bool layer_quant_fits(const sq_layer_step* L);
+// The quantizer passes of a checked layer step in three launches, and the zero regions
+// cleared.  words: 256 bytes of device memory, of which the first 64 are left zero and the
+// rest is the passes' own.
+int quantize_layer(const sq_layer_step* L, uint64_t seed, unsigned* words, const ZeroRegion* zero, int nzero,
+                   cudaStream_t s);
+
+// The GEMM launch of a layer step: planned (checks included) into `plan`, then issued on the
+// stream once the operands' launches are.  zero receives the regions (at most 3) that must be
+// zeroed before, besides the counter word at the start of the workspace.
+struct alignas(64) LayerPlan {
+  char bytes[4096];
+};
+int plan_layer_gemms(const sq_layer_gemms* args, void* workspace, size_t workspace_bytes, int32_t* dev_status,
+                     LayerPlan* plan, ZeroRegion* zero, int* nzero);
+int issue_layer_gemms(const LayerPlan* plan, cudaStream_t s);
+
 }  // namespace sq

@@ -18,6 +18,7 @@
 
 #include <cstdarg>
 #include <cstdio>
+#include <cstring>
 
 #include "sq_device.cuh"
 #include "sq_host.h"
@@ -118,97 +119,137 @@ __global__ void __launch_bounds__(THREADS)
   }
 }
 
+// A tensor as the range pass reads it.  A dense tensor whose rows are not 16-byte aligned is
+// folded: `fold` rows (2 or 4, so that they make whole 16-byte vectors) become one row of
+// fold x cols columns, whose column c stands for column c mod creal, plus `tail` elements of a
+// last partial row; every load is then an aligned vector.  Other unaligned tensors are read
+// element by element, the lanes on consecutive columns.
+enum ViewForm { kViewVec, kViewFolded, kViewStrided };
+
+struct RangeView {
+  const float* x;
+  int64_t R, C, ld;
+  int form;        // ViewForm
+  int64_t creal;   // columns of the tensor (C / creal rows are folded into one)
+  int64_t tail;    // elements of the partial row R (folded tensors)
+};
+
+// The column maxima (ordered bit patterns of |x|: for non-negative floats a larger value is a
+// larger pattern, NaN above Inf) of the thread's part of one tile of tc = 4 << lg columns by 8
+// passes of 1024 / tc rows from r0 on: four columns -- quad qc, or in strided views columns
+// qc + k 2^lg -- of rows r0 + u rpp, with all eight 16-byte loads in flight together.
+// ROWS: rm[u] becomes the maximum with row u's four values.
+template <bool ROWS, int FORM>
+__device__ __forceinline__ void tile_maxima(const RangeView& t, int lg, int64_t cb, int64_t r0, int qc,
+                                            unsigned (&m)[4], unsigned (&rm)[8]) {
+  const int rpp = (kColTx * kColTy) >> lg;
+  const int64_t c0 = cb + 4 * qc;
+  if (FORM != kViewStrided && c0 + 3 < t.C) {
+    // rows past the end re-read the last row, which leaves a maximum unchanged
+    float4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = ld_stream_v4(t.x + min(r0 + u * rpp, t.R - 1) * t.ld + c0);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const unsigned a[4] = {abs_bits(v[u].x), abs_bits(v[u].y), abs_bits(v[u].z), abs_bits(v[u].w)};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) m[k] = max(m[k], a[k]);
+      if (ROWS) rm[u] = max(rm[u], max(max(a[0], a[1]), max(a[2], a[3])));
+    }
+    if (FORM == kViewFolded && t.tail > 0 && r0 + 8 * rpp > t.R) {   // the last row tile takes the partial row too
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (c0 + k < t.tail) m[k] = max(m[k], abs_bits(__ldg(t.x + t.R * t.ld + c0 + k)));
+    }
+    return;
+  }
+  if (FORM == kViewFolded) return;   // whole quads only
+  const int64_t first = FORM == kViewVec ? c0 : cb + qc;   // (kViewVec: the last columns of padded rows)
+  const int step = FORM == kViewVec ? 1 : 1 << lg;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const float* row = t.x + min(r0 + u * rpp, t.R - 1) * t.ld;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t c = first + k * step;
+      const unsigned a = c < t.C ? abs_bits(__ldg(row + c)) : 0u;
+      m[k] = max(m[k], a);
+      if (ROWS) rm[u] = max(rm[u], a);
+    }
+  }
+}
+
+// the thread's column maxima to red[row pass ro][column]
+template <int FORM>
+__device__ __forceinline__ void put_maxima(unsigned* red, int lg, int ro, int qc, const unsigned (&m)[4]) {
+  const int tc = 4 << lg;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) red[ro * tc + (FORM != kViewStrided ? 4 * qc + k : qc + (k << lg))] = m[k];
+}
+
+// the accumulator of view column c
+template <int FORM>
+__device__ __forceinline__ unsigned* column_bits(unsigned* bits, const RangeView& t, int64_t c) {
+  return bits + (FORM == kViewFolded ? c % t.creal : c);
+}
+
+// the maximum of tile column `col` over the block's row passes
+__device__ __forceinline__ unsigned get_maximum(const unsigned* red, int lg, int col) {
+  const int tc = 4 << lg, rpp = (kColTx * kColTy) >> lg;
+  unsigned m = 0;
+  for (int y = 0; y < rpp; ++y) m = max(m, red[y * tc + col]);
+  return m;
+}
+
 // Range pass: block (x, y) reads tile (y, x) of TC = 4 << lg columns (the column count
-// rounded up to a power of two, 4 to 128) by 8 passes of 1024 / TC rows -- thread t owns
-// the four-column quad t mod (TC / 4) and the rows t / (TC / 4) + k 1024 / TC, with all
-// eight 16-byte loads in flight -- and takes its per-column maxima as ordered bit patterns
-// of the non-negative floats (NaN sorts above Inf), sent to range_bits with one atomic max
-// per column.  Same-address atomics from hundreds of tiles of a narrow tensor serialise in
-// L2, so narrow tensors (CL = kRangeCluster) run in clusters of CL blocks along the rows:
-// each block merges its maxima into the first block of its cluster with atomic maxima on
-// that block's shared memory, and only that block sends them on.  Wide tensors (CL = 1)
-// spread their atomics over many addresses and run without clusters, which schedule more
-// slowly.  Grids taller than the 65535-block limit
-// walk the extra tiles in steps of gridDim.y.
+// rounded up to a power of two, 4 to 128) by 8 passes of 1024 / TC rows, and sends its
+// per-column maxima to range_bits with one atomic max per column.  Same-address atomics from
+// hundreds of tiles of a narrow tensor serialise in L2, so narrow tensors (CL =
+// kRangeCluster) run in clusters of CL blocks along the rows: each block merges its maxima
+// into the first block of its cluster with atomic maxima on that block's shared memory, and
+// only that block sends them on.  Wide tensors (CL = 1) spread their atomics over many
+// addresses and run without clusters, which schedule more slowly.  Grids taller than the
+// 65535-block limit walk the extra tiles in steps of gridDim.y.
 // ROWS: the range pass of a weight for both of its roles -- also every row's max|x| over
 // all columns (the per-in-channel ranges), each warp's eight rows of a tile reduced across
 // its lanes and sent to row_bits with one atomic max per row and column block.
 constexpr int kRangeCluster = 8;
 constexpr int64_t kRangeClusterMaxCols = 512;   // clusters for tensors of at most 512 columns
 
-template <int CL, bool ROWS>
-__global__ void __launch_bounds__(kColTx* kColTy)
-    colmax_kernel(const float* __restrict__ x, int64_t R, int64_t C, int64_t ld, int vec, int lg,
-                  unsigned* __restrict__ range_bits, unsigned* __restrict__ row_bits,
-                  int* __restrict__ status) {
+template <int CL, bool ROWS, int FORM>
+__global__ void __launch_bounds__(kColTx* kColTy, ROWS || FORM == kViewStrided ? 4 : 6)
+    colmax_kernel(const RangeView v, int lg, unsigned* __restrict__ range_bits,
+                  unsigned* __restrict__ row_bits, int* __restrict__ status) {
   __shared__ unsigned red[kColTy * kColTx * 4];
   __shared__ unsigned cmax[CL > 1 ? kColTx * 4 : 1];   // the cluster's maxima (first block)
   const int tid = threadIdx.y * kColTx + threadIdx.x;
-  // the tile: tc = 4 << lg columns (one four-column quad per thread) by 8 passes of rpp rows
   const int tc = 4 << lg, rpp = (kColTx * kColTy) >> lg;
   const int qc = tid & ((1 << lg) - 1), ro = tid >> lg;
-  const int64_t c0 = static_cast<int64_t>(blockIdx.x) * tc + 4 * qc;
+  const int64_t cb = static_cast<int64_t>(blockIdx.x) * tc;
   const int64_t tile_rows = 8 * static_cast<int64_t>(rpp);
-  const int64_t tiles = (R + tile_rows - 1) / tile_rows;
+  const int64_t tiles = (v.R + tile_rows - 1) / tile_rows;
   if (CL > 1) {
     if (tid < kColTx * 4) cmax[tid] = 0u;
     cluster_arrive_release();   // the zeroed cmax is visible to the cluster after the wait
   }
-  unsigned m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+  unsigned m[4] = {0u, 0u, 0u, 0u};
   bool row_bad = false;
 #pragma unroll 1
   for (int64_t t = blockIdx.y; t < tiles; t += gridDim.y) {
     const int64_t r0 = t * tile_rows + ro;   // this thread's rows: r0 + u rpp
-    unsigned rm[8];   // ROWS: this thread's four columns of each of its rows
-    if (vec && c0 + 3 < C) {
-      // rows past the end re-read the last row, which leaves a maximum unchanged
-      float4 v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = ld_stream_v4(x + min(r0 + u * rpp, R - 1) * ld + c0);
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const unsigned a0 = abs_bits(v[u].x), a1 = abs_bits(v[u].y);
-        const unsigned a2 = abs_bits(v[u].z), a3 = abs_bits(v[u].w);
-        m0 = max(m0, a0);
-        m1 = max(m1, a1);
-        m2 = max(m2, a2);
-        m3 = max(m3, a3);
-        if (ROWS) rm[u] = max(max(a0, a1), max(a2, a3));
-      }
-    } else {
-#pragma unroll
-      for (int u = 0; u < 8; ++u) rm[u] = 0u;
-#pragma unroll 1
-      for (int u = 0; u < 8; ++u) {
-        const int64_t r = r0 + u * rpp;
-        if (r >= R) break;
-        const float* row = x + r * ld;
-        unsigned a[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (c0 + k < C) a[k] = abs_bits(__ldg(row + c0 + k));
-        m0 = max(m0, a[0]);
-        m1 = max(m1, a[1]);
-        m2 = max(m2, a[2]);
-        m3 = max(m3, a[3]);
-        if (ROWS) {
-#pragma unroll
-          for (int k = 0; k < 8; ++k)  // rm stays in registers: no run-time index
-            if (k == u) rm[k] = max(max(a[0], a[1]), max(a[2], a[3]));
-        }
-      }
-    }
+    unsigned rm[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};   // ROWS: this thread's columns of each of its rows
+    tile_maxima<ROWS, FORM>(v, lg, cb, r0, qc, m, rm);
     if (ROWS) {
       // (lg = 5: a warp's 32 quads are one row of the tile, a warp row per pass)
       // the row accumulators are zeroed by the preceding kernel, which must have completed
       griddep_wait();
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const unsigned m = __reduce_max_sync(0xFFFFFFFFu, rm[u]);
+        const unsigned w = __reduce_max_sync(0xFFFFFFFFu, rm[u]);
         const int64_t r = r0 + u * rpp;
-        if (threadIdx.x == 0 && r < R && m != 0u) {
-          atomicMax(row_bits + r, m);
-          row_bad |= m >= 0x7F800000u;
+        if (threadIdx.x == 0 && r < v.R && w != 0u) {
+          atomicMax(row_bits + r, w);
+          row_bad |= w >= 0x7F800000u;
         }
       }
     }
@@ -216,30 +257,25 @@ __global__ void __launch_bounds__(kColTx* kColTy)
   if (ROWS && row_bad) atomicOr(status, kDevNonFinite);
   // x has been read: the next kernel (the grouping) may start launching
   griddep_launch_dependents();
-  red[ro * tc + 4 * qc + 0] = m0;
-  red[ro * tc + 4 * qc + 1] = m1;
-  red[ro * tc + 4 * qc + 2] = m2;
-  red[ro * tc + 4 * qc + 3] = m3;
+  put_maxima<FORM>(red, lg, ro, qc, m);
   __syncthreads();
   // thread t < tc: column t of the tile
-  unsigned m = 0;
-  if (tid < tc)
-    for (int y = 0; y < rpp; ++y) m = max(m, red[y * tc + tid]);
+  unsigned w = tid < tc ? get_maximum(red, lg, tid) : 0u;
   if (CL > 1) {
     cluster_wait_acquire();
-    if (tid < tc && m != 0) red_max_cluster_u32(mapa_shared(smem_u32(cmax), 0) + tid * 4, m);
+    if (tid < tc && w != 0) red_max_cluster_u32(mapa_shared(smem_u32(cmax), 0) + tid * 4, w);
     cluster_arrive_release();
     cluster_wait_acquire();   // every block's maxima are in the first block's cmax
     if (cluster_ctarank() != 0) return;
-    if (tid < tc) m = cmax[tid];
+    if (tid < tc) w = cmax[tid];
   }
   if (tid >= tc) return;
   // the accumulators are zeroed by the preceding kernel, which must have completed
   griddep_wait();
-  const int64_t c = static_cast<int64_t>(blockIdx.x) * tc + tid;
-  if (c < C && m != 0) {
-    atomicMax(range_bits + c, m);
-    if (m >= 0x7F800000u) atomicOr(status, kDevNonFinite);
+  const int64_t c = cb + tid;
+  if (c < v.C && w != 0) {
+    atomicMax(column_bits<FORM>(range_bits, v, c), w);
+    if (w >= 0x7F800000u) atomicOr(status, kDevNonFinite);
   }
 }
 
@@ -254,87 +290,54 @@ __global__ void __launch_bounds__(kColTx* kColTy)
 // slower).
 constexpr int kWeightRun = 4;
 
-__global__ void __launch_bounds__(kColTx* kColTy)
-    weight_range_kernel(const float* __restrict__ x, int64_t R, int64_t C, int64_t ld, int vec,
-                        unsigned* __restrict__ col_bits, unsigned* __restrict__ row_bits,
-                        int* __restrict__ status) {
-  __shared__ unsigned red[kColTy * kColTx * 4];
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kColTx + tx;
-  const int64_t cblocks = (C + 4 * kColTx - 1) / (4 * kColTx);
-  const int64_t tiles = (R + 8 * kColTy - 1) / (8 * kColTy);
-  const int64_t j0 = static_cast<int64_t>(blockIdx.x) * kWeightRun;
-  bool bad = false;
-  bool waited = false;
+// one row tile's run of column blocks j0 .. j0 + run - 1; *bad: a non-finite value was met
+template <int FORM>
+__device__ __forceinline__ void weight_range_run(const RangeView& v, int64_t tile, int64_t j0, int run, unsigned* red,
+                                                 unsigned* __restrict__ col_bits,
+                                                 unsigned* __restrict__ row_bits, bool* bad) {
+  const int tid = threadIdx.x + threadIdx.y * blockDim.x, tx = tid & 31, ty = tid >> 5;
+  const int64_t cblocks = (v.C + 4 * kColTx - 1) / (4 * kColTx);
+  const int64_t r0 = tile * 8 * kColTy + ty;   // this thread's rows: r0 + u kColTy
+  unsigned rm[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
 #pragma unroll 1
-  for (int64_t t = blockIdx.y; t < tiles; t += gridDim.y) {
-    const int64_t r0 = t * 8 * kColTy + ty;   // this thread's rows: r0 + u kColTy
-    unsigned rm[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) rm[u] = 0u;
-#pragma unroll 1
-    for (int64_t j = j0; j < j0 + kWeightRun && j < cblocks; ++j) {
-      const int64_t c0 = j * 4 * kColTx + 4 * tx;
-      unsigned m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-      if (vec && c0 + 3 < C) {
-        // rows past the end re-read the last row, which leaves a maximum unchanged
-        float4 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = ld_stream_v4(x + min(r0 + u * kColTy, R - 1) * ld + c0);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const unsigned a0 = abs_bits(v[u].x), a1 = abs_bits(v[u].y);
-          const unsigned a2 = abs_bits(v[u].z), a3 = abs_bits(v[u].w);
-          m0 = max(m0, a0);
-          m1 = max(m1, a1);
-          m2 = max(m2, a2);
-          m3 = max(m3, a3);
-          rm[u] = max(rm[u], max(max(a0, a1), max(a2, a3)));
-        }
-      } else {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int64_t r = min(r0 + u * kColTy, R - 1);
-          unsigned a[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (c0 + k < C) a[k] = abs_bits(__ldg(x + r * ld + c0 + k));
-          m0 = max(m0, a[0]);
-          m1 = max(m1, a[1]);
-          m2 = max(m2, a[2]);
-          m3 = max(m3, a[3]);
-          rm[u] = max(rm[u], max(max(a[0], a[1]), max(a[2], a[3])));
-        }
+  for (int64_t j = j0; j < j0 + run && j < cblocks; ++j) {
+    unsigned m[4] = {0u, 0u, 0u, 0u};
+    const int64_t cb = j * 4 * kColTx;
+    tile_maxima<true, FORM>(v, 5, cb, r0, tx, m, rm);
+    put_maxima<FORM>(red, 5, ty, tx, m);
+    __syncthreads();
+    griddep_wait();   // the accumulators are zeroed by the preceding kernel
+    if (tid < 4 * kColTx) {
+      const unsigned w = get_maximum(red, 5, tid);
+      const int64_t c = cb + tid;
+      if (c < v.C && w != 0u) {
+        atomicMax(col_bits + c, w);
+        *bad |= w >= 0x7F800000u;
       }
-      red[ty * 4 * kColTx + 4 * tx + 0] = m0;
-      red[ty * 4 * kColTx + 4 * tx + 1] = m1;
-      red[ty * 4 * kColTx + 4 * tx + 2] = m2;
-      red[ty * 4 * kColTx + 4 * tx + 3] = m3;
-      __syncthreads();
-      if (!waited) {   // the accumulators are zeroed by the preceding kernel
-        griddep_wait();
-        waited = true;
-      }
-      if (tid < 4 * kColTx) {
-        unsigned m = 0;
-        for (int y = 0; y < kColTy; ++y) m = max(m, red[y * 4 * kColTx + tid]);
-        const int64_t c = j * 4 * kColTx + tid;
-        if (c < C && m != 0u) {
-          atomicMax(col_bits + c, m);
-          bad |= m >= 0x7F800000u;
-        }
-      }
-      __syncthreads();   // red is rewritten by the next column block
     }
+    __syncthreads();  // red is rewritten by the next column block
+  }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const unsigned m = __reduce_max_sync(0xFFFFFFFFu, rm[u]);
-      const int64_t r = r0 + u * kColTy;
-      if (tx == 0 && r < R && m != 0u) {
-        atomicMax(row_bits + r, m);
-        bad |= m >= 0x7F800000u;
-      }
+  for (int u = 0; u < 8; ++u) {
+    const unsigned w = __reduce_max_sync(0xFFFFFFFFu, rm[u]);
+    const int64_t r = r0 + u * kColTy;
+    if (tx == 0 && r < v.R && w != 0u) {
+      atomicMax(row_bits + r, w);
+      *bad |= w >= 0x7F800000u;
     }
   }
+}
+
+template <int FORM>
+__global__ void __launch_bounds__(kColTx* kColTy, 4)
+    weight_range_kernel(const RangeView v, unsigned* __restrict__ col_bits, unsigned* __restrict__ row_bits,
+                        int* __restrict__ status) {
+  __shared__ unsigned red[kColTy * kColTx * 4];
+  const int64_t tiles = (v.R + 8 * kColTy - 1) / (8 * kColTy);
+  bool bad = false;
+#pragma unroll 1
+  for (int64_t t = blockIdx.y; t < tiles; t += gridDim.y)
+    weight_range_run<FORM>(v, t, static_cast<int64_t>(blockIdx.x) * kWeightRun, kWeightRun, red, col_bits, row_bits, &bad);
   // x has been read: the next kernel may start launching
   griddep_launch_dependents();
   if (bad) atomicOr(status, kDevNonFinite);
@@ -368,27 +371,85 @@ __global__ void __launch_bounds__(256)
 }
 
 // ======================================================================= quantize
+// tau_0 of a tensor whose range pass ran in a layer's launch: the blocks send their maxima to
+// kTauSlots words in turn (one word would take thousands of same-address atomics), and a
+// reader takes the largest
+constexpr int kTauSlots = 16;
+
+__device__ __forceinline__ float slots_tau(const unsigned* slots) {   // by a whole warp
+  const int lane = threadIdx.x & 31;
+  return __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, lane < kTauSlots ? __ldcg(slots + lane) : 0u));
+}
+
 struct QuantArgs {
   const float* x;
   int64_t R, C, ld;
-  int gran, Q, G, mode;
+  int Q, G;
   uint64_t seed;
   int64_t row0;           // the tensor's first row within the logical tensor (SR index)
   const float* rt;        // &tau_0 (SHIFT) or range[] (PER_COL / PER_ROW)
-  const uint8_t* exp;     // SHIFT: e_c
-  const uint8_t* fold;    // optional: exponents of the other GEMM operand
+  const unsigned* tslots; // SHIFT: tau_0 as the maximum of kTauSlots bit patterns (or null: *rt) ...
+  float* tau_out;         // ... and stored here
+  const uint8_t* exp;     // SHIFT: e_c, or null: formed from crange and tau_0
+  const float* crange;    // ... the channel ranges
+  uint8_t* exp_out;       // ... and written here by the first tile row
+  const uint8_t* fold;    // exponents of the other GEMM operand, or null: formed from
+  const float* frange;    // ... its channel ranges
+  const unsigned* ftslots;   // ... and tau_0 (kTauSlots bit patterns)
   void* codes;
   int64_t ldc;
   void* codes_t;
   int64_t ldt;
   float* scale_out;
-  int vec_in, vec_out, vec_t;
+  int vec_in;              // 16-byte aligned input rows
+  int vec_out, vec_t;      // output rows that take four codes, or 16 transposed bytes, in one store
+  int lg;                 // tiles of 4 << lg columns by 64 << (5 - lg) rows
+  int form, fast;         // Form, and whether the tensor has what its register path needs
+  // The launch runs beside the quantizer launch before it (a layer's tensors): that one let it
+  // launch only after its own wait, so what both read is complete; the wait comes last, and
+  // whoever waits for this launch has then waited for that one too.
+  int beside;
   // group order of the GEMM inner index (or null): codes column c goes to pos_cols[c]
   // (ShiftQuant and per-row grans), codes_t column r to pos_rows[r] (per-column gran)
   const int* pos_cols;
   const int* pos_rows;
 };
 
+// Quantize tile: 8192 elements by 256 threads, tc = 4 << lg columns (128, 64 or 32) by
+// 64 << (5 - lg) rows.  The rows form chunks of 8; a thread owns four consecutive columns of
+// one chunk (a warp: 32 >> lg chunks).  Two ways through a tile:
+//   registers: a tile inside the tensor whose rows are aligned (or shifted into place, or
+//     whose codes go to a group order: Form), the thread's eight loads in flight together,
+//     its rows unrolled.  Straight-line code that every thread runs once is bound by
+//     instruction fetch as soon as tests are spread through it (with the edges handled in the
+//     unrolled body: 8.4 cycles of no-instruction stall per issue, [12544, 256] 12.4 us against
+//     8.7), so this path holds nothing but the common case;
+//   shared memory: everything else.  Each warp copies its rows asynchronously -- 16 bytes a
+//     copy where they are aligned, else one float a copy, the lanes on consecutive columns,
+//     zeros outside the tensor -- and walks them in a rolled loop.
+// Narrower tiles than 128 columns serve tensors whose column count would leave a 128-column
+// grid partly idle (tile_lg).
+constexpr int kQuantThreads = 256;
+constexpr int kTileElems = 8192;
+constexpr int kWarpBytes = kTileElems / 8 * 4;   // a warp's part of the tile in shared memory
+
+static int64_t tile_cols(int lg) { return int64_t(4) << lg; }
+static int64_t tile_rows(int lg) { return int64_t(64) << (5 - lg); }
+
+// The widest tile (128, 64 or 32 columns) whose padded column count is within 1/8 of the
+// best: the quantizer reads 512, 256 or 128 contiguous bytes a row, so wide tiles win unless
+// they idle (147 columns: 256, 192, 160 padded).
+static int tile_lg(int64_t C) {
+  int64_t pad[3], best = INT64_MAX;
+  for (int k = 0; k < 3; ++k) {
+    const int64_t tc = tile_cols(5 - k);
+    pad[k] = (C + tc - 1) / tc * tc;
+    if (pad[k] < best) best = pad[k];
+  }
+  for (int k = 0; k < 2; ++k)
+    if (pad[k] <= best + best / 8) return 5 - k;
+  return 3;
+}
 
 template <typename CodeT>
 __device__ __forceinline__ CodeT encode_code(float v);
@@ -405,321 +466,606 @@ __device__ __forceinline__ uint8_t encode_code<uint8_t>(float v) {
   return static_cast<uint8_t>(__nv_cvt_float_to_fp8(v, __NV_SATFINITE, __NV_E4M3));
 }
 
-// quantize tile: 64 rows x 128 columns, 256 threads.  Lane l owns columns 4l .. 4l+3 of
-// the tile and warp w the eight rows 8w .. 8w+7: every load instruction of a warp reads 512
-// contiguous bytes of one row, and all eight loads of a thread are in flight together.
-// For the transposed copy each thread packs, per column, its eight codes (rows 8w..8w+7)
-// into one chunk; chunk w of tile column c sits at slot c*8 + (w ^ ((c >> 2) & 7)) of the
-// shared staging area, so the chunk stores of a warp and the row reads that follow both
-// touch every bank equally.
-constexpr int kQR = 64;
-constexpr int kQC = 128;
-constexpr int kQRowsPerWarp = kQR / 8;
-
-__device__ __forceinline__ int chunk_slot(int col, int chunk) {
-  return col * 8 + (chunk ^ ((col >> 2) & 7));
-}
-
-// The thread's eight input rows of the block's 64 x 128 tile (four columns each), all
-// loads in flight together; outside the tensor the values are 0.  FULL: the tile lies
-// inside the tensor and its rows are 16-byte aligned.
-template <bool FULL>
-__device__ __forceinline__ void load_quant_tile(const QuantArgs& a, float4 (&xin)[kQRowsPerWarp]) {
-  const int tid = threadIdx.x;
-  const int lane = tid & 31;
-  const int wq = tid >> 5;
-  const int64_t r0 = static_cast<int64_t>(blockIdx.y) * kQR;
-  const int64_t cb = static_cast<int64_t>(blockIdx.x) * kQC + lane * 4;
+// n codes as 32-bit words, the first code in the low bits
+template <typename CodeT, int N>
+__device__ __forceinline__ void encode_words(const float (&q)[N], uint32_t (&w)[N * sizeof(CodeT) / 4]) {
+  if constexpr (sizeof(CodeT) == 2) {
 #pragma unroll
-  for (int i = 0; i < kQRowsPerWarp; ++i) {
-    const int64_t r = r0 + wq * 8 + i;
-    const float* row = a.x + r * a.ld;
-    if (FULL) {
-      xin[i] = ld_stream_v4(row + cb);
-    } else {
-      xin[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (r < a.R) {
-        if (a.vec_in && cb + 3 < a.C) {
-          xin[i] = __ldg(reinterpret_cast<const float4*>(row + cb));
-        } else {
-          if (cb + 0 < a.C) xin[i].x = __ldg(row + cb + 0);
-          if (cb + 1 < a.C) xin[i].y = __ldg(row + cb + 1);
-          if (cb + 2 < a.C) xin[i].z = __ldg(row + cb + 2);
-          if (cb + 3 < a.C) xin[i].w = __ldg(row + cb + 3);
-        }
-      }
+    for (int k = 0; k < N / 2; ++k)
+      w[k] = __byte_perm(__float_as_uint(q[2 * k]), __float_as_uint(q[2 * k + 1]), 0x7632);
+  } else {
+#pragma unroll
+    for (int k = 0; k < N / 4; ++k) {
+      const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(q[4 * k], q[4 * k + 1]), __NV_SATFINITE, __NV_E4M3);
+      const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(q[4 * k + 2], q[4 * k + 3]), __NV_SATFINITE, __NV_E4M3);
+      w[k] = lo | (hi << 16);
     }
   }
 }
 
-// One 64 x 128 tile.  GRAN: SQ_GRAN_*; MODE: SQ_ROUND_*; FOLD: weight codes carry the
-// ShiftMM shift 2^(G-1-fold[i]); FULL: the tile lies inside the tensor and every access
-// is vector-aligned, so no element needs a bounds check.  LOAD: the tile's loads are
-// issued here; otherwise `pre` holds the thread's eight rows, loaded by the caller
-// (load_quant_tile) -- the weight kernel quantizes one load for both roles.
-template <typename CodeT, int GRAN, int MODE, bool FOLD, bool FULL, bool LOAD = true>
-__device__ __forceinline__ void quantize_tile(const QuantArgs& a, uint8_t* tile_t,
-                                              const float4* pre = nullptr) {
-  constexpr int kChunkBytes = 8 * sizeof(CodeT);  // eight codes of one column
-  constexpr int kWords = kChunkBytes / 4;         // 32-bit words per packed column chunk
-  constexpr int kPerWord = 4 / sizeof(CodeT);
-  const int tid = threadIdx.x;
-  const int lane = tid & 31;
-  const int wq = tid >> 5;
-  const int64_t r0 = static_cast<int64_t>(blockIdx.y) * kQR;
-  const int64_t c0 = static_cast<int64_t>(blockIdx.x) * kQC;
-  const int64_t cb = c0 + lane * 4;
-  const float Qf = static_cast<float>(a.Q);
+// Round to nearest even; + 0 turns a negative zero into a zero code.  |x| <= range gives
+// |v| <= Q (1 + 2^-23), so rint never leaves [-Q, Q].
+__device__ __forceinline__ float round_nearest(float v) { return __fadd_rn(rintf(v), 0.0f); }
 
-  // all eight input rows of this thread first, so their loads overlap
-  float4 xin[kQRowsPerWarp];
-#pragma unroll
-  for (int i = 0; i < kQRowsPerWarp; ++i) {
-    if (!LOAD) {
-      xin[i] = pre[i];
-      continue;
-    }
-    const int64_t r = r0 + wq * 8 + i;
-    const float* row = a.x + r * a.ld;
-    if (FULL) {
-      xin[i] = ld_stream_v4(row + cb);
-    } else {
-      xin[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (r < a.R) {
-        if (a.vec_in && cb + 3 < a.C) {
-          xin[i] = __ldg(reinterpret_cast<const float4*>(row + cb));
-        } else {
-          if (cb + 0 < a.C) xin[i].x = __ldg(row + cb + 0);
-          if (cb + 1 < a.C) xin[i].y = __ldg(row + cb + 1);
-          if (cb + 2 < a.C) xin[i].z = __ldg(row + cb + 2);
-          if (cb + 3 < a.C) xin[i].w = __ldg(row + cb + 3);
-        }
-      }
-    }
-  }
+// Stochastic rounding on the draw of generator state z, clamped to [-Q, Q].  The sum
+// v + 1.5 2^23 rounded down has spacing 1, so l is floor(v) exactly for |v| < 2^22 (and +0
+// for a zero); beyond, l stays on v's side of [-Q, Q] and the clamp decides.
+__device__ __forceinline__ float round_stochastic(float v, uint64_t z, float Qf) {
+  const float l = __fadd_rn(__fadd_rd(v, 12582912.0f), -12582912.0f);
+  const float frac = __fsub_rn(v, l);
+  const float u = __fmul_rn(static_cast<float>(splitmix64_top24(z)), 5.9604644775390625e-08f);  // * 2^-24, exact
+  const float q = u < frac ? __fadd_rn(l, 1.0f) : l;
+  return fminf(fmaxf(q, -Qf), Qf);
+}
 
-  // per-column multipliers: 2^e_c (SHIFT) or Q / range_c (PER_COL); per-column shifts
-  float colmul[4];
-  bool colzero[4];
-  int colfold[4];
-  float invS = 0.0f;
-  bool zero_all = false;
+// the exponent of channel c: given, or formed from its range and tau_0
+__device__ __forceinline__ int channel_exponent(float r, float tau, int G) {
+  return isfinite(tau) ? group_exponent(r, tau, G) : 0;
+}
+
+// Q / range of a per-channel scale; 0 and *zero for a channel that quantizes to zero
+__device__ __forceinline__ float channel_inv(float rg, float Qf, bool* zero) {
+  const float inv = __fdiv_rn(Qf, rg);
+  *zero = !(rg > 0.0f) || !isfinite(rg) || !isfinite(inv);
+  return *zero ? 0.0f : inv;
+}
+
+// the folded shift of inner channel i of the other operand, as a factor
+__device__ __forceinline__ float fold_factor(const QuantArgs& a, float ftau, int64_t i) {
+  const int e = a.fold != nullptr ? static_cast<int>(__ldg(a.fold + i))
+                                  : channel_exponent(__ldcg(a.frange + i), ftau, a.G);
+  return pow2f(a.G - 1 - e);
+}
+
+// ShiftQuant's per-tensor values
+struct TensorScale {
+  float tau, invS;
+  bool zero;    // tau_0 is 0 or not finite, or Q / tau_0 overflows: every code is 0
+  bool merged;  // 2^e Q / tau_0 is finite for every e: one multiplication per element
+};
+
+__device__ __forceinline__ TensorScale tensor_scale(const QuantArgs& a, float Qf) {
+  TensorScale t;
+  t.tau = a.tslots != nullptr ? slots_tau(a.tslots) : __ldcg(a.rt);
+  t.invS = __fdiv_rn(Qf, t.tau);
+  t.zero = !(t.tau > 0.0f) || !isfinite(t.tau) || !isfinite(t.invS);
+  t.merged = isfinite(__fmul_rn(t.invS, pow2f(a.G - 1)));
+  return t;
+}
+
+// What a thread needs of column c: the multiplier (SHIFT: 2^e Q / tau_0, where
+// fl(fl(x 2^e) fl(Q / tau_0)) = fl(x (2^e fl(Q / tau_0))) as scaling by 2^e is exact -- or, not
+// merged, Q / tau_0 alone with the 2^e in `scale`; PER_COL: Q / range), whether the column's
+// codes are all 0, and the folded shift (PER_ROW).
+struct ColumnValues {
+  float mul, scale, fold;
+  bool zero;
+};
+
+template <int GRAN, bool FOLD>
+__device__ __forceinline__ ColumnValues column_values(const QuantArgs& a, const TensorScale& ts,
+                                                      float ftau, int64_t c, float Qf, bool write) {
+  ColumnValues v = {1.0f, 1.0f, 1.0f, false};
   if (GRAN == SQ_GRAN_SHIFT) {
-    const float tau = __ldg(a.rt);
-    invS = __fdiv_rn(Qf, tau);
-    zero_all = !(tau > 0.0f) || !isfinite(tau) || !isfinite(invS);
+    const int e = a.exp != nullptr ? static_cast<int>(__ldg(a.exp + c))
+                                   : channel_exponent(__ldcg(a.crange + c), ts.tau, a.G);
+    if (write && a.exp_out != nullptr) a.exp_out[c] = static_cast<uint8_t>(e);
+    v.scale = pow2f(e);
+    v.mul = ts.zero ? 0.0f : (ts.merged ? __fmul_rn(ts.invS, v.scale) : ts.invS);
+    v.zero = ts.zero;
+  } else if (GRAN == SQ_GRAN_PER_COL) {
+    const float rg = __ldcg(a.rt + c);
+    v.mul = channel_inv(rg, Qf, &v.zero);
+    if (write) a.scale_out[c] = v.zero ? 0.0f : __fdiv_rn(rg, Qf);
+  } else if (FOLD) {
+    v.fold = fold_factor(a, ftau, c);
   }
+  return v;
+}
+
+// The per-row values of a chunk's eight rows, held one row per lane of each group of eight
+// lanes and handed round by shuffles: the multiplier (PER_ROW: Q / range) and the folded
+// shift (PER_COL).
+struct RowValues {
+  float mul, fold;
+  unsigned zero;  // bit i: row i of the lane's group quantizes to zero
+};
+
+template <int GRAN, bool FOLD>
+__device__ __forceinline__ RowValues row_values(const QuantArgs& a, float ftau, int64_t r0, float Qf, bool write) {
+  RowValues v = {1.0f, 1.0f, 0u};
+  const int lane = threadIdx.x & 31;
+  const int64_t r = r0 + (lane & 7);
+  if (GRAN == SQ_GRAN_PER_ROW) {
+    bool z = true;
+    if (r < a.R) {
+      const float rg = __ldcg(a.rt + r);
+      v.mul = channel_inv(rg, Qf, &z);
+      if (write) a.scale_out[r] = z ? 0.0f : __fdiv_rn(rg, Qf);
+    }
+    v.zero = (__ballot_sync(0xFFFFFFFFu, z) >> (lane & 24)) & 0xFFu;
+  }
+  if (GRAN == SQ_GRAN_PER_COL && FOLD && r < a.R) v.fold = fold_factor(a, ftau, r);
+  return v;
+}
+
+// The thread's place in the tile at (bx, by).
+struct TilePos {
+  int chunk, col;   // its chunk, and its first column in the tile
+  int64_t r, c;     // its first row and column in the tensor
+};
+
+__device__ __forceinline__ TilePos tile_pos(int lg, unsigned bx, unsigned by) {
+  const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+  TilePos p;
+  p.chunk = (wq << (5 - lg)) + (lane >> lg);
+  p.col = 4 * (lane & ((1 << lg) - 1));
+  p.r = (static_cast<int64_t>(by) << (11 - lg)) + p.chunk * 8;
+  p.c = (static_cast<int64_t>(bx) << (lg + 2)) + p.col;
+  return p;
+}
+
+// This warp's rows of x into its part of the tile: the thread's quad of row i of its chunk
+// ends up at its slot i (quad_slot).
+__device__ __forceinline__ uint32_t quad_slot(uint32_t warp_smem, int lg, int i) {
+  const int lane = threadIdx.x & 31;
+  // row (lane >> lg) 8 + i of the warp's rows, quad (lane mod 2^lg) of the row
+  return warp_smem + ((((lane >> lg) * 8 + i) << lg) + (lane & ((1 << lg) - 1))) * 16;
+}
+
+__device__ __forceinline__ void load_tile(const QuantArgs& a, unsigned bx, unsigned by, uint32_t warp_smem) {
+  const int lg = a.lg;
+  const TilePos p = tile_pos(lg, bx, by);
+  if (a.vec_in && (static_cast<int64_t>(bx) + 1) << (lg + 2) <= a.C) {
+    const float* src = a.x + p.r * a.ld + p.c;
+    const uint32_t dst = quad_slot(warp_smem, lg, 0), step = 16u << lg;
+    if (p.r + 8 <= a.R) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) cp_async_16(dst + i * step, src + i * a.ld, true);
+    } else {
+#pragma unroll 1
+      for (int i = 0; i < 8; ++i) {
+        const bool in = p.r + i < a.R;
+        cp_async_16(dst + i * step, in ? src + i * a.ld : a.x, in);
+      }
+    }
+  } else {
+    // copy k of a lane: row k / (tc / 32) of the warp's rows, column lane + 32 (k mod (tc / 32))
+    const int lane = threadIdx.x & 31, lp = lg - 3;
+    const int64_t r0 = (static_cast<int64_t>(by) << (11 - lg)) + (((threadIdx.x >> 5) << (5 - lg)) << 3);
+    const int64_t c0 = (static_cast<int64_t>(bx) << (lg + 2)) + lane;
+#pragma unroll 4
+    for (int k = 0; k < 32; ++k) {
+      const int row = k >> lp, col = 32 * (k & ((1 << lp) - 1));
+      const bool in = r0 + row < a.R && c0 + col < a.C;
+      cp_async_4(warp_smem + ((row << (lg + 2)) + col + lane) * 4,
+                 in ? a.x + (r0 + row) * a.ld + c0 + col : a.x, in);
+    }
+  }
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncwarp();
+}
+
+// The place (16-byte units of BF16, 8-byte units of E4M3 chunks) of a tile column's chunk in
+// the shared staging area: in the part of the warp that owns the chunk, the low three bits of
+// the column mixed with the chunk index so that the chunk stores of a warp and the column
+// reads that follow both spread over the banks.
+template <typename CodeT>
+__device__ __forceinline__ uint32_t chunk_addr(uint32_t tile_smem, int lg, int col, int chunk) {
+  const int sub = chunk & ((1 << (5 - lg)) - 1), w = chunk >> (5 - lg);
+  const int pos = (col & ~7) | ((col ^ (col >> 2) ^ chunk) & 7);
+  return tile_smem + w * kWarpBytes + (((sub << (lg + 2)) + pos) * 8) * static_cast<int>(sizeof(CodeT));
+}
+
+// The transposed copy from the staged chunks: every thread stores 16 bytes (one BF16 chunk or
+// two E4M3 chunks) of a tile column at a time.
+template <typename CodeT>
+__device__ __forceinline__ void store_transposed(const QuantArgs& a, uint32_t tile_smem, unsigned bx,
+                                                 unsigned by) {
+  constexpr int E = 16 / sizeof(CodeT);   // codes per store
+  const int lg = a.lg;
+  const int64_t c0 = static_cast<int64_t>(bx) << (lg + 2), r0 = static_cast<int64_t>(by) << (11 - lg);
+  __syncthreads();
+  if (lg == 5 && a.vec_t && a.pos_rows == nullptr && r0 + 64 <= a.R && c0 + 128 <= a.C) {
+    // a whole 64 x 128 tile: a thread's stores are 32 (BF16) or 64 (E4M3) columns apart, its
+    // places in the staging area a constant apart
+    constexpr int kSpc = sizeof(CodeT) == 2 ? 3 : 2;       // log2(stores per column)
+    constexpr int kCols = kQuantThreads >> kSpc;           // columns between a thread's stores
+    const int lc = threadIdx.x >> kSpc, st = threadIdx.x & ((1 << kSpc) - 1);
+    CodeT* dst = static_cast<CodeT*>(a.codes_t) + (c0 + lc) * a.ldt + r0 + st * E;
+    uint32_t from[2];   // of its chunk, or its two chunks
+#pragma unroll
+    for (int h = 0; h < 16 / (8 * static_cast<int>(sizeof(CodeT))); ++h)
+      from[h] = chunk_addr<CodeT>(tile_smem, 5, lc, sizeof(CodeT) == 2 ? st : 2 * st + h);
+#pragma unroll
+    for (int k = 0; k < 128 / kCols; ++k) {
+      uint4 v;
+      if constexpr (sizeof(CodeT) == 2) {
+        v = ld_shared_v4_u32(from[0] + k * kCols * 16);
+      } else {
+        const uint2 lo = ld_shared_v2_u32(from[0] + k * kCols * 8), hi = ld_shared_v2_u32(from[1] + k * kCols * 8);
+        v = make_uint4(lo.x, lo.y, hi.x, hi.y);
+      }
+      *reinterpret_cast<uint4*>(dst) = v;
+      dst += kCols * a.ldt;
+    }
+    return;
+  }
+  if (a.pos_rows != nullptr) {
+    // group-ordered: element (column c, row r) goes to pos_rows[r]; a thread keeps its row
+    const int lr = 11 - lg;                // log2(rows)
+    const int rr = threadIdx.x & ((1 << lr) - 1), step = kQuantThreads >> lr;
+    const int64_t r = r0 + rr;
+    if (r >= a.R) return;
+    int lc = threadIdx.x >> lr;
+    const int ncol = static_cast<int>(min(a.C - c0, int64_t(4) << lg));
+    CodeT* d = static_cast<CodeT*>(a.codes_t) + (c0 + lc) * a.ldt + __ldg(a.pos_rows + r);
+#pragma unroll 4
+    for (; lc < ncol; lc += step) {
+      *d = ld_shared_code<CodeT>(chunk_addr<CodeT>(tile_smem, lg, lc, rr >> 3) + (rr & 7) * static_cast<int>(sizeof(CodeT)));
+      d += step * a.ldt;
+    }
+    return;
+  }
+  uint8_t* ct = static_cast<uint8_t*>(a.codes_t);
+  const int spc = 8 - lg - (sizeof(CodeT) == 1 ? 1 : 0);   // log2(stores per column)
+#pragma unroll 2
+  for (int k = 0; k < kTileElems / E / kQuantThreads; ++k) {
+    const int idx = threadIdx.x + k * kQuantThreads;
+    const int lc = idx >> spc, st = idx & ((1 << spc) - 1);
+    const int64_t c = c0 + lc, rs = r0 + st * E;
+    if (c >= a.C || rs >= a.R) continue;
+    uint4 v;
+    if constexpr (sizeof(CodeT) == 2) {
+      v = ld_shared_v4_u32(chunk_addr<CodeT>(tile_smem, lg, lc, st));
+    } else {
+      const uint2 lo = ld_shared_v2_u32(chunk_addr<CodeT>(tile_smem, lg, lc, 2 * st));
+      const uint2 hi = ld_shared_v2_u32(chunk_addr<CodeT>(tile_smem, lg, lc, 2 * st + 1));
+      v = make_uint4(lo.x, lo.y, hi.x, hi.y);
+    }
+    CodeT* dst = reinterpret_cast<CodeT*>(ct) + c * a.ldt + rs;
+    if (a.vec_t && rs + E <= a.R) {
+      *reinterpret_cast<uint4*>(dst) = v;
+    } else {
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (rs + e < a.R)
+          dst[e] = static_cast<CodeT>(w[e * sizeof(CodeT) / 4] >> (8 * ((e * sizeof(CodeT)) & 3)));
+    }
+  }
+}
+
+// The values a thread keeps over its rows.
+struct QuadState {
+  float mul[4], pre[4], cfold[4];   // per column (ColumnValues)
+  unsigned czero;                   // bit j: column j's codes are all 0
+  bool merged;                      // TensorScale
+  bool rare;   // inputs quantize to zero for another reason than their value, or need a second scale
+  RowValues rv;
+  uint64_t state;                   // generator state of element (row, column 0 of the quad)
+  TilePos p;
+};
+
+template <int GRAN, int MODE, bool FOLD>
+__device__ __forceinline__ QuadState quad_state(const QuantArgs& a, unsigned bx, unsigned by) {
+  const float Qf = static_cast<float>(a.Q);
+  QuadState t;
+  t.p = tile_pos(a.lg, bx, by);
+  TensorScale ts = {};
+  if (GRAN == SQ_GRAN_SHIFT) ts = tensor_scale(a, Qf);
+  const float ftau = FOLD && a.fold == nullptr ? slots_tau(a.ftslots) : 0.0f;
+  t.merged = ts.merged;
+  t.czero = 0u;
+  const bool first = by == 0 && t.p.chunk == 0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const int64_t c = cb + j;
-    colmul[j] = 1.0f;
-    colzero[j] = false;
-    colfold[j] = 0;
-    if (FULL || c < a.C) {
-      if (GRAN == SQ_GRAN_SHIFT) {
-        colmul[j] = pow2f(__ldg(a.exp + c));
-      } else if (GRAN == SQ_GRAN_PER_COL) {
-        const float rg = __ldg(a.rt + c);
-        colmul[j] = __fdiv_rn(Qf, rg);
-        colzero[j] = !(rg > 0.0f) || !isfinite(rg) || !isfinite(colmul[j]);
-      }
-      if (GRAN == SQ_GRAN_PER_ROW && FOLD) colfold[j] = a.G - 1 - __ldg(a.fold + c);
+    ColumnValues v = {1.0f, 1.0f, 1.0f, false};
+    if (t.p.c + j < a.C) v = column_values<GRAN, FOLD>(a, ts, ftau, t.p.c + j, Qf, first);
+    t.mul[j] = v.mul;
+    t.pre[j] = v.scale;
+    t.cfold[j] = v.fold;
+    t.czero |= v.zero ? 1u << j : 0u;
+  }
+  t.rv = row_values<GRAN, FOLD>(a, ftau, t.p.r, Qf, bx == 0 && t.p.col < 32);
+  t.state = 0;   // seed + (idx + 1) gamma
+  if (MODE == SQ_ROUND_STOCHASTIC)
+    t.state = a.seed + (static_cast<uint64_t>(a.row0 + t.p.r) * static_cast<uint64_t>(a.C) +
+                        static_cast<uint64_t>(t.p.c) + 1ull) * kSplitMixGamma;
+  t.rare = t.czero != 0u || (GRAN == SQ_GRAN_SHIFT && !ts.merged) ||
+           (GRAN == SQ_GRAN_PER_ROW && t.rv.zero != 0u);
+  if (GRAN == SQ_GRAN_SHIFT && bx == 0 && by == 0 && threadIdx.x == 0) {
+    *a.scale_out = ts.zero ? 0.0f : __fdiv_rn(ts.tau, Qf);
+    if (a.tau_out != nullptr) *a.tau_out = ts.tau;
+  }
+  return t;
+}
+
+// The four codes of row i of the quad.
+template <typename CodeT, int GRAN, int MODE, bool FOLD>
+__device__ __forceinline__ void quantize_quad(const QuadState& t, const float (&x)[4], int i, uint64_t state,
+                                              float Qf, uint32_t (&words)[sizeof(CodeT)]) {
+  const int src = threadIdx.x & 24;
+  const float rmul = GRAN == SQ_GRAN_PER_ROW ? __shfl_sync(0xFFFFFFFFu, t.rv.mul, src | i) : 1.0f;
+  const float rfold = GRAN == SQ_GRAN_PER_COL && FOLD ? __shfl_sync(0xFFFFFFFFu, t.rv.fold, src | i) : 1.0f;
+  float q[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float v = __fmul_rn(x[j], GRAN == SQ_GRAN_PER_ROW ? rmul : t.mul[j]);
+    q[j] = MODE == SQ_ROUND_NEAREST_EVEN
+               ? round_nearest(v)
+               : round_stochastic(v, state + static_cast<uint64_t>(j) * kSplitMixGamma, Qf);
+    if (FOLD) q[j] = __fmul_rn(q[j], GRAN == SQ_GRAN_PER_ROW ? t.cfold[j] : rfold);
+  }
+  encode_words<CodeT, 4>(q, words);
+}
+
+template <typename CodeT>
+__device__ __forceinline__ CodeT code_of_word(const uint32_t (&words)[sizeof(CodeT)], int j) {
+  return static_cast<CodeT>(words[j * sizeof(CodeT) / 4] >> (8 * ((j * sizeof(CodeT)) & 3)));
+}
+
+// A row's codes into the thread's slot of that row (where the row of x was, or would be).
+template <typename CodeT>
+__device__ __forceinline__ void keep_words(uint32_t slot, const uint32_t (&words)[sizeof(CodeT)]) {
+  if constexpr (sizeof(CodeT) == 2)
+    st_shared_v2(slot, words[0], words[1]);
+  else
+    st_shared_u32(slot, words[0]);
+}
+
+// The chunk of each of the quad's columns -- its code of every row, gathered from the thread's
+// slots -- into the staging area.
+template <typename CodeT>
+__device__ __forceinline__ void stage_chunks(const TilePos& p, int lg, uint32_t tile_smem) {
+  const uint32_t slot0 = quad_slot(tile_smem + (threadIdx.x >> 5) * kWarpBytes, lg, 0), step = 16u << lg;
+  uint32_t words[8][sizeof(CodeT)];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    if constexpr (sizeof(CodeT) == 2) {
+      const uint2 v = ld_shared_v2_u32(slot0 + i * step);
+      words[i][0] = v.x;
+      words[i][1] = v.y;
+    } else {
+      words[i][0] = ld_shared_u32(slot0 + i * step);
     }
   }
+  __syncwarp();   // every lane's slots have been read: the chunks may overwrite them
+  // (the quad's columns differ in the low two bits of the column alone, which chunk_addr
+  // exclusive-ors into the low bits of the place)
+  constexpr uint32_t kChunkBytes = 8 * sizeof(CodeT);
+  const uint32_t at0 = chunk_addr<CodeT>(tile_smem, lg, p.col, p.chunk);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t to = at0 ^ (j * kChunkBytes);
+    if constexpr (sizeof(CodeT) == 2) {
+      uint32_t w[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        w[k] = __byte_perm(words[2 * k][j >> 1], words[2 * k + 1][j >> 1], (j & 1) ? 0x7632 : 0x5410);
+      st_shared_v4(to, w[0], w[1], w[2], w[3]);
+    } else {
+      uint32_t w[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const uint32_t lo = __byte_perm(words[4 * k][0], words[4 * k + 1][0], j | ((4 + j) << 4));
+        const uint32_t hi = __byte_perm(words[4 * k + 2][0], words[4 * k + 3][0], j | ((4 + j) << 4));
+        w[k] = __byte_perm(lo, hi, 0x5410);
+      }
+      st_shared_v2(to, w[0], w[1]);
+    }
+  }
+}
 
-  uint32_t packed[4][kWords];
+// ---------------------------------------------------------------- register path
+// What a launch's register path expects of its tensor; tiles that differ take the other path.
+enum Form {
+  kAligned,   // rows 16-byte aligned in and out
+  kShifted,   // rows of x start anywhere
+  kOrdered    // aligned rows of x, codes in a group order
+};
+
+template <int FORM>
+__device__ __forceinline__ bool register_tile(const QuantArgs& a, unsigned bx, unsigned by) {
+  const int64_t r1 = (static_cast<int64_t>(by) + 1) << (11 - a.lg);
+  const int64_t c1 = (static_cast<int64_t>(bx) + 1) << (a.lg + 2);
+  if (!a.fast) return false;
+  // shifted rows read whole tile rows and up to three elements more: what lies past the last
+  // column comes from the following row, which must be there and long enough
+  if (FORM == kShifted) return r1 < a.R && c1 + 4 <= a.C + a.ld;
+  // aligned tiles may be partial, in whole quads (a group order: whole columns)
+  return c1 <= a.C || (FORM == kAligned && (a.C & 3) == 0);
+}
+
+template <int FORM>
+__device__ __forceinline__ void load_registers(const QuantArgs& a, unsigned bx, unsigned by, float4 (&x)[8]) {
+  const TilePos p = tile_pos(a.lg, bx, by);
+  if (FORM != kShifted) {
+    // quads and rows outside the tensor read its first column and its last row: their codes are
+    // not stored
+    const float* src = a.x + (p.c < a.C ? p.c : 0);
+    if (p.r + 8 <= a.R) {
+      src += p.r * a.ld;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = ld_stream_v4(src + i * a.ld);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = ld_stream_v4(src + min(p.r + i, a.R - 1) * a.ld);
+    }
+    return;
+  }
+  // Of each row the lanes read the aligned vectors that cover the tile, and each takes the
+  // elements past its own vector from its neighbour -- the last lane of a row from the vector
+  // after the tile, which lane i of the row's lanes reads for row i.
+  const int lane = threadIdx.x & 31, lpr = 1 << a.lg;   // lanes per row
+  const int64_t off = p.r * a.ld + p.c;
+  const bool last = (lane & (lpr - 1)) == lpr - 1;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) x[i] = ld_stream_v4(a.x + ((off + i * a.ld) & ~int64_t(3)));
+  const float4 e = ld_stream_v4(a.x + ((off - p.col + lpr * 4 + (lane & 7) * a.ld) & ~int64_t(3)));
+  const int grp = lane & ~(lpr - 1);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int sh = static_cast<int>((off + i * a.ld) & 3);   // the same for all lanes of a row
+    const float4 v = x[i];
+    float4 n;
+    n.x = __shfl_down_sync(0xFFFFFFFFu, v.x, 1);
+    n.y = __shfl_down_sync(0xFFFFFFFFu, v.y, 1);
+    n.z = __shfl_down_sync(0xFFFFFFFFu, v.z, 1);
+    const float ex = __shfl_sync(0xFFFFFFFFu, e.x, grp | i);
+    const float ey = __shfl_sync(0xFFFFFFFFu, e.y, grp | i);
+    const float ez = __shfl_sync(0xFFFFFFFFu, e.z, grp | i);
+    if (last) {
+      n.x = ex;
+      n.y = ey;
+      n.z = ez;
+    }
+    if (sh == 1) x[i] = make_float4(v.y, v.z, v.w, n.x);
+    if (sh == 2) x[i] = make_float4(v.z, v.w, n.x, n.y);
+    if (sh == 3) x[i] = make_float4(v.w, n.x, n.y, n.z);
+  }
+}
+
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD>
+__device__ __forceinline__ void quantize_registers(const QuantArgs& a, const QuadState& t, const float4 (&xin)[8],
+                                                   uint32_t tile_smem) {
+  const float Qf = static_cast<float>(a.Q);
+  const uint64_t row_step = static_cast<uint64_t>(a.C) * kSplitMixGamma;
+  const bool ordered = FORM == kOrdered && a.pos_cols != nullptr;
+  CodeT* dst = static_cast<CodeT*>(a.codes) + t.p.r * a.ldc + t.p.c;
+  // the codes are kept in the thread's slots for the transposed copy and for a group order
+  const bool kept = a.codes_t != nullptr || ordered;
+  const uint32_t warp_smem = tile_smem + (threadIdx.x >> 5) * kWarpBytes;
+  uint64_t state = t.state;
+  const uint32_t keep = quad_slot(warp_smem, a.lg, 0), step = 16u << a.lg;
+  // rows of the quad to store
+  const int rows = a.codes == nullptr || ordered || t.p.c >= a.C ? 0 : static_cast<int>(min(a.R - t.p.r, int64_t(8)));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float x[4] = {xin[i].x, xin[i].y, xin[i].z, xin[i].w};
+    uint32_t words[sizeof(CodeT)];
+    quantize_quad<CodeT, GRAN, MODE, FOLD>(t, x, i, state, Qf, words);
+    state += row_step;
+    if (i < rows) {
+      if (FORM == kShifted && t.p.c + 3 >= a.C) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (t.p.c + j < a.C) dst[j] = code_of_word<CodeT>(words, j);
+      } else if constexpr (sizeof(CodeT) == 2) {
+        *reinterpret_cast<uint2*>(dst) = make_uint2(words[0], words[1]);
+      } else {
+        *reinterpret_cast<uint32_t*>(dst) = words[0];
+      }
+    }
+    dst += a.ldc;
+    if (kept) keep_words<CodeT>(keep + i * step, words);
+  }
+  if (ordered) {
+    // The channels of a group keep their order, so 32 consecutive columns go to a few runs of
+    // consecutive places: one column a lane writes whole runs, where a lane's own four columns
+    // would write two bytes of every eight (four times the partial sectors).
+    const int lane = threadIdx.x & 31, groups = 1 << (a.lg - 3);   // of 32 columns in the tile
+    const int64_t cb = t.p.c - t.p.col + lane, rb = t.p.r - 8 * (lane >> a.lg);   // the warp's first row
+    int at[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+      if (g < groups) at[g] = __ldg(a.pos_cols + cb + 32 * g);
+    const int nrows = static_cast<int>(min(a.R - rb, int64_t(64 >> (a.lg - 2))));
+    // (column 32 g + lane of the warp's row r)
+    uint32_t from = warp_smem + (lane >> 2) * 16 + (lane & 3) * static_cast<int>(sizeof(CodeT));
+    CodeT* d = static_cast<CodeT*>(a.codes) + rb * a.ldc;
+    __syncwarp();
+#pragma unroll 2
+    for (int r = 0; r < nrows; ++r) {
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+        if (g < groups) d[at[g]] = ld_shared_code<CodeT>(from + g * 128);
+      from += step;
+      d += a.ldc;
+    }
+    __syncwarp();   // the chunks may overwrite the slots
+  }
+  if (a.codes_t != nullptr) stage_chunks<CodeT>(t.p, a.lg, tile_smem);
+}
+
+// ------------------------------------------------------------ shared-memory path
+template <typename CodeT, int GRAN, int MODE, bool FOLD>
+__device__ __forceinline__ void quantize_rows(const QuantArgs& a, const QuadState& t, uint32_t tile_smem) {
+  const float Qf = static_cast<float>(a.Q);
+  const uint32_t slot0 = quad_slot(tile_smem + (threadIdx.x >> 5) * kWarpBytes, a.lg, 0), step = 16u << a.lg;
+  const uint64_t row_step = static_cast<uint64_t>(a.C) * kSplitMixGamma;
+  uint64_t state = t.state;
+  const int rows = static_cast<int>(a.R - t.p.r < 8 ? (a.R - t.p.r < 0 ? 0 : a.R - t.p.r) : 8);
+  // four codes in one store; otherwise the place of each column's code in a row (-1: none)
+  const bool wide = a.vec_out && a.pos_cols == nullptr && t.p.c + 3 < a.C;
+  int64_t at[4] = {-1, -1, -1, -1};
 #pragma unroll
   for (int j = 0; j < 4; ++j)
+    if (a.codes != nullptr && !wide && t.p.c + j < a.C)
+      at[j] = a.pos_cols != nullptr ? __ldg(a.pos_cols + t.p.c + j) : t.p.c + j;
+  CodeT* dst = static_cast<CodeT*>(a.codes) + t.p.r * a.ldc + (wide ? t.p.c : 0);
+#pragma unroll 1
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t slot = slot0 + i * step;
+    const float4 x4 = ld_shared_v4_f32(slot);
+    float x[4] = {x4.x, x4.y, x4.z, x4.w};
+    if (t.rare) {
 #pragma unroll
-    for (int k = 0; k < kWords; ++k) packed[j][k] = 0u;
-
-  // stochastic rounding: the generator state of element (r, c) is seed + (idx+1) gamma with
-  // idx = (row0 + r) C + c; it advances by gamma per column and by C gamma per row
-  uint64_t sr_state = 0;
-  if (MODE == SQ_ROUND_STOCHASTIC)
-    sr_state = a.seed + (static_cast<uint64_t>(a.row0 + r0 + wq * 8) * static_cast<uint64_t>(a.C) +
-                         static_cast<uint64_t>(cb) + 1ull) * kSplitMixGamma;
-  const uint64_t sr_row_step = static_cast<uint64_t>(a.C) * kSplitMixGamma;
-
-#pragma unroll
-  for (int i = 0; i < kQRowsPerWarp; ++i) {
-    const int64_t r = r0 + wq * 8 + i;
-    const bool row_in = FULL || r < a.R;
-    float rowmul = 1.0f;
-    bool rowzero = false;
-    int rowfold = 0;
-    if (row_in) {
-      if (GRAN == SQ_GRAN_PER_ROW) {
-        const float rg = __ldg(a.rt + r);
-        rowmul = __fdiv_rn(Qf, rg);
-        rowzero = !(rg > 0.0f) || !isfinite(rg) || !isfinite(rowmul);
+      for (int j = 0; j < 4; ++j) {
+        if (GRAN == SQ_GRAN_SHIFT && !t.merged) x[j] = __fmul_rn(x[j], t.pre[j]);
+        if (((t.czero >> j) & 1u) || (GRAN == SQ_GRAN_PER_ROW && ((t.rv.zero >> i) & 1u))) x[j] = 0.0f;
       }
-      if (GRAN == SQ_GRAN_PER_COL && FOLD) rowfold = a.G - 1 - __ldg(a.fold + r);
     }
-    const float xv[4] = {xin[i].x, xin[i].y, xin[i].z, xin[i].w};
-    CodeT out[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      float v;
-      bool z;
-      if (GRAN == SQ_GRAN_SHIFT) {
-        v = __fmul_rn(__fmul_rn(xv[j], colmul[j]), invS);  // x 2^e exactly, then * Q/tau
-        z = zero_all;
-      } else if (GRAN == SQ_GRAN_PER_COL) {
-        v = __fmul_rn(xv[j], colmul[j]);
-        z = colzero[j];
-      } else {
-        v = __fmul_rn(xv[j], rowmul);
-        z = rowzero;
-      }
-      if (!FULL) z = z || !row_in || cb + j >= a.C;
-      float q;
-      if (MODE == SQ_ROUND_NEAREST_EVEN) {
-        // |x| <= range gives |v| <= Q (1 + 2^-23), so rint never leaves [-Q, Q]
-        q = rintf(v);
-      } else {
-        const float l = floorf(v);
-        const float frac = __fsub_rn(v, l);
-        const uint32_t h24 = splitmix64_top24(sr_state + static_cast<uint64_t>(j) * kSplitMixGamma +
-                                              static_cast<uint64_t>(i) * sr_row_step);
-        const float u = __fmul_rn(static_cast<float>(h24), 5.9604644775390625e-08f);  // * 2^-24, exact
-        q = (u < frac) ? __fadd_rn(l, 1.0f) : l;
-        q = fminf(fmaxf(q, -Qf), Qf);
-      }
-      if (z) q = 0.0f;
-      if (FOLD) {
-        const int f = (GRAN == SQ_GRAN_PER_ROW) ? colfold[j] : rowfold;
-        q = __fmul_rn(q, pow2f(f));
-      }
-      out[j] = encode_code<CodeT>(__fadd_rn(q, 0.0f));  // +0 for a zero code
-      packed[j][i / kPerWord] |= static_cast<uint32_t>(out[j]) << (8 * sizeof(CodeT) * (i % kPerWord));
-    }
-    if (a.codes && row_in && a.pos_cols != nullptr) {
-      CodeT* dst = static_cast<CodeT*>(a.codes) + r * a.ldc;
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (FULL || cb + j < a.C) dst[__ldg(a.pos_cols + cb + j)] = out[j];
-    } else if (a.codes && row_in) {
-      CodeT* dst = static_cast<CodeT*>(a.codes) + r * a.ldc + cb;
-      if (FULL || (a.vec_out && cb + 3 < a.C)) {
-        if constexpr (sizeof(CodeT) == 2) {
-          uint2 w;
-          w.x = static_cast<uint32_t>(out[0]) | (static_cast<uint32_t>(out[1]) << 16);
-          w.y = static_cast<uint32_t>(out[2]) | (static_cast<uint32_t>(out[3]) << 16);
-          *reinterpret_cast<uint2*>(dst) = w;
-        } else {
-          const uint32_t w = static_cast<uint32_t>(out[0]) | (static_cast<uint32_t>(out[1]) << 8) |
-                             (static_cast<uint32_t>(out[2]) << 16) |
-                             (static_cast<uint32_t>(out[3]) << 24);
-          *reinterpret_cast<uint32_t*>(dst) = w;
-        }
+    uint32_t words[sizeof(CodeT)];
+    quantize_quad<CodeT, GRAN, MODE, FOLD>(t, x, i, state, Qf, words);
+    state += row_step;
+    if (a.codes != nullptr && i < rows) {
+      if (wide) {
+        if constexpr (sizeof(CodeT) == 2)
+          *reinterpret_cast<uint2*>(dst) = make_uint2(words[0], words[1]);
+        else
+          *reinterpret_cast<uint32_t*>(dst) = words[0];
       } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (cb + j < a.C) dst[j] = out[j];
+          if (at[j] >= 0) dst[at[j]] = code_of_word<CodeT>(words, j);
       }
+      dst += a.ldc;
     }
+    if (a.codes_t != nullptr) keep_words<CodeT>(slot, words);
   }
-
-  if (a.codes_t) {
-    const uint32_t base = smem_u32(tile_t);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t dst = base + chunk_slot(lane * 4 + j, wq) * kChunkBytes;
-      if constexpr (kWords == 4)
-        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(packed[j][0]),
-                     "r"(packed[j][1]), "r"(packed[j][2]), "r"(packed[j][3]) : "memory");
-      else
-        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst), "r"(packed[j][0]),
-                     "r"(packed[j][1]) : "memory");
-    }
-    __syncthreads();
-    if (a.pos_rows != nullptr) {
-      // group-ordered transposed copy: element (column c, row r) goes to pos_rows[r]
-      CodeT* ctp = static_cast<CodeT*>(a.codes_t);
-      for (int idx = tid; idx < kQC * kQR; idx += 256) {
-        const int lc = idx / kQR, rr = idx % kQR;
-        const int64_t c = c0 + lc, r = r0 + rr;
-        if (!FULL && (c >= a.C || r >= a.R)) continue;
-        const CodeT v = reinterpret_cast<const CodeT*>(tile_t + chunk_slot(lc, rr >> 3) * kChunkBytes)[rr & 7];
-        ctp[c * a.ldt + __ldg(a.pos_rows + r)] = v;
-      }
-      goto scales;
-    }
-    {
-    // each transposed row (one tile column) holds 64 codes = 8 chunks; 16-byte stores
-    constexpr int kChunksPerStore = 16 / kChunkBytes;            // 1 (BF16) or 2 (E4M3)
-    constexpr int kStoresPerRow = 8 / kChunksPerStore;
-    constexpr int E = 16 / sizeof(CodeT);                         // codes per 16-byte store
-    uint8_t* ct = static_cast<uint8_t*>(a.codes_t);
-#pragma unroll
-    for (int idx = tid; idx < kQC * kStoresPerRow; idx += 256) {
-      const int lc = idx / kStoresPerRow, st = idx % kStoresPerRow;
-      const int64_t c = c0 + lc;
-      const int64_t rs = r0 + st * E;
-      if (!FULL && (c >= a.C || rs >= a.R)) continue;
-      uint4 v;
-      if constexpr (kChunksPerStore == 1) {
-        v = *reinterpret_cast<const uint4*>(tile_t + chunk_slot(lc, st) * kChunkBytes);
-      } else {
-        const uint2 lo = *reinterpret_cast<const uint2*>(tile_t + chunk_slot(lc, 2 * st) * kChunkBytes);
-        const uint2 hi = *reinterpret_cast<const uint2*>(tile_t + chunk_slot(lc, 2 * st + 1) * kChunkBytes);
-        v = make_uint4(lo.x, lo.y, hi.x, hi.y);
-      }
-      uint8_t* dst = ct + (c * a.ldt + rs) * static_cast<int64_t>(sizeof(CodeT));
-      if (FULL || (a.vec_t && rs + E <= a.R)) {
-        *reinterpret_cast<uint4*>(dst) = v;
-      } else {
-        const uint8_t* vb = reinterpret_cast<const uint8_t*>(&v);
-        for (int e = 0; e < E && rs + e < a.R; ++e)
-          for (int b = 0; b < static_cast<int>(sizeof(CodeT)); ++b)
-            dst[e * sizeof(CodeT) + b] = vb[e * sizeof(CodeT) + b];
-      }
-    }
-    }
-  }
-scales:
-  // scales: s = tau_0 / Q, or range / Q per channel (0 for an all-zero channel)
-  if (GRAN == SQ_GRAN_SHIFT) {
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
-      const float tau = __ldg(a.rt);
-      *a.scale_out = zero_all ? 0.0f : __fdiv_rn(tau, Qf);
-    }
-  } else if (GRAN == SQ_GRAN_PER_COL) {
-    if (blockIdx.y == 0 && wq == 0) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (FULL || cb + j < a.C)
-          a.scale_out[cb + j] = colzero[j] ? 0.0f : __fdiv_rn(__ldg(a.rt + cb + j), Qf);
-    }
-  } else {
-    if (blockIdx.x == 0 && lane == 0) {
-#pragma unroll
-      for (int i = 0; i < kQRowsPerWarp; ++i) {
-        const int64_t r = r0 + wq * 8 + i;
-        if (FULL || r < a.R) {
-          const float rg = __ldg(a.rt + r);
-          const float inv = __fdiv_rn(Qf, rg);
-          const bool z = !(rg > 0.0f) || !isfinite(rg) || !isfinite(inv);
-          a.scale_out[r] = z ? 0.0f : __fdiv_rn(rg, Qf);
-        }
-      }
-    }
-  }
+  if (a.codes_t != nullptr) stage_chunks<CodeT>(t.p, a.lg, tile_smem);
 }
 
-template <typename CodeT, int GRAN, int MODE, bool FOLD>
-__global__ void __launch_bounds__(256) quantize_kernel(const QuantArgs a) {
-  __shared__ __align__(16) uint8_t tile_t[kQC * 8 * 8 * sizeof(CodeT)];
+// One tile of a tensor.
+// WAIT: x may be read before the preceding kernel has completed (it did not write x), its
+// results only after the wait.
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, bool WAIT = false>
+__device__ __forceinline__ void quantize_block(const QuantArgs& a, unsigned bx, unsigned by, uint32_t tile_smem) {
+  bool fast = register_tile<FORM>(a, bx, by);
+  float4 x[8];
+  if (fast) load_registers<FORM>(a, bx, by, x);
+  if (WAIT) griddep_wait();
+  const QuadState t = quad_state<GRAN, MODE, FOLD>(a, bx, by);
+  fast = fast && !__any_sync(0xFFFFFFFFu, t.rare);   // (each warp by itself: their parts of the tile are their own)
+  if (fast) {
+    quantize_registers<CodeT, FORM, GRAN, MODE, FOLD>(a, t, x, tile_smem);
+  } else {
+    load_tile(a, bx, by, tile_smem + (threadIdx.x >> 5) * kWarpBytes);
+    quantize_rows<CodeT, GRAN, MODE, FOLD>(a, t, tile_smem);
+  }
+  if (a.codes_t != nullptr) store_transposed<CodeT>(a, tile_smem, bx, by);
+}
+
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD>
+__global__ void __launch_bounds__(kQuantThreads, 4) quantize_kernel(const QuantArgs a) {
+  __shared__ __align__(128) uint8_t tile[8 * kWarpBytes];
   // launched early behind the range pass: nothing it wrote (nor x) is read before it is done
-  griddep_wait();
-  const bool full = (static_cast<int64_t>(blockIdx.y) + 1) * kQR <= a.R &&
-                    (static_cast<int64_t>(blockIdx.x) + 1) * kQC <= a.C && a.vec_in &&
-                    (a.codes == nullptr || a.vec_out) && (a.codes_t == nullptr || a.vec_t);
-  if (full)
-    quantize_tile<CodeT, GRAN, MODE, FOLD, true>(a, tile_t);
-  else
-    quantize_tile<CodeT, GRAN, MODE, FOLD, false>(a, tile_t);
+  if (!a.beside) griddep_wait();
+  griddep_launch_dependents();
+  quantize_block<CodeT, FORM, GRAN, MODE, FOLD>(a, blockIdx.x, blockIdx.y, smem_u32(tile));
+  if (a.beside) griddep_wait();
 }
 
 // Launch with programmatic stream serialization: the kernel may begin launching while the
@@ -742,70 +1088,238 @@ static cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, 
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <typename CodeT>
-static void launch_quantize(const QuantArgs& a, dim3 grid, cudaStream_t s) {
-  const bool fold = a.fold != nullptr;
-  if (a.gran == SQ_GRAN_SHIFT) {
-    if (a.mode == SQ_ROUND_NEAREST_EVEN)
-      launch_pdl(quantize_kernel<CodeT, SQ_GRAN_SHIFT, SQ_ROUND_NEAREST_EVEN, false>, grid, dim3(256), s, a);
-    else
-      launch_pdl(quantize_kernel<CodeT, SQ_GRAN_SHIFT, SQ_ROUND_STOCHASTIC, false>, grid, dim3(256), s, a);
-  } else if (a.gran == SQ_GRAN_PER_COL) {
-    if (a.mode == SQ_ROUND_NEAREST_EVEN) {
-      if (fold) launch_pdl(quantize_kernel<CodeT, SQ_GRAN_PER_COL, SQ_ROUND_NEAREST_EVEN, true>, grid, dim3(256), s, a);
-      else launch_pdl(quantize_kernel<CodeT, SQ_GRAN_PER_COL, SQ_ROUND_NEAREST_EVEN, false>, grid, dim3(256), s, a);
-    } else {
-      if (fold) launch_pdl(quantize_kernel<CodeT, SQ_GRAN_PER_COL, SQ_ROUND_STOCHASTIC, true>, grid, dim3(256), s, a);
-      else launch_pdl(quantize_kernel<CodeT, SQ_GRAN_PER_COL, SQ_ROUND_STOCHASTIC, false>, grid, dim3(256), s, a);
-    }
+template <typename CodeT, int FORM, int GRAN, bool FOLD>
+static void launch_mode(const QuantArgs& a, int mode, dim3 grid, cudaStream_t s) {
+  if (mode == SQ_ROUND_NEAREST_EVEN)
+    launch_pdl(quantize_kernel<CodeT, FORM, GRAN, SQ_ROUND_NEAREST_EVEN, FOLD>, grid, dim3(kQuantThreads), s, a);
+  else
+    launch_pdl(quantize_kernel<CodeT, FORM, GRAN, SQ_ROUND_STOCHASTIC, FOLD>, grid, dim3(kQuantThreads), s, a);
+}
+
+template <typename CodeT, int FORM>
+static void launch_gran(const QuantArgs& a, int gran, int mode, dim3 grid, cudaStream_t s) {
+  const bool fold = FORM != kOrdered && (a.fold != nullptr || a.frange != nullptr);   // group-ordered codes carry no fold
+  if (gran == SQ_GRAN_SHIFT) {
+    launch_mode<CodeT, FORM, SQ_GRAN_SHIFT, false>(a, mode, grid, s);
+  } else if (gran == SQ_GRAN_PER_COL) {
+    if (fold) launch_mode<CodeT, FORM, SQ_GRAN_PER_COL, FORM != kOrdered>(a, mode, grid, s);
+    else launch_mode<CodeT, FORM, SQ_GRAN_PER_COL, false>(a, mode, grid, s);
   } else {
-    if (a.mode == SQ_ROUND_NEAREST_EVEN) {
-      if (fold) launch_pdl(quantize_kernel<CodeT, SQ_GRAN_PER_ROW, SQ_ROUND_NEAREST_EVEN, true>, grid, dim3(256), s, a);
-      else launch_pdl(quantize_kernel<CodeT, SQ_GRAN_PER_ROW, SQ_ROUND_NEAREST_EVEN, false>, grid, dim3(256), s, a);
-    } else {
-      if (fold) launch_pdl(quantize_kernel<CodeT, SQ_GRAN_PER_ROW, SQ_ROUND_STOCHASTIC, true>, grid, dim3(256), s, a);
-      else launch_pdl(quantize_kernel<CodeT, SQ_GRAN_PER_ROW, SQ_ROUND_STOCHASTIC, false>, grid, dim3(256), s, a);
-    }
+    if (fold) launch_mode<CodeT, FORM, SQ_GRAN_PER_ROW, FORM != kOrdered>(a, mode, grid, s);
+    else launch_mode<CodeT, FORM, SQ_GRAN_PER_ROW, false>(a, mode, grid, s);
+  }
+}
+
+template <typename CodeT>
+static void launch_quantize(const QuantArgs& a, int gran, int mode, dim3 grid, cudaStream_t s) {
+  switch (a.form) {
+    case kAligned: launch_gran<CodeT, kAligned>(a, gran, mode, grid, s); break;
+    case kShifted: launch_gran<CodeT, kShifted>(a, gran, mode, grid, s); break;
+    default: launch_gran<CodeT, kOrdered>(a, gran, mode, grid, s); break;
   }
 }
 
 // Both roles of a weight from one pass over it (Sec. 5.1): the forward GEMM's
 // per-out-channel codes (gran PER_COL, written transposed, the fold indexed by row) and loss
 // propagation's per-in-channel codes (gran PER_ROW, natural layout, the fold indexed by
-// column), both from the one load of the block's tile held in registers.  Re-reading the
+// column), both from the one load of the block's tile into shared memory.  Re-reading the
 // tile for the second role (from L2) put a second load latency in every block: 87 us for
-// large_linear's [4096, 11008] weight against 76 us now.  The tile held across both roles
-// needs about 98 registers; three blocks per SM (80, a few bytes spilled) measured 76 us, two (98) 93 us,
-// four (64, spilling) 73 us on the wide weights but slower on small ones.
-template <typename CodeT, bool FF, bool FD>
-__global__ void __launch_bounds__(256, 3) quantize_weight_kernel(const QuantArgs af, const QuantArgs ad) {
-  __shared__ __align__(16) uint8_t tile_t[kQC * 8 * 8 * sizeof(CodeT)];
-  griddep_wait();
-  const bool inside = (static_cast<int64_t>(blockIdx.y) + 1) * kQR <= af.R &&
-                      (static_cast<int64_t>(blockIdx.x) + 1) * kQC <= af.C && af.vec_in;
-  float4 xin[kQRowsPerWarp];   // both roles read the same tensor: af and ad share x, R, C, ld
-  if (inside)
-    load_quant_tile<true>(af, xin);
+// large_linear's [4096, 11008] weight against 76 us with the tile kept.
+template <typename CodeT, int FORM, bool FF, bool FD, bool WAIT = false>
+__device__ __forceinline__ void quantize_weight_block(const QuantArgs& af, const QuantArgs& ad, unsigned bx,
+                                                      unsigned by, uint32_t tile_smem) {
+  // both roles read the same tensor: af and ad share x, R, C, ld, lg
+  constexpr int kCol = SQ_GRAN_PER_COL, kRow = SQ_GRAN_PER_ROW, kRn = SQ_ROUND_NEAREST_EVEN;
+  bool fast = register_tile<FORM>(af, bx, by) && register_tile<FORM>(ad, bx, by);
+  float4 x[8];
+  if (fast) load_registers<FORM>(af, bx, by, x);
+  if (WAIT) griddep_wait();
+  const QuadState td = quad_state<kRow, kRn, FD>(ad, bx, by);
+  fast = fast && !__any_sync(0xFFFFFFFFu, td.rare);
+  if (fast) {
+    quantize_registers<CodeT, FORM, kRow, kRn, FD>(ad, td, x, tile_smem);
+  } else {   // the per-in-channel role has no transposed copy: it leaves the tile as it is
+    load_tile(af, bx, by, tile_smem + (threadIdx.x >> 5) * kWarpBytes);
+    quantize_rows<CodeT, kRow, kRn, FD>(ad, td, tile_smem);
+  }
+  const QuadState tf = quad_state<kCol, kRn, FF>(af, bx, by);
+  if (fast && __any_sync(0xFFFFFFFFu, tf.rare)) {
+    load_tile(af, bx, by, tile_smem + (threadIdx.x >> 5) * kWarpBytes);
+    fast = false;
+  }
+  if (fast)
+    quantize_registers<CodeT, FORM, kCol, kRn, FF>(af, tf, x, tile_smem);
   else
-    load_quant_tile<false>(af, xin);
-  if (inside && af.vec_t)
-    quantize_tile<CodeT, SQ_GRAN_PER_COL, SQ_ROUND_NEAREST_EVEN, FF, true, false>(af, tile_t, xin);
-  else
-    quantize_tile<CodeT, SQ_GRAN_PER_COL, SQ_ROUND_NEAREST_EVEN, FF, false, false>(af, tile_t, xin);
-  if (inside && ad.vec_out)
-    quantize_tile<CodeT, SQ_GRAN_PER_ROW, SQ_ROUND_NEAREST_EVEN, FD, true, false>(ad, tile_t, xin);
-  else
-    quantize_tile<CodeT, SQ_GRAN_PER_ROW, SQ_ROUND_NEAREST_EVEN, FD, false, false>(ad, tile_t, xin);
+    quantize_rows<CodeT, kCol, kRn, FF>(af, tf, tile_smem);
+  store_transposed<CodeT>(af, tile_smem, bx, by);
+}
+
+template <typename CodeT, int FORM, bool FF, bool FD>
+__global__ void __launch_bounds__(kQuantThreads, 4) quantize_weight_kernel(const QuantArgs af, const QuantArgs ad) {
+  __shared__ __align__(128) uint8_t tile[8 * kWarpBytes];
+  if (!af.beside) griddep_wait();
+  griddep_launch_dependents();
+  quantize_weight_block<CodeT, FORM, FF, FD>(af, ad, blockIdx.x, blockIdx.y, smem_u32(tile));
+  if (af.beside) griddep_wait();
+}
+
+template <typename CodeT, int FORM>
+static void launch_weight_folds(const QuantArgs& af, const QuantArgs& ad, dim3 grid, cudaStream_t s) {
+  const bool ff = af.fold != nullptr || af.frange != nullptr, fd = ad.fold != nullptr || ad.frange != nullptr;
+  const dim3 block(kQuantThreads);
+  if (ff && fd) launch_pdl(quantize_weight_kernel<CodeT, FORM, true, true>, grid, block, s, af, ad);
+  else if (ff) launch_pdl(quantize_weight_kernel<CodeT, FORM, true, false>, grid, block, s, af, ad);
+  else if (fd) launch_pdl(quantize_weight_kernel<CodeT, FORM, false, true>, grid, block, s, af, ad);
+  else launch_pdl(quantize_weight_kernel<CodeT, FORM, false, false>, grid, block, s, af, ad);
 }
 
 template <typename CodeT>
-static void launch_quantize_weight(const QuantArgs& af, const QuantArgs& ad, dim3 grid,
-                                   cudaStream_t s) {
-  const bool ff = af.fold != nullptr, fd = ad.fold != nullptr;
-  if (ff && fd) launch_pdl(quantize_weight_kernel<CodeT, true, true>, grid, dim3(256), s, af, ad);
-  else if (ff) launch_pdl(quantize_weight_kernel<CodeT, true, false>, grid, dim3(256), s, af, ad);
-  else if (fd) launch_pdl(quantize_weight_kernel<CodeT, false, true>, grid, dim3(256), s, af, ad);
-  else launch_pdl(quantize_weight_kernel<CodeT, false, false>, grid, dim3(256), s, af, ad);
+static void launch_quantize_weight(const QuantArgs& af, const QuantArgs& ad, dim3 grid, cudaStream_t s) {
+  if (af.form == kShifted)
+    launch_weight_folds<CodeT, kShifted>(af, ad, grid, s);
+  else
+    launch_weight_folds<CodeT, kAligned>(af, ad, grid, s);
+}
+
+// ============================================================= a layer's quantizer passes
+// The quantizer passes of a layer step (X, dY and W: three tensors, eleven launches one by
+// one, each short next to its launch gap and its last wave) as three launches: the
+// accumulators zeroed, every tensor's range pass, every tensor's quantization.  The grouping
+// needs no launch of its own: the range pass also keeps tau_0 (kTauSlots words per tensor),
+// and a quantizer block forms the exponents of its own columns, and the shifts it folds into
+// weight codes, from the ranges and tau_0.
+struct LayerInit {
+  unsigned* p[5];
+  int64_t n[5];
+};
+
+// The first of the three, launched behind whatever precedes it: it waits for that before it
+// writes, and lets the range pass launch only then.
+__global__ void __launch_bounds__(256) layer_init_kernel(const LayerInit z) {
+  griddep_wait();
+  griddep_launch_dependents();
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+#pragma unroll
+  for (int k = 0; k < 5; ++k)
+    for (int64_t i = i0; i < z.n[k]; i += stride) z.p[k][i] = 0u;
+}
+
+constexpr int kZeroVecs = 2048;   // 16-byte words a zeroing block clears
+constexpr int kZeroRegions = 3;
+
+struct LayerRange {
+  RangeView w, g, x;
+  int wrun;                       // column blocks a weight block walks
+  int glg, xlg;
+  unsigned wgx, ggx, xgx;         // blocks across the columns
+  unsigned zend, wend, gend;      // first block past the zeroing, W's and dY's blocks
+  uint4* zero[kZeroRegions];      // regions the layer's GEMMs want zeroed
+  int64_t zvecs[kZeroRegions];    // in 16-byte words
+  unsigned zblocks[kZeroRegions];
+  unsigned *wcols, *wrows, *gcols, *xcols, *gtau, *xtau;
+  int* status;
+};
+
+// one tile of a ShiftQuant tensor: column maxima and their largest to a tau_0 slot.  An atomic
+// goes out only where it would raise the value seen.
+template <int FORM>
+__device__ __forceinline__ void layer_range_tile(const RangeView& v, int lg, unsigned bx, unsigned by, unsigned* red,
+                                                 unsigned* cols, unsigned* tau, int* status) {
+  const int tid = threadIdx.x;
+  const int tc = 4 << lg, rpp = (kColTx * kColTy) >> lg;
+  const int qc = tid & ((1 << lg) - 1), ro = tid >> lg;
+  const int64_t cb = static_cast<int64_t>(bx) * tc;
+  unsigned m[4] = {0u, 0u, 0u, 0u}, rm[8];
+  tile_maxima<false, FORM>(v, lg, cb, static_cast<int64_t>(by) * 8 * rpp + ro, qc, m, rm);
+  put_maxima<FORM>(red, lg, ro, qc, m);
+  __syncthreads();
+  griddep_wait();   // the accumulators are zero
+  griddep_launch_dependents();
+  if (tid >= 128) return;
+  unsigned w = 0u;
+  const int64_t c = cb + tid;
+  if (tid < tc && c < v.C) {
+    w = get_maximum(red, lg, tid);
+    unsigned* p = column_bits<FORM>(cols, v, c);
+    if (w > __ldcg(p)) atomicMax(p, w);
+  }
+  w = __reduce_max_sync(0xFFFFFFFFu, w);
+  if ((tid & 31) == 0) {
+    unsigned* p = tau + (bx + by) % kTauSlots;
+    if (w > __ldcg(p)) atomicMax(p, w);
+    if (w >= 0x7F800000u) atomicOr(status, kDevNonFinite);
+  }
+}
+
+// a tile of whichever form the tensor has; PLAIN: all three are kViewVec
+template <bool PLAIN>
+__device__ __forceinline__ void layer_range_any(const RangeView& v, int lg, unsigned gx, unsigned b, unsigned* red,
+                                                unsigned* cols, unsigned* tau, int* status) {
+  if (PLAIN || v.form == kViewVec)
+    layer_range_tile<kViewVec>(v, lg, b % gx, b / gx, red, cols, tau, status);
+  else if (v.form == kViewFolded)
+    layer_range_tile<kViewFolded>(v, lg, b % gx, b / gx, red, cols, tau, status);
+  else
+    layer_range_tile<kViewStrided>(v, lg, b % gx, b / gx, red, cols, tau, status);
+}
+
+template <bool PLAIN>
+__global__ void __launch_bounds__(256, 4) layer_range_kernel(const LayerRange a) {
+  __shared__ unsigned red[kColTy * kColTx * 4];
+  unsigned b = blockIdx.x;
+  if (b < a.zend) {
+    // (the preceding GEMM may still read these until the first kernel has waited for it)
+    griddep_wait();
+    griddep_launch_dependents();
+    int k = 0;
+    while (k + 1 < kZeroRegions && b >= a.zblocks[k]) b -= a.zblocks[k++];
+    const int64_t end = min(a.zvecs[k], (static_cast<int64_t>(b) + 1) * kZeroVecs);
+    for (int64_t i = static_cast<int64_t>(b) * kZeroVecs + threadIdx.x; i < end; i += 256)
+      a.zero[k][i] = make_uint4(0u, 0u, 0u, 0u);
+  } else if (b < a.wend) {
+    b -= a.zend;
+    bool bad = false;
+    if (PLAIN || a.w.form == kViewVec)
+      weight_range_run<kViewVec>(a.w, b / a.wgx, static_cast<int64_t>(b % a.wgx) * a.wrun, a.wrun, red, a.wcols,
+                                 a.wrows, &bad);
+    else
+      weight_range_run<kViewStrided>(a.w, b / a.wgx, static_cast<int64_t>(b % a.wgx) * a.wrun, a.wrun, red, a.wcols,
+                                     a.wrows, &bad);
+    griddep_launch_dependents();
+    if (bad) atomicOr(a.status, kDevNonFinite);
+  } else if (b < a.gend) {
+    b -= a.wend;
+    layer_range_any<PLAIN>(a.g, a.glg, a.ggx, b, red, a.gcols, a.gtau, a.status);
+  } else {
+    b -= a.gend;
+    layer_range_any<PLAIN>(a.x, a.xlg, a.xgx, b, red, a.xcols, a.xtau, a.status);
+  }
+}
+
+// The blocks of X, W and dY one list after another: X was the last tensor of the range pass,
+// so as much of it as fits is still in L2.
+struct LayerQuant {
+  QuantArgs x, g, wf, wd;
+  unsigned xgx, ggx, wgx;
+  unsigned xend, wend;   // first block past X's and W's
+};
+
+template <typename CodeT, int FORM>
+__global__ void __launch_bounds__(kQuantThreads, 4) layer_quantize_kernel(const LayerQuant q) {
+  __shared__ __align__(128) uint8_t tile[8 * kWarpBytes];
+  const uint32_t smem = smem_u32(tile);
+  griddep_launch_dependents();
+  unsigned b = blockIdx.x;
+  if (b < q.xend) {
+    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_NEAREST_EVEN, false, true>(q.x, b % q.xgx, b / q.xgx, smem);
+  } else if (b < q.wend) {
+    b -= q.xend;
+    quantize_weight_block<CodeT, FORM, true, true, true>(q.wf, q.wd, b % q.wgx, b / q.wgx, smem);
+  } else {
+    b -= q.wend;
+    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_STOCHASTIC, false, true>(q.g, b % q.ggx, b / q.ggx, smem);
+  }
 }
 
 // ============================================================ group order (Sec. 3.2)
@@ -895,69 +1409,280 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// How the range pass reads x [rows, cols].  Folding applies to dense unaligned tensors; a
+// weight's row maxima need its own rows (fold = false).
+static RangeView range_view(const float* x, int64_t rows, int64_t cols, int64_t ld, bool fold) {
+  RangeView v = {x, rows, cols, ld, (ld % 4 == 0) && aligned16(x) ? kViewVec : kViewStrided, cols, 0};
+  const int64_t f = cols % 2 == 0 ? 2 : 4;   // rows that make a multiple of four elements
+  if (v.form == kViewStrided && fold && ld == cols && aligned16(x) && rows >= f) {
+    v.R = rows / f;
+    v.C = v.ld = f * cols;
+    v.form = kViewFolded;
+    v.tail = (rows - v.R * f) * cols;
+  }
+  return v;
+}
+
+// log2 of a quarter of the range pass's tile width: the column count rounded up to a power of
+// two, 4 to 128
+static int range_lg(int64_t cols) {
+  int lg = 0;
+  while (lg < 5 && (int64_t(4) << lg) < cols) ++lg;
+  return lg;
+}
+
 // The range pass of x [rows, cols] (0 < rows, 0 < cols < 2^36, checked by the callers):
 // one block per tile, narrow tensors in whole clusters along the rows; with
 // row_bits also the per-row maxima.
 static cudaError_t launch_range(const float* x, int64_t rows, int64_t cols, int64_t ld,
                                 unsigned* col_bits, unsigned* row_bits, int* status,
                                 cudaStream_t s) {
-  // the tile: the column count rounded up to a power of two (4 .. 128) wide, 1024 elements;
+  const RangeView v = range_view(x, rows, cols, ld, row_bits == nullptr);
   // a weight's row ranges need whole 128-column warp rows
-  int lg = 5;
-  if (row_bits == nullptr)
-    for (lg = 0; lg < 5 && (int64_t(4) << lg) < cols; ++lg) {
-    }
+  const int lg = row_bits != nullptr ? 5 : range_lg(v.C);
   const int64_t tc = int64_t(4) << lg;
-  const int64_t cblocks = (cols + tc - 1) / tc;   // < 2^29: cols < 2^36, tc = 128 past 64
-  const int64_t tiles = (rows + 8 * (256 >> lg) - 1) / (8 * (256 >> lg));
+  const int64_t cblocks = (v.C + tc - 1) / tc;   // < 2^31: C < 2^38, tc = 128 past 64
+  const int64_t tiles = (v.R + 8 * (256 >> lg) - 1) / (8 * (256 >> lg));
   const int cl = cols <= kRangeClusterMaxCols ? kRangeCluster : 1;
-  const int vec = (ld % 4 == 0) && aligned16(x);
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.blockDim = dim3(kColTx, kColTy);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaError_t err;
   if (row_bits != nullptr && cl == 1) {
     // a wide weight: runs of column blocks per block (weight_range_kernel)
     const int64_t runs = (cblocks + kWeightRun - 1) / kWeightRun;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(static_cast<unsigned>(runs), static_cast<unsigned>(tiles < 65535 ? tiles : 65535));
-    cfg.blockDim = dim3(kColTx, kColTy);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t err = cudaLaunchKernelEx(&cfg, weight_range_kernel, x, rows, cols, ld, vec,
-                                         col_bits, row_bits, status);
+    err = cudaLaunchKernelEx(&cfg, v.form == kViewVec ? weight_range_kernel<kViewVec> : weight_range_kernel<kViewStrided>, v,
+                             col_bits, row_bits, status);
     if (err == cudaSuccess) err = cudaGetLastError();
     return err;
   }
   const int64_t max_rblocks = 65535 / cl * cl;
   int64_t rblocks = (tiles + cl - 1) / cl * cl;
   if (rblocks > max_rblocks) rblocks = max_rblocks;
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3(static_cast<unsigned>(cblocks), static_cast<unsigned>(rblocks));
-  cfg.blockDim = dim3(kColTx, kColTy);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = 1;
   attr[1].val.clusterDim.y = cl;
   attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
   cfg.numAttrs = cl > 1 ? 2 : 1;
-  cudaError_t err;
-  if (row_bits != nullptr)   // a narrow weight (wide ones returned above)
-    err = cudaLaunchKernelEx(&cfg, colmax_kernel<kRangeCluster, true>, x, rows, cols, ld, vec, lg,
-                             col_bits, row_bits, status);
-  else
-    err = cl > 1 ? cudaLaunchKernelEx(&cfg, colmax_kernel<kRangeCluster, false>, x, rows, cols, ld, vec,
-                                      lg, col_bits, row_bits, status)
-                 : cudaLaunchKernelEx(&cfg, colmax_kernel<1, false>, x, rows, cols, ld, vec, lg, col_bits,
-                                      row_bits, status);
+  auto kernel = row_bits != nullptr   // a narrow weight (wide ones returned above)
+                    ? (v.form == kViewVec ? colmax_kernel<kRangeCluster, true, kViewVec>
+                                          : colmax_kernel<kRangeCluster, true, kViewStrided>)
+                : cl > 1 ? (v.form == kViewVec      ? colmax_kernel<kRangeCluster, false, kViewVec>
+                            : v.form == kViewFolded ? colmax_kernel<kRangeCluster, false, kViewFolded>
+                                                    : colmax_kernel<kRangeCluster, false, kViewStrided>)
+                         : (v.form == kViewVec      ? colmax_kernel<1, false, kViewVec>
+                            : v.form == kViewFolded ? colmax_kernel<1, false, kViewFolded>
+                                                    : colmax_kernel<1, false, kViewStrided>);
+  err = cudaLaunchKernelEx(&cfg, kernel, v, lg, col_bits, row_bits, status);
   if (err == cudaSuccess) err = cudaGetLastError();
   return err;
+}
+
+// the sizes one quantizer launch takes (64-row tiles in a grid's 65535 rows)
+static bool quant_grid_ok(int64_t rows, int64_t cols) {
+  return (cols + 127) / 128 <= 0x7FFFFFFF && (rows + 63) / 64 <= 65535;
+}
+
+static dim3 quant_grid(const QuantArgs& a) {
+  return dim3(static_cast<unsigned>((a.C + tile_cols(a.lg) - 1) / tile_cols(a.lg)),
+              static_cast<unsigned>((a.R + tile_rows(a.lg) - 1) / tile_rows(a.lg)));
+}
+
+// alignment of the tensor and its outputs (given with their group orders), and from it the
+// form of the launch's register path
+static void set_alignment(QuantArgs* a, int cbytes) {
+  a->vec_in = aligned16(a->x) && a->ld % 4 == 0;
+  a->vec_out = a->codes != nullptr && a->ldc % 4 == 0 && reinterpret_cast<uintptr_t>(a->codes) % (4 * cbytes) == 0;
+  a->vec_t = a->codes_t != nullptr && (a->ldt * cbytes) % 16 == 0 && aligned16(a->codes_t);
+  a->lg = tile_lg(a->C);
+  const bool ordered = a->pos_cols != nullptr || a->pos_rows != nullptr;
+  a->form = ordered ? kOrdered : (a->vec_in ? kAligned : kShifted);
+  const bool in = a->form == kShifted ? aligned16(a->x) : a->vec_in != 0;
+  a->fast = in && (a->codes == nullptr || a->vec_out || a->pos_cols != nullptr);
+}
+
+// both roles of a weight (the folds are set by the caller)
+static void weight_args(QuantArgs* af, QuantArgs* ad, const float* w, int64_t rows, int64_t cols, int64_t ld,
+                        int bits, int n_groups, const float* range_out_ch, const float* range_in_ch,
+                        void* codes_fwd, int64_t ld_fwd, float* scale_fwd, void* codes_dgrad,
+                        int64_t ld_dgrad, float* scale_dgrad) {
+  const int cbytes = code_bytes(code_type(bits, n_groups));
+  memset(af, 0, sizeof(*af));
+  af->x = w;
+  af->R = rows;
+  af->C = cols;
+  af->ld = ld;
+  af->Q = q_of_bits(bits);
+  af->G = n_groups;
+  *ad = *af;
+  af->rt = range_out_ch;
+  af->codes_t = codes_fwd;
+  af->ldt = ld_fwd;
+  af->scale_out = scale_fwd;
+  set_alignment(af, cbytes);
+  ad->rt = range_in_ch;
+  ad->codes = codes_dgrad;
+  ad->ldc = ld_dgrad;
+  ad->scale_out = scale_dgrad;
+  set_alignment(ad, cbytes);
+}
+
+// ------------------------------------------------------------- a layer's passes
+int check_layer_quant(const sq_layer_step* L) {
+  const int64_t M = L->M, K = L->K, N = L->N;
+  if (K >= (int64_t(1) << 36) || N >= (int64_t(1) << 36)) return fail(SQ_EINVAL, "calibrate: too many columns");
+  const struct { int64_t cols, ld, ldt; const void* t; } t[2] = {{K, L->ld_x, L->ld_xt, L->xt_codes},
+                                                                {N, L->ld_g, L->ld_gt, L->gt_codes}};
+  for (int i = 0; i < 2; ++i) {
+    if (t[i].ld < t[i].cols) return fail(SQ_EINVAL, "quantize: ld_codes < cols");
+    if (t[i].t != nullptr && t[i].ldt < M) return fail(SQ_EINVAL, "quantize: ld_t < rows");
+    if (!quant_grid_ok(M, t[i].cols))
+      return fail(SQ_EUNSUPPORTED, "quantize: tensor too large for one launch (%lld x %lld)",
+                  static_cast<long long>(M), static_cast<long long>(t[i].cols));
+  }
+  if (L->ld_wf < K) return fail(SQ_EINVAL, "quantize_weight: ld_fwd < rows");
+  if (L->ld_wd < N) return fail(SQ_EINVAL, "quantize_weight: ld_dgrad < cols");
+  if (!quant_grid_ok(K, N))
+    return fail(SQ_EUNSUPPORTED, "quantize_weight: tensor too large for one launch (%lld x %lld)",
+                static_cast<long long>(K), static_cast<long long>(N));
+  return SQ_OK;
+}
+
+// blocks of a range pass of v in tiles of 4 << lg columns, and across the columns
+static int64_t range_blocks(const RangeView& v, int lg, unsigned* gx) {
+  const int64_t tc = int64_t(4) << lg, rows = 8 * (256 >> lg);
+  const int64_t nx = (v.C + tc - 1) / tc;
+  *gx = static_cast<unsigned>(nx);
+  return nx * ((v.R + rows - 1) / rows);
+}
+
+bool layer_quant_fits(const sq_layer_step* L) {
+  // every block index in 31 bits, with room to spare
+  const double m = L->M / 32.0 + 1, k = L->K / 32.0 + 1, n = L->N / 32.0 + 1;
+  return m * (k + n) + k * n < 1e9;
+}
+
+// The codes of a layer's tensors: one launch while its blocks stay within two resident waves
+// (four blocks on each of 152 SMs), where launches and their tails are what counts; above, one
+// launch per tensor, each running beside the tail of the one before it, each body with the
+// instruction cache and the registers to itself.  Whole steps, one launch against three:
+// 256 x 512 x 512 (4-bit) 24.7 / 26.6 us; 12608 x 768 x 3072 (6-bit) 271 / 261 us,
+// 4096 x 11008 x 4096 (8-bit) 957 / 939 us (with the three one after another 123 us where
+// beside one another take 115 us: 12544 x 2304 x 256, 4-bit).
+constexpr unsigned kLayerQuantMaxBlocks = 8 * 152;
+
+template <typename CodeT>
+static cudaError_t launch_layer_quantize(const LayerQuant& q, unsigned blocks, cudaStream_t s) {
+  if (blocks > kLayerQuantMaxBlocks) {
+    QuantArgs g = q.g, wf = q.wf;
+    g.beside = wf.beside = 1;
+    launch_quantize<CodeT>(q.x, SQ_GRAN_SHIFT, SQ_ROUND_NEAREST_EVEN, quant_grid(q.x), s);
+    launch_quantize_weight<CodeT>(wf, q.wd, quant_grid(wf), s);
+    launch_quantize<CodeT>(g, SQ_GRAN_SHIFT, SQ_ROUND_STOCHASTIC, quant_grid(g), s);
+    return cudaGetLastError();
+  }
+  const bool aligned = q.x.form == kAligned && q.g.form == kAligned && q.wf.form == kAligned;
+  return aligned ? launch_pdl(layer_quantize_kernel<CodeT, kAligned>, dim3(blocks), dim3(kQuantThreads), s, q)
+                 : launch_pdl(layer_quantize_kernel<CodeT, kShifted>, dim3(blocks), dim3(kQuantThreads), s, q);
+}
+
+int quantize_layer(const sq_layer_step* L, uint64_t seed, unsigned* words, const ZeroRegion* zero, int nzero,
+                   cudaStream_t s) {
+  const int64_t M = L->M, K = L->K, N = L->N;
+  const int cbytes = code_bytes(code_type(L->bits, L->n_groups));
+  unsigned* xtau = words + kTauSlots;
+  unsigned* gtau = words + 2 * kTauSlots;
+  auto bits = [](float* p) { return reinterpret_cast<unsigned*>(p); };
+  // 1. accumulators
+  LayerInit z = {{bits(L->x_range), bits(L->g_range), bits(L->wf_range), bits(L->wd_range), words},
+                 {K, N, N, K, 3 * kTauSlots}};
+  const int64_t widest = K > N ? K : N;
+  const int64_t ib = (widest + 255) / 256;
+  cudaError_t err = launch_pdl(layer_init_kernel, dim3(static_cast<unsigned>(ib < 152 ? ib : 152)), dim3(256), s, z);
+  if (err != cudaSuccess) return cuda_fail(err, "layer_init_kernel launch");
+  // 2. ranges
+  LayerRange r;
+  memset(&r, 0, sizeof(r));
+  r.w = range_view(L->w, K, N, N, false);
+  r.g = range_view(L->dy, M, N, N, true);
+  r.x = range_view(L->x, M, K, K, true);
+  r.glg = range_lg(r.g.C);
+  r.xlg = range_lg(r.x.C);
+  // runs of column blocks only where a weight is wide (see weight_range_kernel)
+  r.wrun = N > kRangeClusterMaxCols ? kWeightRun : 1;
+  int64_t blocks = 0;
+  for (int k = 0; k < nzero; ++k) {
+    r.zero[k] = static_cast<uint4*>(zero[k].p);
+    r.zvecs[k] = static_cast<int64_t>(zero[k].bytes / 16);
+    r.zblocks[k] = static_cast<unsigned>((r.zvecs[k] + kZeroVecs - 1) / kZeroVecs);
+    blocks += r.zblocks[k];
+  }
+  r.zend = static_cast<unsigned>(blocks);
+  r.wgx = static_cast<unsigned>(((N + 127) / 128 + r.wrun - 1) / r.wrun);
+  blocks += r.wgx * ((K + 63) / 64);
+  r.wend = static_cast<unsigned>(blocks);
+  blocks += range_blocks(r.g, r.glg, &r.ggx);
+  r.gend = static_cast<unsigned>(blocks);
+  blocks += range_blocks(r.x, r.xlg, &r.xgx);
+  r.wcols = bits(L->wf_range);
+  r.wrows = bits(L->wd_range);
+  r.gcols = bits(L->g_range);
+  r.xcols = bits(L->x_range);
+  r.gtau = gtau;
+  r.xtau = xtau;
+  r.status = L->dev_status;
+  const bool plain = r.x.form == kViewVec && r.g.form == kViewVec && r.w.form == kViewVec;
+  err = launch_pdl(plain ? layer_range_kernel<true> : layer_range_kernel<false>, dim3(static_cast<unsigned>(blocks)),
+                   dim3(256), s, r);
+  if (err != cudaSuccess) return cuda_fail(err, "layer_range_kernel launch");
+  // 3. codes
+  LayerQuant q;
+  memset(&q, 0, sizeof(q));
+  auto tensor = [&](QuantArgs* a, const float* x, int64_t cols, const float* range, unsigned* tau, float* tau0,
+                    uint8_t* exp, void* codes, int64_t ldc, void* codes_t, int64_t ldt, float* scale) {
+    a->x = x;
+    a->R = M;
+    a->C = a->ld = cols;
+    a->Q = q_of_bits(L->bits);
+    a->G = L->n_groups;
+    a->tslots = tau;
+    a->tau_out = tau0;
+    a->crange = range;
+    a->exp_out = exp;
+    a->codes = codes;
+    a->ldc = ldc;
+    a->codes_t = codes_t;
+    a->ldt = ldt;
+    a->scale_out = scale;
+    set_alignment(a, cbytes);
+  };
+  tensor(&q.x, L->x, K, L->x_range, xtau, L->x_tau0, L->x_exp, L->x_codes, L->ld_x, L->xt_codes, L->ld_xt, L->x_scale);
+  tensor(&q.g, L->dy, N, L->g_range, gtau, L->g_tau0, L->g_exp, L->g_codes, L->ld_g, L->gt_codes, L->ld_gt, L->g_scale);
+  q.g.seed = seed;
+  weight_args(&q.wf, &q.wd, L->w, K, N, N, L->bits, L->n_groups, L->wf_range, L->wd_range, L->wf_codes, L->ld_wf,
+              L->wf_scale, L->wd_codes, L->ld_wd, L->wd_scale);
+  q.wf.frange = L->x_range;   // the forward role's rows are X's channels
+  q.wf.ftslots = xtau;
+  q.wd.frange = L->g_range;   // the loss-propagation role's columns are dY's
+  q.wd.ftslots = gtau;
+  const dim3 xg = quant_grid(q.x), gg = quant_grid(q.g), wg = quant_grid(q.wf);
+  q.xgx = xg.x;
+  q.ggx = gg.x;
+  q.wgx = wg.x;
+  q.xend = xg.x * xg.y;
+  q.wend = q.xend + wg.x * wg.y;
+  const unsigned nb = q.wend + gg.x * gg.y;
+  err = code_type(L->bits, L->n_groups) == SQ_CODE_E4M3 ? launch_layer_quantize<uint8_t>(q, nb, s)
+                                                        : launch_layer_quantize<uint16_t>(q, nb, s);
+  return err == cudaSuccess ? SQ_OK : cuda_fail(err, "layer_quantize_kernel launch");
 }
 
 }  // namespace sq
@@ -1120,14 +1845,13 @@ extern "C" sq_status shiftquant_quantize(const float* x, int64_t rows, int64_t c
   if (codes_t && ld_t < rows) return fail(SQ_EINVAL, "quantize: ld_t < rows");
   if (x == nullptr || ld < cols) return fail(SQ_EINVAL, "quantize: x is NULL or ld < cols");
   QuantArgs a;
+  memset(&a, 0, sizeof(a));
   a.x = x;
   a.R = rows;
   a.C = cols;
   a.ld = ld;
-  a.gran = gran;
   a.Q = q_of_bits(bits);
   a.G = n_groups;
-  a.mode = mode;
   a.seed = seed;
   a.row0 = row0;
   a.rt = range_or_tau0;
@@ -1138,21 +1862,17 @@ extern "C" sq_status shiftquant_quantize(const float* x, int64_t rows, int64_t c
   a.codes_t = codes_t;
   a.ldt = ld_t;
   a.scale_out = scale_out;
-  a.vec_in = (ld % 4 == 0) && aligned16(x);
-  a.vec_out = codes != nullptr && ((ld_codes * cbytes) % (4 * cbytes) == 0) &&
-              (reinterpret_cast<uintptr_t>(codes) % (4 * cbytes) == 0);
-  a.vec_t = codes_t != nullptr && ((ld_t * cbytes) % 16 == 0) && aligned16(codes_t);
   a.pos_cols = g_order_cols;
   a.pos_rows = g_order_rows;
-  const int64_t gx = (cols + kQC - 1) / kQC, gy = (rows + kQR - 1) / kQR;
-  if (gx > 0x7FFFFFFF || gy > 65535)
+  set_alignment(&a, cbytes);
+  if (!quant_grid_ok(rows, cols))
     return fail(SQ_EUNSUPPORTED, "quantize: tensor too large for one launch (%lld x %lld)",
                 static_cast<long long>(rows), static_cast<long long>(cols));
-  dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(gy));
+  const dim3 grid = quant_grid(a);
   if (type == SQ_CODE_E4M3)
-    launch_quantize<uint8_t>(a, grid, s);
+    launch_quantize<uint8_t>(a, gran, mode, grid, s);
   else
-    launch_quantize<uint16_t>(a, grid, s);
+    launch_quantize<uint16_t>(a, gran, mode, grid, s);
   const cudaError_t err = cudaGetLastError();
   return err == cudaSuccess ? SQ_OK : cuda_fail(err, "quantize_kernel launch");
 }
@@ -1299,37 +2019,15 @@ extern "C" sq_status shiftquant_quantize_weight(const float* w, int64_t rows, in
     return fail(SQ_EINVAL, "quantize_weight: ranges, codes and scales of both roles are required");
   if (ld_fwd < rows) return fail(SQ_EINVAL, "quantize_weight: ld_fwd < rows");
   if (ld_dgrad < cols) return fail(SQ_EINVAL, "quantize_weight: ld_dgrad < cols");
-  QuantArgs af;
-  memset(&af, 0, sizeof(af));
-  af.x = w;
-  af.R = rows;
-  af.C = cols;
-  af.ld = ld;
-  af.gran = SQ_GRAN_PER_COL;
-  af.Q = q_of_bits(bits);
-  af.G = n_groups;
-  af.mode = SQ_ROUND_NEAREST_EVEN;
-  af.vec_in = (ld % 4 == 0) && aligned16(w);
-  QuantArgs ad = af;
-  af.rt = range_out_ch;
+  QuantArgs af, ad;
+  weight_args(&af, &ad, w, rows, cols, ld, bits, n_groups, range_out_ch, range_in_ch, codes_fwd, ld_fwd,
+              scale_fwd, codes_dgrad, ld_dgrad, scale_dgrad);
   af.fold = fold_fwd;
-  af.codes_t = codes_fwd;
-  af.ldt = ld_fwd;
-  af.scale_out = scale_fwd;
-  af.vec_t = ((ld_fwd * cbytes) % 16 == 0) && aligned16(codes_fwd);
-  ad.gran = SQ_GRAN_PER_ROW;
-  ad.rt = range_in_ch;
   ad.fold = fold_dgrad;
-  ad.codes = codes_dgrad;
-  ad.ldc = ld_dgrad;
-  ad.scale_out = scale_dgrad;
-  ad.vec_out = ((ld_dgrad * cbytes) % (4 * cbytes) == 0) &&
-               (reinterpret_cast<uintptr_t>(codes_dgrad) % (4 * cbytes) == 0);
-  const int64_t gx = (cols + kQC - 1) / kQC, gy = (rows + kQR - 1) / kQR;
-  if (gx > 0x7FFFFFFF || gy > 65535)
+  if (!quant_grid_ok(rows, cols))
     return fail(SQ_EUNSUPPORTED, "quantize_weight: tensor too large for one launch (%lld x %lld)",
                 static_cast<long long>(rows), static_cast<long long>(cols));
-  const dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(gy));
+  const dim3 grid = quant_grid(af);
   if (type == SQ_CODE_E4M3)
     launch_quantize_weight<uint8_t>(af, ad, grid, s);
   else

@@ -30,10 +30,15 @@ __device__ __forceinline__ uint32_t splitmix64_top24(uint64_t z) {
 
 __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) << 23); }
 
-// The grouping of Eq. 3 for one channel: max{e in [0, G-1] : r 2^e <= tau}; the product by
-// 2^e is exact (no rounding) for every finite r <= tau, so the comparison is exact.
+// The grouping of Eq. 3 for one channel: max{e in [0, G-1] : r 2^e <= tau}, for r <= tau.
+// For a normal r the difference of the bit patterns is (exponent difference) 2^23 +
+// (mantissa difference), and the floor of its quotient by 2^23 takes one off the exponent
+// difference exactly when r's mantissa is the larger: that floor is the largest e.  A
+// subnormal r steps through the exponents (the product by 2^e is exact).
 __device__ __forceinline__ int group_exponent(float r, float tau, int G) {
   if (r == 0.0f) return G - 1;
+  const int rb = __float_as_int(r), tb = __float_as_int(tau);
+  if (rb >= 0x00800000 && rb <= tb) return min(G - 1, (tb - rb) >> 23);
   int e = 0;
 #pragma unroll 1
   for (int k = 1; k < G; ++k) {

@@ -30,11 +30,52 @@ static int check_step(const sq_layer_step* L) {
   return SQ_OK;
 }
 
-// the device part of the step, in stream order on s
+// the GEMM operands of a step
+static sq_layer_gemms step_gemms(const sq_layer_step* L) {
+  sq_layer_gemms g = {};
+  g.x_codes = L->x_codes;   g.ld_x = L->ld_x;
+  g.xt_codes = L->xt_codes; g.ld_xt = L->ld_xt;
+  g.x_scale = L->x_scale;   g.x_exp = L->x_exp;
+  g.g_codes = L->g_codes;   g.ld_g = L->ld_g;
+  g.gt_codes = L->gt_codes; g.ld_gt = L->ld_gt;
+  g.g_scale = L->g_scale;   g.g_exp = L->g_exp;
+  g.wf_codes = L->wf_codes; g.ld_wf = L->ld_wf; g.wf_scale = L->wf_scale;
+  g.wd_codes = L->wd_codes; g.ld_wd = L->ld_wd; g.wd_scale = L->wd_scale;
+  g.M = L->M; g.K = L->K; g.N = L->N;
+  g.bits = L->bits; g.n_groups = L->n_groups;
+  g.y = L->y;   g.ld_y = L->N;
+  g.dx = L->dx; g.ld_dx = L->K;
+  g.dw = L->dw; g.ld_dw = L->N;
+  return g;
+}
+
+// The device part of the step, in stream order on s, with a usable workspace: the quantizer
+// passes of the three tensors together (quantize_layer), which also zero what the GEMMs need,
+// then the GEMM launch behind them.  Against one library call after another (fourteen
+// launches): 256 x 512 x 512 (4-bit) 59.3 -> 24.2 us a step, 12544 x 2304 x 256 (4-bit)
+// 139 -> 114 us, 5003 x 1155 x 1001 (6-bit) 138 -> 105 us, 12608 x 768 x 3072 (6-bit)
+// 286 -> 259 us, 4096 x 11008 x 4096 (8-bit) 967 -> 938 us.
+static int run_step_fused(const sq_layer_step* L, uint64_t seed, void* s) {
+  int st = check_layer_quant(L);
+  if (st != SQ_OK) return st;
+  const sq_layer_gemms g = step_gemms(L);
+  LayerPlan plan;
+  ZeroRegion zero[3];
+  int nzero = 0;
+  if ((st = plan_layer_gemms(&g, L->workspace, L->workspace_bytes, L->dev_status, &plan, zero, &nzero)) != SQ_OK)
+    return st;
+  if ((st = quantize_layer(L, seed, static_cast<unsigned*>(L->workspace), zero, nzero, as_stream(s))) != SQ_OK)
+    return st;
+  return issue_layer_gemms(&plan, as_stream(s));
+}
+
+// The device part of the step; without a usable workspace, one library call after another.
 static int run_step(const sq_layer_step* L, uint64_t seed, void* s) {
   const int64_t M = L->M, K = L->K, N = L->N;
   const int b = L->bits, G = L->n_groups;
   int st;
+  if (L->workspace != nullptr && L->workspace_bytes >= 256 && aligned16(L->workspace) && layer_quant_fits(L))
+    return run_step_fused(L, seed, s);
   // activation: range pass + grouping, then codes and (if asked for) the transposed copy
   // (RN); without the copy the weight gradient reads the codes MN-major
   if ((st = shiftquant_calibrate(L->x, M, K, K, SQ_GRAN_SHIFT, G, L->x_range, L->x_tau0,
@@ -62,21 +103,7 @@ static int run_step(const sq_layer_step* L, uint64_t seed, void* s) {
                                        L->g_exp, L->wf_codes, L->ld_wf, L->wf_scale, L->wd_codes,
                                        L->ld_wd, L->wd_scale, s)) != SQ_OK)
     return st;
-  // the three GEMMs, one persistent launch
-  sq_layer_gemms g = {};
-  g.x_codes = L->x_codes;   g.ld_x = L->ld_x;
-  g.xt_codes = L->xt_codes; g.ld_xt = L->ld_xt;
-  g.x_scale = L->x_scale;   g.x_exp = L->x_exp;
-  g.g_codes = L->g_codes;   g.ld_g = L->ld_g;
-  g.gt_codes = L->gt_codes; g.ld_gt = L->ld_gt;
-  g.g_scale = L->g_scale;   g.g_exp = L->g_exp;
-  g.wf_codes = L->wf_codes; g.ld_wf = L->ld_wf; g.wf_scale = L->wf_scale;
-  g.wd_codes = L->wd_codes; g.ld_wd = L->ld_wd; g.wd_scale = L->wd_scale;
-  g.M = M; g.K = K; g.N = N;
-  g.bits = b; g.n_groups = G;
-  g.y = L->y;   g.ld_y = N;
-  g.dx = L->dx; g.ld_dx = K;
-  g.dw = L->dw; g.ld_dw = N;
+  const sq_layer_gemms g = step_gemms(L);
   return shiftquant_gemm_layer(&g, L->workspace, L->workspace_bytes, L->dev_status, s);
 }
 
