@@ -581,11 +581,12 @@ struct BwdChan {
   float t, u, mg, mgx, zs, dg, db;
 };
 
-__device__ __forceinline__ BwdChan bwd_chan_of(const L1bnArgs& a, int64_t c, float gscale, float Rf) {
+// (t: the step of dy's codes)
+__device__ __forceinline__ BwdChan bwd_chan_sums(const L1bnArgs& a, int64_t c, float t, float Rf) {
   const int64_t C = a.C;
   const float* ch = a.ch;
   BwdChan k;
-  k.t = __fmul_rn(gscale, pow2f(-static_cast<int>(__ldcg(a.ge + c))));
+  k.t = t;
   const float sq = ch[kChSq * C + c], s = ch[kChS * C + c];
   const float P = __ll2float_rn(stat_sum(a.st, kStP, C, c));
   k.u = sq > 0.0f ? __fdiv_rn(ch[kChGq * C + c], sq) : 0.0f;
@@ -596,6 +597,10 @@ __device__ __forceinline__ BwdChan bwd_chan_of(const L1bnArgs& a, int64_t c, flo
   k.zs = __fdiv_rn(__ll2float_rn(stat_sum(a.st, kStZ, C, c)), Rf);
   k.db = __fmul_rn(P, k.t);
   return k;
+}
+
+__device__ __forceinline__ BwdChan bwd_chan_of(const L1bnArgs& a, int64_t c, float gscale, float Rf) {
+  return bwd_chan_sums(a, c, __fmul_rn(gscale, pow2f(-static_cast<int>(__ldcg(a.ge + c)))), Rf);
 }
 
 // channel c's backward constants into the state (for the output pass), dgamma and dbeta
@@ -952,6 +957,540 @@ __global__ void __launch_bounds__(kL1Threads, 2) l1bn_bwd_coop_kernel(const L1bn
   bwd_out_pass<false>(a, g.lgo, bo, sc);
 }
 
+// ----------------------------------------------------------------- resident form
+// For tensors whose codes fit the SMs' shared memory (up to about 200 KB a block) a call is one
+// cooperative launch of at most one 1024-thread block per SM, each owning a tile of tc columns
+// by a slab of rows for the whole call.  What the other forms write to and read back from
+// global memory between their passes stays with the block: the codes always, and x (dy) itself
+// where it fits as binary32 (FP32), so that it is read from HBM once.  Otherwise it streams
+// through a ring of kResRing rows a thread, copied asynchronously; the quantizer phase walks
+// the rows backwards, so that it starts with those the ring still holds and finds the next
+// ones in L2.  A block that owns all rows of its columns (gy == 1) also needs no other block
+// for its channel sums, and the grid barriers shrink to those of the per-tensor maxima: tau_0,
+// and sigma's in the forward.  Channel sums, constants, codes and exponents are left in the
+// state as by the other forms, and every step is the same operation on the same values, so
+// results are the same bit for bit.
+// Bound by instruction issue on top of its traffic: about 55 instructions an element in the
+// forward and 89 in the backward (two 64-bit multiplies of the generator among them), on one
+// block per SM whose phases wait at 2-4 grid barriers of about 1.5 us.  Forward and backward
+// together, 8-bit, the cooperative form (or, above 1024 channels, the chain) before and this
+// form now: [200704, 64] 129 and 109 us (ring), [3136, 2048] 115 and 80 us (whole).
+constexpr int kResThreads = 1024;
+constexpr int kResWarps = kResThreads / 32;
+constexpr int kResRing = 6;   // 96 KB a block in flight or resident
+constexpr size_t kResDyn = 232448 - 8192;   // dynamic shared memory of a block, less room for its static part
+
+struct ResGeom {
+  int lgq;        // log2(quads across the tile): tc = 4 << lgq
+  int gx, gy;     // tiles across the channels, row slabs
+  int64_t rows;   // rows of a slab
+  int per;        // rows of a thread, at most
+  int G;
+  int* status;
+};
+
+// Dynamic shared memory: the quads of x (every row of a thread, or the ring), the codes (in
+// place of x's quads, or 4 bytes a quad), the output table (forward), the reductions' words.
+struct ResSmem {
+  size_t codes, lut, red, total;
+};
+__host__ __device__ inline ResSmem res_smem(bool fwd, bool fp32, int lgq, int64_t rows, int per) {
+  const size_t tc = size_t(4) << lgq, row = kResThreads * size_t(16);
+  ResSmem m;
+  m.codes = fp32 ? 0 : kResRing * row;
+  m.lut = fp32 ? ((static_cast<size_t>(rows) << lgq) * 16 + 127) & ~size_t(127) : m.codes + static_cast<size_t>(per) * kResThreads * 4;
+  m.red = m.lut + (fwd ? tc * kLutStride * sizeof(float) : 0);
+  m.total = m.red + (kResWarps * (tc + 1) + tc) * sizeof(int);
+  return m;
+}
+
+// The thread's place: its quad, its rows r0 + k rpp (k < n), its slots in shared memory (x's
+// quad of row k, k mod kResRing in the ring; the codes of row k).
+struct ResPos {
+  int quad, n;
+  int64_t c, r0, rpp;
+  uint32_t slot, code, cstep;
+};
+constexpr uint32_t kResStep = kResThreads * 16;
+
+template <bool FP32>
+__device__ __forceinline__ ResPos res_pos(const ResGeom& g, int64_t R, uint32_t data, size_t codes) {
+  ResPos p;
+  const int tq = 1 << g.lgq, tid = threadIdx.x;
+  p.quad = tid & (tq - 1);
+  p.rpp = kResThreads >> g.lgq;
+  const int bx = blockIdx.x % g.gx, by = blockIdx.x / g.gx;
+  p.c = static_cast<int64_t>(bx) * (4 << g.lgq) + 4 * p.quad;
+  p.r0 = by * g.rows + (tid >> g.lgq);
+  const int64_t r1 = min(R, (by + int64_t(1)) * g.rows);
+  p.n = p.r0 < r1 ? static_cast<int>((r1 - p.r0 + p.rpp - 1) / p.rpp) : 0;
+  p.slot = data + tid * 16;
+  p.code = FP32 ? p.slot : data + static_cast<uint32_t>(codes) + tid * 4;
+  p.cstep = FP32 ? kResStep : kResThreads * 4;
+  return p;
+}
+
+// Sums (or maxima) of a block's columns: v[j] of every thread, over the threads of its quad;
+// the result of tile column `tid` for tid < tc.
+template <bool MAX, typename T>
+__device__ __forceinline__ T res_reduce(const T (&v)[4], const ResGeom& g, const ResPos& p, T* red) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tq = 1 << g.lgq, tc = 4 << g.lgq;
+  T* tot = red + kResWarps * (tc + 1);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    T x = v[j];
+    for (int o = 16; o >= tq; o >>= 1) {
+      const T y = __shfl_xor_sync(0xFFFFFFFFu, x, o);
+      x = MAX ? max(x, y) : x + y;
+    }
+    if (lane < tq) red[warp * (tc + 1) + 4 * p.quad + j] = x;   // (tq <= 16: lane < tq is quad `lane`)
+  }
+  __syncthreads();
+  for (int c = warp; c < tc; c += kResWarps) {   // a warp per column, a lane per warp's value
+    const T x = red[lane * (tc + 1) + c];
+    const T t = MAX ? __reduce_max_sync(0xFFFFFFFFu, x) : __reduce_add_sync(0xFFFFFFFFu, x);
+    if (lane == 0) tot[c] = t;
+  }
+  __syncthreads();
+  return threadIdx.x < tc ? tot[threadIdx.x] : T(0);   // (the next reduction's first barrier frees tot)
+}
+
+// Starts the copy of a row's quad at src to its slot.  v16: aligned and inside the tensor.
+__device__ __forceinline__ void res_copy(const L1bnArgs& a, const ResPos& p, const float* src, bool v16, uint32_t slot) {
+  if (v16) {
+    cp_async_16(slot, src, true);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) cp_async_4(slot + 4 * j, p.c + j < a.C ? src + j : a.in, p.c + j < a.C);
+  }
+}
+
+// Four codes to p (a quad of codes, packed): one word where the rows of codes are aligned.
+__device__ __forceinline__ void res_store_codes(int8_t* p, uint32_t w, const L1bnArgs& a, int64_t c, bool word) {
+  if (word) {
+    *reinterpret_cast<uint32_t*>(p) = w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (c + j < a.C) p[j] = static_cast<int8_t>(w >> (8 * j));
+  }
+}
+
+// The copies of the range phase: every row (FP32), or the thread's last kResRing rows.
+template <bool FP32>
+__device__ __forceinline__ void res_start(const L1bnArgs& a, const ResGeom& g, const ResPos& p) {
+  const bool v16 = a.vec_in && p.c + 3 < a.C;
+  const int64_t sx = p.rpp * a.ld_in;
+  int k = FP32 ? 0 : max(p.n - kResRing, 0);
+  const float* src = a.in + (p.r0 + k * p.rpp) * a.ld_in + p.c;
+#pragma unroll 2
+  for (; k < p.n; ++k, src += sx) res_copy(a, p, src, v16, p.slot + (FP32 ? k : k % kResRing) * kResStep);
+  cp_async_commit();
+}
+
+// The range phase: the column maxima sent to the range slots.
+template <bool FP32>
+__device__ __forceinline__ void res_range(const L1bnArgs& a, const ResGeom& g, const ResPos& p, unsigned* slots,
+                                          unsigned* red) {
+  unsigned m[4] = {0u, 0u, 0u, 0u};
+  const int held = FP32 ? p.n : min(p.n, kResRing);   // rows in shared memory: the last ones
+  if (!FP32 && p.c < a.C) {
+    constexpr int U = 8;
+    const int n = p.n - held;
+    const int64_t sx = p.rpp * a.ld_in;
+    const float* src = a.in + p.r0 * a.ld_in + p.c;
+    for (int k = 0; k < n; k += U, src += U * sx) {
+      float v[U][4];
+#pragma unroll
+      for (int u = 0; u < U; ++u)   // rows past the end re-read the first of these
+        load4(src + (k + u < n ? u * sx : 0), p.c, a.C, a.vec_in, v[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) m[j] = max(m[j], __float_as_uint(v[u][j]) & 0x7FFFFFFFu);
+    }
+  }
+  cp_async_wait_all();   // (each thread reads its own copies only)
+  uint32_t slot = p.slot;   // in any order: a ring's slots 0 .. held - 1 hold the held rows
+  for (int k = 0; k < held; ++k, slot += kResStep) {
+    const float4 v = ld_shared_v4_f32(slot);
+    m[0] = max(m[0], __float_as_uint(v.x) & 0x7FFFFFFFu);
+    m[1] = max(m[1], __float_as_uint(v.y) & 0x7FFFFFFFu);
+    m[2] = max(m[2], __float_as_uint(v.z) & 0x7FFFFFFFu);
+    m[3] = max(m[3], __float_as_uint(v.w) & 0x7FFFFFFFu);
+  }
+  const unsigned w = res_reduce<true, unsigned>(m, g, p, red);
+  const int64_t c = static_cast<int64_t>(blockIdx.x % g.gx) * (4 << g.lgq) + threadIdx.x;
+  if (threadIdx.x < (4 << g.lgq) && c < a.C) {
+    if (w != 0u) atomicMax(slots + (blockIdx.x / g.gx % kSpread) * a.C + c, w);
+    if (w >= 0x7F800000u) atomicOr(g.status, kDevNonFinite);
+  }
+}
+
+// tau_0, and the exponents of the block's columns into sexp (and, with the ranges, from the
+// blocks of the first slab into the state).
+__device__ __forceinline__ float res_group(const L1bnArgs& a, const ResGeom& g, const unsigned* slots, float* range_out,
+                                           float* tau_out, uint8_t* exp_out, uint8_t* sexp, uint32_t* red) {
+  unsigned m = 0;
+  for (int64_t c = threadIdx.x; c < a.C; c += kResThreads) m = max(m, slot_range(slots, a.C, c));
+  const unsigned tb = block_max(m, red);
+  const float tau = __uint_as_float(tb);
+  const bool nonfinite = tb >= 0x7F800000u;
+  const int64_t c = static_cast<int64_t>(blockIdx.x % g.gx) * (4 << g.lgq) + threadIdx.x;
+  if (threadIdx.x < (4 << g.lgq)) {
+    int e = 0;
+    if (c < a.C) {
+      const unsigned r = slot_range(slots, a.C, c);
+      e = nonfinite ? 0 : group_exponent(__uint_as_float(r), tau, g.G);
+      if (blockIdx.x < static_cast<unsigned>(g.gx)) {
+        range_out[c] = __uint_as_float(r);
+        exp_out[c] = static_cast<uint8_t>(e);
+      }
+    }
+    sexp[threadIdx.x] = static_cast<uint8_t>(e);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *tau_out = tau;
+  __syncthreads();
+  return tau;
+}
+
+__device__ __forceinline__ uint32_t pack_codes4(const int (&q)[4]) {
+  return __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
+}
+
+// The code of one element, as shift_code gives it for an element of a tensor with a finite
+// tau_0 (where |v| <= Q (1 + 2^-23)): v + 1.5 2^23 has spacing 1, so its bit pattern less that
+// of 1.5 2^23 is v rounded -- to nearest even, or down for the stochastic draw of generator
+// state z.
+__device__ __forceinline__ int res_code_rn(float v) {
+  return __float_as_int(__fadd_rn(v, 12582912.0f)) - 0x4B400000;
+}
+__device__ __forceinline__ int res_code_sr(float v, uint64_t z, int Q) {
+  const float t = __fadd_rd(v, 12582912.0f);
+  const float frac = __fsub_rn(v, __fadd_rn(t, -12582912.0f));
+  const float u = __fmul_rn(static_cast<float>(splitmix64_top24(z)), 5.9604644775390625e-08f);   // * 2^-24, exact
+  const int q = __float_as_int(t) - 0x4B400000 + (u < frac ? 1 : 0);
+  return min(max(q, -Q), Q);
+}
+
+template <bool FP32>
+__global__ void __launch_bounds__(kResThreads, 1) l1bn_fwd_res_kernel(const L1bnArgs a, const ResGeom g) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ uint8_t sexp[kL1MaxCols];
+  __shared__ uint32_t redm[32];
+  __shared__ int smean[kL1MaxCols];
+  __shared__ float cs[kL1MaxCols], cm[kL1MaxCols], csq[kL1MaxCols], cgq[kL1MaxCols], cbq[kL1MaxCols];
+  const int tc = 4 << g.lgq, tid = threadIdx.x;
+  const ResSmem sm = res_smem(true, FP32, g.lgq, g.rows, g.per);
+  float* lut = reinterpret_cast<float*>(dyn + sm.lut);
+  int* red = reinterpret_cast<int*>(dyn + sm.red);
+  const ResPos p = res_pos<FP32>(g, a.R, smem_u32(dyn), sm.codes);
+  unsigned* ctr = a.sync;
+  unsigned* smax_bits = a.sync + 1;   // the largest sigma (bit pattern), where the blocks share it so
+  unsigned* slots = a.sync + 64;
+  const unsigned nb = gridDim.x;
+  unsigned target = nb;
+  const int64_t c_own = static_cast<int64_t>(blockIdx.x % g.gx) * tc + tid;   // column of thread tid < tc
+  const bool own = tid < tc && c_own < a.C;
+  const bool lead = blockIdx.x < static_cast<unsigned>(g.gx);                 // a block of the first slab
+  const int64_t slab = blockIdx.x / g.gx;
+  // 1. range; the sums the later phases add into start at zero
+  res_start<FP32>(a, g, p);
+  zero_sums(a.st, 3 * kSpread * a.C);   // kStS1, kStS, kStZ
+  uint32_t mg = 0, mb = 0;
+  for (int64_t c = tid; c < a.C; c += kResThreads) {
+    mg = max(mg, __float_as_uint(a.gamma[c]) & 0x7FFFFFFFu);
+    mb = max(mb, __float_as_uint(a.beta[c]) & 0x7FFFFFFFu);
+  }
+  const float gmax = __uint_as_float(block_max(mg, redm));
+  const float bmax = __uint_as_float(block_max(mb, redm));
+  res_range<FP32>(a, g, p, slots, reinterpret_cast<unsigned*>(red));
+  if (!grid_barrier(ctr, target, g.status)) return;
+  // 2. tau_0, exponents; codes and their sums
+  const float tau = res_group(a, g, slots, a.ch + kChXRange * a.C, a.scal + kScXTau, a.xe, sexp, redm);
+  const float Qf = static_cast<float>(a.Q), invS = __fdiv_rn(Qf, tau);
+  const bool zero = !(tau > 0.0f) || !isfinite(tau) || !isfinite(invS);
+  const float scale = zero ? 0.0f : __fdiv_rn(tau, Qf), mulS = zero ? 0.0f : invS;
+  if (blockIdx.x == 0 && tid == 0) a.scal[kScXScale] = scale;
+  {
+    float pe[4];
+    int acc[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) pe[j] = pow2f(sexp[4 * p.quad + j]);
+    const int64_t sq = p.rpp * a.C, sx = p.rpp * a.ld_in;
+    const bool v16 = a.vec_in && p.c + 3 < a.C, word = (a.C & 3) == 0 && p.c < a.C;
+    int8_t* pq = a.xq + (p.r0 + (p.n - 1) * p.rpp) * a.C + p.c;
+    const float* src = a.in + (p.r0 + (p.n - 1 - kResRing) * p.rpp) * a.ld_in + p.c;   // a ring ahead
+    uint32_t code = p.code + (p.n - 1) * p.cstep;
+    uint32_t slot = p.slot + (p.n - 1) % kResRing * kResStep;
+    for (int k = p.n - 1; k >= 0; --k) {
+      if (!FP32) cp_async_wait<kResRing - 1>();
+      const float4 v = ld_shared_v4_f32(FP32 ? code : slot);
+      float x[4] = {v.x, v.y, v.z, v.w};   // (0 past C)
+      if (zero) x[0] = x[1] = x[2] = x[3] = 0.0f;
+      int q[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        q[j] = res_code_rn(__fmul_rn(__fmul_rn(x[j], pe[j]), mulS));
+        acc[j] += q[j];
+      }
+      const uint32_t w = pack_codes4(q);
+      st_shared_u32(code, w);
+      res_store_codes(pq, w, a, p.c, word);
+      if (!FP32) {
+        if (k >= kResRing) res_copy(a, p, src, v16, slot);
+        cp_async_commit();
+        src -= sx;
+        slot = slot == p.slot ? p.slot + (kResRing - 1) * kResStep : slot - kResStep;
+      }
+      code -= p.cstep;
+      pq -= sq;
+    }
+    const int t = res_reduce<false, int>(acc, g, p, red);
+    if (own) atomicAdd(reinterpret_cast<unsigned long long*>(stat_slot(a.st, kStS1, a.C, slab) + c_own),
+                       static_cast<unsigned long long>(static_cast<long long>(t)));
+  }
+  if (g.gy > 1 && !grid_barrier(ctr, target += nb, g.status)) return;
+  // 3. means and deviation sums (with one slab the thread's own atomics are the whole sum)
+  if (tid < tc) smean[tid] = own ? static_cast<int>(rne_div(stat_sum(a.st, kStS1, a.C, c_own), a.R)) : 0;
+  __syncthreads();
+  {
+    // Four codes at a time, biased to unsigned bytes b = q + 128 (and the means likewise).  The
+    // sums stay within 16-bit halves over a thread's rows (at most 64): |q - m| <= 255 a byte;
+    // for the signs, bit 8 of 256 + q - m is set where q >= m, and of 255 + q - m where q > m, and
+    // sum sign = #(q > m) + #(q >= m) - rows.
+    uint32_t mw = 0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mw |= (static_cast<uint32_t>(smean[4 * p.quad + j] + 128) & 0xFFu) << (8 * j);
+    const uint32_t lo = 0x00FF00FFu, bit = 0x01000100u;
+    const uint32_t oe = bit - (mw & lo), oo = bit - ((mw >> 8) & lo);   // 256 - mean, even and odd columns
+    uint32_t ae = 0u, ao = 0u, ge = 0u, go = 0u;
+    uint32_t code = p.code;
+#pragma unroll 4
+    for (int k = 0; k < p.n; ++k, code += p.cstep) {
+      const uint32_t w = ld_shared_u32(code) ^ 0x80808080u;
+      const uint32_t d = __vabsdiffu4(w, mw);
+      ae += d & lo;
+      ao += (d >> 8) & lo;
+      const uint32_t e = (w & lo) + oe, o = ((w >> 8) & lo) + oo;
+      ge += (e & bit) + ((e - 0x00010001u) & bit);
+      go += (o & bit) + ((o - 0x00010001u) & bit);
+    }
+    const unsigned sabs[4] = {ae & 0xFFFFu, ao & 0xFFFFu, ae >> 16, ao >> 16};
+    const int ssgn[4] = {static_cast<int>((ge & 0xFFFFu) >> 8) - p.n, static_cast<int>((go & 0xFFFFu) >> 8) - p.n,
+                         static_cast<int>(ge >> 24) - p.n, static_cast<int>(go >> 24) - p.n};
+    const unsigned ts = res_reduce<false, unsigned>(sabs, g, p, reinterpret_cast<unsigned*>(red));
+    const int tz = res_reduce<false, int>(ssgn, g, p, red);
+    if (own) {
+      atomicAdd(reinterpret_cast<unsigned long long*>(stat_slot(a.st, kStS, a.C, slab) + c_own),
+                static_cast<unsigned long long>(ts));
+      atomicAdd(reinterpret_cast<unsigned long long*>(stat_slot(a.st, kStZ, a.C, slab) + c_own),
+                static_cast<unsigned long long>(static_cast<long long>(tz)));
+    }
+  }
+  if (g.gy > 1 && !grid_barrier(ctr, target += nb, g.status)) return;
+  // 4. sigma's per-tensor maximum: over all channels by every block, or -- one slab, whose
+  // sums other blocks have not waited for, and many channels -- shared through one word
+  const float Rf = __ll2float_rn(a.R);
+  FwdChan f = {0.0f, 0.0f, 0.0f};
+  if (own) {
+    f.s = __fmul_rn(scale, pow2f(-static_cast<int>(sexp[tid])));
+    f.m = static_cast<float>(smean[tid]);
+    f.sig = __fmul_rn(__fdiv_rn(__ll2float_rn(stat_sum(a.st, kStS, a.C, c_own)), Rf), f.s);
+  }
+  float smax;
+  if (g.gy == 1 || a.C > kResThreads) {
+    const unsigned b = __float_as_uint(f.sig) & 0x7FFFFFFFu;
+    if (own && lead && b != 0u) atomicMax(smax_bits, b);
+    if (!grid_barrier(ctr, target += nb, g.status)) return;
+    smax = __uint_as_float(__ldcg(smax_bits));
+  } else {
+    uint32_t ms = 0;
+    if (tid < a.C) {
+      const float s_c = __fmul_rn(scale, pow2f(-static_cast<int>(__ldcg(a.xe + tid))));
+      const float sig = __fmul_rn(__fdiv_rn(__ll2float_rn(stat_sum(a.st, kStS, a.C, tid)), Rf), s_c);
+      ms = __float_as_uint(sig) & 0x7FFFFFFFu;
+    }
+    smax = __uint_as_float(block_max(ms, redm));
+  }
+  // 5. the block's channel constants and output tables
+  if (tid < tc) {
+    const float sq = own ? quant8(f.sig, smax) : 0.0f;
+    const float gq = own ? quant8(a.gamma[c_own], gmax) : 0.0f, bq = own ? quant8(a.beta[c_own], bmax) : 0.0f;
+    cs[tid] = f.s;
+    cm[tid] = f.m;
+    csq[tid] = sq;
+    cgq[tid] = gq;
+    cbq[tid] = bq;
+    if (own && lead) {
+      const int64_t C = a.C;
+      a.ch[kChS * C + c_own] = f.s;
+      a.ch[kChM * C + c_own] = f.m;
+      a.ch[kChSig * C + c_own] = f.sig;
+      a.ch[kChSq * C + c_own] = sq;
+      a.ch[kChGq * C + c_own] = gq;
+      a.ch[kChBq * C + c_own] = bq;
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < tc * kLutStride; i += kResThreads) {
+    const int c = i / kLutStride;
+    lut[i] = l1bn_out_of(i % kLutStride - 127, cs[c], cm[c], csq[c], cgq[c], cbq[c]);
+  }
+  __syncthreads();
+  // 6. output
+  if (p.c < a.C) {
+    const int col0 = 4 * p.quad * kLutStride + 127;
+    uint32_t code = p.code;
+    float* py = a.out + p.r0 * a.ld_out + p.c;
+    const int64_t sy = p.rpp * a.ld_out;
+#pragma unroll 4
+    for (int k = 0; k < p.n; ++k, code += p.cstep, py += sy) {
+      const uint32_t w = ld_shared_u32(code);
+      float y[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) y[j] = lut[col0 + j * kLutStride + code_at(w, j)];
+      store4(py, p.c, a.C, a.vec_out, y);
+    }
+  }
+}
+
+template <bool FP32>
+__global__ void __launch_bounds__(kResThreads, 1) l1bn_bwd_res_kernel(const L1bnArgs a, const ResGeom g) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ uint8_t sexp[kL1MaxCols];
+  __shared__ uint32_t redm[32];
+  __shared__ BwdChan sc[kL1MaxCols];
+  const int tc = 4 << g.lgq, tid = threadIdx.x;
+  const ResSmem sm = res_smem(false, FP32, g.lgq, g.rows, g.per);
+  int* red = reinterpret_cast<int*>(dyn + sm.red);
+  const ResPos p = res_pos<FP32>(g, a.R, smem_u32(dyn), sm.codes);
+  unsigned* ctr = a.sync;
+  unsigned* slots = a.sync + 64;
+  const unsigned nb = gridDim.x;
+  const int64_t c_own = static_cast<int64_t>(blockIdx.x % g.gx) * tc + tid;
+  const bool own = tid < tc && c_own < a.C;
+  const int64_t slab = blockIdx.x / g.gx;
+  // 1. range of dy
+  res_start<FP32>(a, g, p);
+  zero_sums(a.st + kStP * kSpread * a.C, 2 * kSpread * a.C);   // kStP, kStD
+  res_range<FP32>(a, g, p, slots, reinterpret_cast<unsigned*>(red));
+  if (!grid_barrier(ctr, nb, g.status)) return;
+  // 2. its codes p (stochastic rounding), and the sums of p and p (q - m)
+  const float tau = res_group(a, g, slots, a.ch + kChGRange * a.C, a.scal + kScGTau, a.ge, sexp, redm);
+  const float Qf = static_cast<float>(a.Q), invS = __fdiv_rn(Qf, tau);
+  const bool zero = !(tau > 0.0f) || !isfinite(tau) || !isfinite(invS);
+  const float gscale = zero ? 0.0f : __fdiv_rn(tau, Qf), mulS = zero ? 0.0f : invS;
+  if (blockIdx.x == 0 && tid == 0) a.scal[kScGScale] = gscale;
+  int m[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (p.c + j < a.C) m[j] = static_cast<int>(a.ch[kChM * a.C + p.c + j]);
+  {
+    float pe[4];
+    int accp[4] = {0, 0, 0, 0}, accd[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) pe[j] = pow2f(sexp[4 * p.quad + j]);
+    const int64_t sq = p.rpp * a.C, sx = p.rpp * a.ld_in;
+    const bool v16 = a.vec_in && p.c + 3 < a.C, word = (a.C & 3) == 0 && p.c < a.C;
+    const int64_t last = (p.r0 + (p.n - 1) * p.rpp) * a.C + p.c;   // element of the thread's last row
+    const int8_t* px = a.xq + last;
+    int8_t* pp = a.gq + last;
+    const float* src = a.in + (p.r0 + (p.n - 1 - kResRing) * p.rpp) * a.ld_in + p.c;   // a ring ahead
+    // generator state of the quad's first element: seed + (r C + c + 1) gamma
+    uint64_t z = a.seed + (static_cast<uint64_t>(last) + 1ull) * kSplitMixGamma;
+    const uint64_t zstep = static_cast<uint64_t>(sq) * kSplitMixGamma;
+    uint32_t code = p.code + (p.n - 1) * p.cstep;
+    uint32_t slot = p.slot + (p.n - 1) % kResRing * kResStep;
+    uint32_t qx = p.n > 0 && p.c < a.C ? load_codes_w(px, p.c, a.C) : 0u;   // x's codes, a row ahead
+    for (int k = p.n - 1; k >= 0; --k) {
+      px -= sq;
+      const uint32_t qn = k > 0 && p.c < a.C ? load_codes_w(px, p.c, a.C) : 0u;
+      if (!FP32) cp_async_wait<kResRing - 1>();
+      const float4 v = ld_shared_v4_f32(FP32 ? code : slot);
+      float x[4] = {v.x, v.y, v.z, v.w};   // (0 past C, and 0 has the code 0 whatever the draw)
+      if (zero) x[0] = x[1] = x[2] = x[3] = 0.0f;
+      int pc[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float xs = __fmul_rn(__fmul_rn(x[j], pe[j]), mulS);
+        pc[j] = res_code_sr(xs, z + static_cast<uint64_t>(j) * kSplitMixGamma, a.Q);
+        accp[j] += pc[j];
+        accd[j] += pc[j] * code_at(qx, j);
+      }
+      const uint32_t w = pack_codes4(pc);
+      st_shared_u32(code, w);
+      res_store_codes(pp, w, a, p.c, word);
+      if (!FP32) {
+        if (k >= kResRing) res_copy(a, p, src, v16, slot);
+        cp_async_commit();
+        src -= sx;
+        slot = slot == p.slot ? p.slot + (kResRing - 1) * kResStep : slot - kResStep;
+      }
+      code -= p.cstep;
+      pp -= sq;
+      z -= zstep;
+      qx = qn;
+    }
+    // sum p (q - m) = sum p q - m sum p
+#pragma unroll
+    for (int j = 0; j < 4; ++j) accd[j] -= m[j] * accp[j];
+    const int tp = res_reduce<false, int>(accp, g, p, red), td = res_reduce<false, int>(accd, g, p, red);
+    if (own) {
+      atomicAdd(reinterpret_cast<unsigned long long*>(stat_slot(a.st, kStP, a.C, slab) + c_own),
+                static_cast<unsigned long long>(static_cast<long long>(tp)));
+      atomicAdd(reinterpret_cast<unsigned long long*>(stat_slot(a.st, kStD, a.C, slab) + c_own),
+                static_cast<unsigned long long>(static_cast<long long>(td)));
+    }
+  }
+  if (g.gy > 1 && !grid_barrier(ctr, 2 * nb, g.status)) return;
+  // 3. channel constants (with one slab the thread's own atomics are the whole sums), dx
+  if (own) {
+    BwdChan k = bwd_chan_sums(a, c_own, __fmul_rn(gscale, pow2f(-static_cast<int>(sexp[tid]))), __ll2float_rn(a.R));
+    sc[tid] = k;
+    if (blockIdx.x < static_cast<unsigned>(g.gx)) put_bwd_chan(a, c_own, k);
+  }
+  __syncthreads();
+  if (p.c < a.C) {
+    float tt[4], mgc[4], u4[4], k3[4][3];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const BwdChan& v = sc[p.c + j < a.C ? 4 * p.quad + j : 4 * p.quad];
+      tt[j] = v.t;
+      mgc[j] = v.mg;
+      u4[j] = v.u;
+#pragma unroll
+      for (int sgn = -1; sgn <= 1; ++sgn) k3[j][sgn + 1] = __fmul_rn(v.mgx, __fsub_rn(static_cast<float>(sgn), v.zs));
+    }
+    uint32_t code = p.code;
+    float* pd = a.out + p.r0 * a.ld_out + p.c;
+    const int8_t* px = a.xq + p.r0 * a.C + p.c;
+    const int64_t sd = p.rpp * a.ld_out, sq = p.rpp * a.C;
+    constexpr int U = 4;   // x's codes come from L2, U rows at a time
+    for (int k = 0; k < p.n; k += U) {
+      uint32_t qx[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u, px += sq) qx[u] = k + u < p.n ? load_codes_w(px, p.c, a.C) : 0u;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (k + u >= p.n) break;
+        const uint32_t w = ld_shared_u32(code);
+        float dx[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int d = code_at(qx[u], j) - m[j];
+          const float gr = __fmul_rn(static_cast<float>(code_at(w, j)), tt[j]);
+          const float kj = d > 0 ? k3[j][2] : (d < 0 ? k3[j][0] : k3[j][1]);
+          dx[j] = __fmul_rn(u4[j], __fsub_rn(__fsub_rn(gr, mgc[j]), kj));
+        }
+        store4(pd, p.c, a.C, a.vec_out, dx);
+        code += p.cstep;
+        pd += sd;
+      }
+    }
+  }
+}
+
 // Self-test of the grid barrier's expiry path: block 0 never arrives, so every block's
 // bounded wait runs out (about 1 s), records SQ_DEV_TIMEOUT and returns.
 __global__ void __launch_bounds__(kL1Threads) l1bn_selftest_barrier_kernel(unsigned* ctr, int* status) {
@@ -1123,6 +1662,85 @@ static int launch_coop(const L1bnArgs& a, int G, int blocks, int32_t* dev_status
   return err == cudaSuccess ? SQ_OK : cuda_fail(err, FWD ? "l1bn_fwd_coop_kernel launch" : "l1bn_bwd_coop_kernel launch");
 }
 
+// The resident form's geometry for [R, C] on the current device: of the tile widths 64, 32 and
+// 16 (or the channel count rounded up to a power of two, if that is less) the one whose blocks
+// have the least to do -- the elements of a block, 1.4 times where x (dy) is read twice --
+// and the wider of two alike, whose rows are longer.  False where the codes do not fit, or the
+// device runs no cooperative launches.
+template <bool FWD>
+static bool res_plan(int64_t R, int64_t C, ResGeom* g, bool* fp32) {
+  static int cached[64];   // [device]: SMs + 1, 0 = not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  if (cached[dev] == 0) {
+    int coop = 0, sms = 0, smem = 0;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    bool ok = coop && sms > 0 && smem >= 232448;
+    const void* kernels[4] = {reinterpret_cast<const void*>(l1bn_fwd_res_kernel<false>),
+                              reinterpret_cast<const void*>(l1bn_fwd_res_kernel<true>),
+                              reinterpret_cast<const void*>(l1bn_bwd_res_kernel<false>),
+                              reinterpret_cast<const void*>(l1bn_bwd_res_kernel<true>)};
+    for (const void* k : kernels)
+      ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kResDyn)) == cudaSuccess;
+    cudaGetLastError();
+    cached[dev] = ok ? sms + 1 : 1;
+  }
+  const int sms = cached[dev] - 1;
+  double best = 0.0;
+  const int widest = tile_lg(C) < 4 ? tile_lg(C) : 4;
+  for (int lgq = widest; lgq >= (widest < 2 ? widest : 2); --lgq) {
+    const int64_t tc = int64_t(4) << lgq, gx = (C + tc - 1) / tc;
+    if (gx > sms) continue;
+    int64_t gy = sms / gx;
+    const int64_t rpp = kResThreads >> lgq, most = (R + rpp - 1) / rpp;   // a row per thread at least
+    if (gy > most) gy = most;
+    const int64_t rows = (R + gy - 1) / gy;
+    if (rows > (int64_t(1) << 20)) continue;
+    gy = (R + rows - 1) / rows;
+    const int64_t per = (rows + rpp - 1) / rpp;
+    if (per > 64) continue;
+    const bool full = res_smem(FWD, true, lgq, rows, static_cast<int>(per)).total <= kResDyn;
+    if (!full && res_smem(FWD, false, lgq, rows, static_cast<int>(per)).total > kResDyn) continue;
+    const double cost = static_cast<double>(rows) * tc * (full ? 1.0 : 1.4);
+    if (best != 0.0 && cost >= 0.98 * best) continue;
+    best = cost;
+    g->lgq = lgq;
+    g->gx = static_cast<int>(gx);
+    g->gy = static_cast<int>(gy);
+    g->rows = rows;
+    g->per = static_cast<int>(per);
+    *fp32 = full;
+  }
+  return best != 0.0;
+}
+
+// The resident form of a call: the barrier counter and range slots zeroed, one cooperative
+// launch.
+template <bool FWD>
+static int launch_res(const L1bnArgs& a, int G, ResGeom g, bool fp32, int32_t* dev_status, cudaStream_t s) {
+  cudaError_t err = cudaMemsetAsync(a.sync, 0, 256 + kSpread * static_cast<size_t>(a.C) * sizeof(unsigned), s);
+  if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync (l1bn sync)");
+  g.G = G;
+  g.status = dev_status;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(static_cast<unsigned>(g.gx * g.gy));
+  cfg.blockDim = dim3(kResThreads);
+  cfg.dynamicSmemBytes = res_smem(FWD, fp32, g.lgq, g.rows, g.per).total;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  err = cudaLaunchKernelEx(&cfg, FWD ? (fp32 ? l1bn_fwd_res_kernel<true> : l1bn_fwd_res_kernel<false>)
+                                     : (fp32 ? l1bn_bwd_res_kernel<true> : l1bn_bwd_res_kernel<false>), a, g);
+  if (err == cudaSuccess) err = cudaGetLastError();
+  return err == cudaSuccess ? SQ_OK : cuda_fail(err, FWD ? "l1bn_fwd_res_kernel launch" : "l1bn_bwd_res_kernel launch");
+}
+
 // the single-launch form serves this call: few enough channels for every block to form
 // the per-tensor maxima over all of them, and a device that runs cooperative launches
 // with at least one block per output column tile
@@ -1199,6 +1817,9 @@ extern "C" sq_status shiftquant_l1bn_forward(const float* x, int64_t rows, int64
   a.beta = beta;
   a.vec_in = (ld_x % 4 == 0) && aligned16(x);
   a.vec_out = (ld_y % 4 == 0) && aligned16(y);
+  ResGeom g;
+  bool fp32 = false;
+  if (res_plan<true>(rows, channels, &g, &fp32)) return launch_res<true>(a, n_groups, g, fp32, dev_status, s);
   if (const int blocks = coop_use<true>(channels)) return launch_coop<true>(a, n_groups, blocks, dev_status, s);
   // the channel sums start at zero (a kernel, not a memset, so that the launches after the
   // range pass stay a chain of kernels, each launched behind the one before)
@@ -1254,6 +1875,9 @@ extern "C" sq_status shiftquant_l1bn_backward(const float* dy, int64_t rows, int
   a.dbeta = dbeta;
   a.vec_in = (ld_dy % 4 == 0) && aligned16(dy);
   a.vec_out = (ld_dx % 4 == 0) && aligned16(dx);
+  ResGeom g;
+  bool fp32 = false;
+  if (res_plan<false>(rows, channels, &g, &fp32)) return launch_res<false>(a, n_groups, g, fp32, dev_status, s);
   if (const int blocks = coop_use<false>(channels)) return launch_coop<false>(a, n_groups, blocks, dev_status, s);
   const int64_t nz = 2 * kSpread * channels;
   l1bn_zero_kernel<<<static_cast<unsigned>((nz + 255) / 256 < 1024 ? (nz + 255) / 256 : 1024), 256, 0, s>>>(
