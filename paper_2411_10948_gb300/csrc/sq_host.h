@@ -64,4 +64,24 @@ int plan_layer_gemms(const sq_layer_gemms* args, void* workspace, size_t workspa
                      LayerPlan* plan, ZeroRegion* zero, int* nzero);
 int issue_layer_gemms(const LayerPlan* plan, cudaStream_t s);
 
+// Launch with programmatic stream serialization: the kernel may begin launching while the
+// preceding kernel of the stream finishes, and waits for it (griddep_wait) before reading
+// anything.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t s,
+                              Args... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = 0;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 }  // namespace sq

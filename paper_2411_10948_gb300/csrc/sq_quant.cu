@@ -1068,26 +1068,6 @@ __global__ void __launch_bounds__(kQuantThreads, 4) quantize_kernel(const QuantA
   if (a.beside) griddep_wait();
 }
 
-// Launch with programmatic stream serialization: the kernel may begin launching while the
-// preceding kernel of the stream finishes, and waits for it (griddep_wait) before reading
-// anything.
-template <typename... Params, typename... Args>
-static cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t s,
-                              Args... args) {
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <typename CodeT, int FORM, int GRAN, bool FOLD>
 static void launch_mode(const QuantArgs& a, int mode, dim3 grid, cudaStream_t s) {
   if (mode == SQ_ROUND_NEAREST_EVEN)
