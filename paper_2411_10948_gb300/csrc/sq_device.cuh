@@ -330,13 +330,6 @@ __device__ __forceinline__ CodeT ld_shared_code(uint32_t addr) {
   return static_cast<CodeT>(v);
 }
 
-// one 32-byte sector: dst 32-byte aligned
-__device__ __forceinline__ void st_global_v8(float* dst, const float (&v)[8]) {
-  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]),
-               "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
-               : "memory");
-}
-
 // ------------------------------------------------------------------- tcgen05
 // Every tcgen05 instruction of a kernel uses one CTA-group size kCg: 1 (a CTA's own
 // tiles) or 2 (a CTA pair's 256-row tiles).  With kCg = 2, allocation and release are

@@ -29,7 +29,7 @@
 //               tile, ahead of the epilogue
 //   warps 4-11  epilogue: tcgen05.ld, int32 accumulation across chunks, dequantizing
 //               multiply, TMA stores of 32 x 32 boxes (or int32 TMA reductions into a
-//               split-K workspace; direct 32-byte stores on pair tiles; plain stores where
+//               split-K workspace; plain stores where
 //               the output rows are not 16-byte aligned)
 // Work units reach the roles through a small shared-memory ring that the producer of the
 // CTA (a pair's leader) fills: with a scheduling counter it takes each next unit from it
@@ -107,7 +107,6 @@ struct GemmParams {
   int mode;  // 0: per-column scale (forward, loss propagation); 1: row/column shifts (wgrad)
   int G;
   int vec_y;  // output rows 16-byte aligned: 16-byte stores
-  int vec_y32;  // ... 32-byte aligned
   const float* a_scale;
   const float* b_scale;
   const uint8_t* row_exp;
@@ -208,54 +207,93 @@ __device__ __noinline__ void write_acc_box(long long* acc, int64_t ld_acc, int64
   }
 }
 
+// One 32 x 32 output box of an epilogue warp (see emit_box) of a GEMM whose outputs are fp32
+// values and nothing else: T's integers `vals` times the column factors at `fac`, times the
+// row's factor first where kRow, staged and sent by a TMA store.
+template <bool kRow>
+__device__ __forceinline__ void emit_plain(const uint32_t (&vals)[32], bool as_float, uint32_t fac, float rfac,
+                                           const CUtensorMap* tma_y, uint32_t buf, int32_t row0, int32_t col0,
+                                           int lane) {
+  const uint32_t line = buf + lane * 128 + ((lane & 7) << 4);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float4 f4 = ld_shared_v4_f32(fac + k * 16);
+    const float f[4] = {f4.x, f4.y, f4.z, f4.w};
+    uint32_t o[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const uint32_t a = vals[k * 4 + e];
+      const float val = as_float ? __uint_as_float(a) : __int2float_rn(static_cast<int32_t>(a));
+      o[e] = __float_as_uint(__fmul_rn(kRow ? __fmul_rn(val, rfac) : val, f[e]));
+    }
+    st_shared_v4(line ^ (k << 4), o[0], o[1], o[2], o[3]);
+  }
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) {
+    tma_store_2d(tma_y, buf, col0, row0);
+    bulk_commit();
+  }
+}
+
+// The box of a split of K: T's integers are added into the int32 workspace by a TMA reduction.
+__device__ __forceinline__ void emit_sums(const uint32_t (&vals)[32], bool as_float, const CUtensorMap* tma_ws,
+                                          uint32_t buf, int32_t row0, int32_t col0, int lane) {
+  const uint32_t line = buf + lane * 128 + ((lane & 7) << 4);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    uint32_t o[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      o[e] = as_float ? static_cast<uint32_t>(__float2int_rn(__uint_as_float(vals[k * 4 + e]))) : vals[k * 4 + e];
+    st_shared_v4(line ^ (k << 4), o[0], o[1], o[2], o[3]);
+  }
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) {
+    tma_reduce_add_2d(tma_ws, buf, col0, row0);
+    bulk_commit();
+  }
+}
+
 // One 32 x 32 output box of an epilogue warp: lane = row, vals = the lane's 32 columns as
 // exact integers (FP32 patterns when `as_float`, else int32); fac = shared-memory address
 // of the box's 32 column factors (16-byte aligned), rfac the row's factor (weight gradient
 // only: the forward and loss-propagation outputs take the column factor alone).  The box is staged in shared
-// memory (128-byte swizzle) and leaves either as dequantized fp32 values through
-// row-contiguous 16-byte stores (eight lanes per 128-byte row, four rows per instruction),
-// as int32 partial sums through a TMA reduce-add into the split-K workspace, or -- past the
+// memory (128-byte swizzle) and leaves either as dequantized fp32 values (a TMA store, or a
+// lane a column where rows are not 16-byte aligned), as int32 partial sums through a TMA reduce-add into the split-K workspace, or -- past the
 // int32 range -- as int64 additions (64-bit atomics, a row of 32 columns per instruction)
 // into the int64 workspace.  The exactness-check integers are written when asked.
-// kDirect (pair tiles): a plain fp32 box whose rows are 32-byte aligned skips the staging --
-// each lane stores its row's 32 columns as four 32-byte sectors.  In a pair the tensor core
-// takes most of the shared-memory bandwidth, and a box's staging writes, its TMA reads and
-// the wait for them cost the MMAs more than the sector-wise stores cost L2: layer launches
-// of 12608 x 768 x 3072 (6-bit) 165.4 -> 155.7 us, 4096 x 11008 x 4096 (8-bit) 715 -> 703 us,
-// 16384 x 4096 x 11008 (6-bit) 2139 -> 2125 us.  Single tiles keep the staged TMA stores:
-// their launches are bound by the output stream, which full 128-byte lines serve better
-// (12544 x 2304 x 256, 4-bit: 57.9 us staged, 64.6 us direct; every second box direct 62.1).
-template <bool kDirect>
+// Two warps per scheduler drain a tile, so a box costs its instructions and their latency:
+// the two usual ways out (emit_plain, emit_sums) are straight-line code of their own, without
+// a test of the way out per element.  Layer launches with the tests inside / with pairs
+// storing 32-byte sectors from registers / so: 12544 x 2304 x 256 (4-bit) 52.3 / - / 46.8 us,
+// 12608 x 768 x 3072 (6-bit) 165 / 155 / 143 us, 4096 x 11008 x 4096 (8-bit) 715 / 700 / 674 us.
+// (The rarer ways out as functions shared with these cost the kernels with several chunks a unit
+// registers: 149, 698 us.)
 __device__ __forceinline__ void emit_box(const GemmParams& p, const CUtensorMap* tma_y,
                                          const CUtensorMap* tma_ws, const uint32_t (&vals)[32],
                                          bool as_float, uint32_t fac, float rfac, uint32_t buf,
                                          int64_t row0, int64_t col0, int lane) {
   const bool tma_out = p.ws != nullptr ? !p.wide : p.vec_y != 0;
-  if (kDirect && p.vec_y32 && p.ws == nullptr && p.acc == nullptr && p.colmax == nullptr &&
-      col0 + kOutBox <= p.N) {
-    float* dst = p.y + (row0 + lane) * p.ldy + col0;
-    const bool in = row0 + lane < p.M;
-#pragma unroll
-    for (int k = 0; k < kOutBox / 8; ++k) {
-      const float4 fa = ld_shared_v4_f32(fac + k * 32), fb = ld_shared_v4_f32(fac + k * 32 + 16);
-      const float f[8] = {fa.x, fa.y, fa.z, fa.w, fb.x, fb.y, fb.z, fb.w};
-      float o[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const uint32_t a = vals[k * 8 + e];
-        const float val = as_float ? __uint_as_float(a) : __int2float_rn(static_cast<int32_t>(a));
-        o[e] = __fmul_rn(p.mode == 1 ? __fmul_rn(val, rfac) : val, f[e]);
-      }
-      if (in) st_global_v8(dst + k * 8, o);
-    }
-    return;
-  }
   if (lane == 0) {
     // the last TMA store has read the box (it may belong to another GEMM of the launch,
     // whatever this box's own way out)
     bulk_wait_read<0>();
   }
   __syncwarp();
+  const int32_t r32 = static_cast<int32_t>(row0), c32 = static_cast<int32_t>(col0);
+  if (p.ws == nullptr && p.acc == nullptr && p.colmax == nullptr && tma_out) {
+    if (p.mode == 1)
+      emit_plain<true>(vals, as_float, fac, rfac, tma_y, buf, r32, c32, lane);
+    else
+      emit_plain<false>(vals, as_float, fac, rfac, tma_y, buf, r32, c32, lane);
+    return;
+  }
+  if (p.ws != nullptr && !p.wide) {
+    emit_sums(vals, as_float, tma_ws, buf, r32, c32, lane);
+    return;
+  }
   if (p.acc != nullptr && p.ws == nullptr) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -345,37 +383,20 @@ __device__ __forceinline__ void emit_box(const GemmParams& p, const CUtensorMap*
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) {
-      if (p.ws != nullptr)
-        tma_reduce_add_2d(tma_ws, buf, static_cast<int32_t>(col0), static_cast<int32_t>(row0));
-      else
-        tma_store_2d(tma_y, buf, static_cast<int32_t>(col0), static_cast<int32_t>(row0));
+      tma_store_2d(tma_y, buf, c32, r32);
       bulk_commit();
     }
     return;
   }
+  // rows that start anywhere: a lane a column, so that each store is one run of 128 bytes
+  // (5003 x 1155 x 1001, 6-bit: the launch 67 us with four columns a lane, 52 us so)
   __syncwarp();
-  const int lr = lane >> 3;         // row within a group of four
-  const int lc = lane & 7;          // 16-byte chunk within the 128-byte row
-  const int64_t col = col0 + lc * 4;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int rr = i * 4 + lr;
-    const int64_t row = row0 + rr;
-    uint32_t v0, v1, v2, v3;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v0), "=r"(v1), "=r"(v2), "=r"(v3)
-                 : "r"(buf + rr * 128 + ((lc ^ (rr & 7)) << 4)));
-    if (row < p.M) {
-      float* dst = p.y + row * p.ldy + col;
-      if (p.vec_y && col + 3 < p.N) {
-        *reinterpret_cast<uint4*>(dst) = make_uint4(v0, v1, v2, v3);
-      } else {
-        if (col + 0 < p.N) dst[0] = __uint_as_float(v0);
-        if (col + 1 < p.N) dst[1] = __uint_as_float(v1);
-        if (col + 2 < p.N) dst[2] = __uint_as_float(v2);
-        if (col + 3 < p.N) dst[3] = __uint_as_float(v3);
-      }
-    }
+  const int64_t col = col0 + lane;
+  const int rows = p.M - row0 < 32 ? static_cast<int>(p.M - row0) : 32;
+  float* dst = p.y + row0 * p.ldy + col;
+  if (col < p.N) {
+#pragma unroll 8
+    for (int rr = 0; rr < rows; ++rr, dst += p.ldy) *dst = __uint_as_float(staged(buf, rr, lane));
   }
   __syncwarp();  // the staging box is free for the next one
 }
@@ -1040,7 +1061,7 @@ __global__ void __launch_bounds__(kThreads, 1) shiftmm_kernel(const __grid_const
           const int64_t col0 = n0 + h * 128 + s * 32;
           if (row0 >= p.M || col0 >= p.N) continue;  // warp-uniform: nothing of this box exists
           const uint32_t buf = stage_out0;
-          emit_box<kPair>(p, tma_y, tma_ws, v, true, smem_u32(fac + h * 128 + s * 32), rfac, buf, row0,
+          emit_box(p, tma_y, tma_ws, v, true, smem_u32(fac + h * 128 + s * 32), rfac, buf, row0,
                            col0, lane);
         }
         __syncwarp();
@@ -1113,7 +1134,7 @@ __global__ void __launch_bounds__(kThreads, 1) shiftmm_kernel(const __grid_const
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[i] = acc[s * 32 + i];
           const uint32_t buf = stage_out0;
-          emit_box<kPair>(p, tma_y, tma_ws, v, false, smem_u32(fac + h * 128 + s * 32), rfac, buf, row0,
+          emit_box(p, tma_y, tma_ws, v, false, smem_u32(fac + h * 128 + s * 32), rfac, buf, row0,
                            col0, lane);
         }
         __syncwarp();
@@ -1613,7 +1634,6 @@ static int prepare_job(const GemmJob& j, const Plan* pl, int bits, int G, int32_
   p.mode = j.which == 2 ? 1 : 0;
   p.G = G;
   p.vec_y = (j.ldy % 4 == 0) && aligned16(j.y);
-  p.vec_y32 = (j.ldy % 8 == 0) && (reinterpret_cast<uintptr_t>(j.y) & 31u) == 0;
   p.a_scale = j.a_scale;
   p.b_scale = j.b_scale;
   p.row_exp = j.row_exp;
