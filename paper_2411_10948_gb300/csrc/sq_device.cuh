@@ -27,24 +27,41 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   return t;
 }
 
-// 16-byte streaming load (read-only path, no L1 allocation, 256-byte L2 prefetch).  The
-// asm is volatile so a run of these stays in program order: all of them are issued before
-// the first result is used, whatever register budget the compiler aims for.
+// 16-byte streaming load (no L1 allocation, 256-byte L2 prefetch).  The asm is volatile so a
+// run of these stays in program order: all of them are issued before the first result is used,
+// whatever register budget the compiler aims for.  Not through the read-only path: a kernel
+// launched behind the one that writes its input (griddep_wait) is resident while the input
+// changes, and that path is for data that stays as it is as long as the kernel runs.
 __device__ __forceinline__ float4 ld_stream_v4(const float* p) {
   float4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.f32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.L2::256B.v4.f32 {%0, %1, %2, %3}, [%4];"
                : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                : "l"(p));
   return v;
 }
 
-// the same load as a pure function of the address (no volatile): the compiler may batch
-// a run of them ahead of their uses, keeping all of them in flight together
-__device__ __forceinline__ float4 ld_nc_v4(const float* p) {
-  float4 v;
-  asm("ld.global.nc.L1::no_allocate.L2::256B.v4.f32 {%0, %1, %2, %3}, [%4];"
-      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-      : "l"(p));
+// One value by a coherent load (through L1, as a plain load), issued where it stands: volatile,
+// so that the compiler neither sinks it to its use nor moves it across a griddep_wait.  With
+// plain loads, a 5003 x 1155 x 1001 layer step (6-bit) took 5 us more; past
+// L1 (__ldcg), a 12544 x 2304 x 256 step (4-bit) 6 us, and [100352, 147] codes 5 us more.
+__device__ __forceinline__ float ld_here(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int ld_here(const int* p) {
+  int v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int ld_here(const uint8_t* p) {
+  int v;
+  asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_here(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
 
@@ -70,7 +87,11 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 // ----------------------------------------------------- programmatic dependent launch
 // Wait until the preceding kernel of the stream has completed and its writes are visible
-// (a no-op for a kernel launched without programmatic stream serialization).
+// (a no-op for a kernel launched without programmatic stream serialization).  What a preceding
+// kernel may write is read by coherent loads after the wait (ld_here, __ldcg, __ldcs, plain loads
+// through unrestricted pointers, TMA), never through the read-only path (__ldg, or const __restrict__
+// pointers, which the compiler reads through it): that path may return what this kernel's or an
+// earlier kernel's blocks on the SM fetched before the data was written.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Let the next kernel of the stream (if launched with programmatic stream serialization)
 // start its launch; it still waits for this grid's completion before reading its results.

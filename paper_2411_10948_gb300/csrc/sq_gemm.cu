@@ -166,20 +166,20 @@ __device__ __forceinline__ void epilogue_value(const GemmParams& p, int64_t row,
                                                long long* out_t) {
   if (p.mode == 0) {
     // Y = T * (s_A 2^-(G-1) * s_B[col]);  T already carries the shifts
-    const float f = __fmul_rn(a_fac, __ldg(p.b_scale + col));
+    const float f = __fmul_rn(a_fac, ld_here(p.b_scale + col));
     *out_y = __fmul_rn(__int2float_rn(t), f);
     *out_t = t;
   } else {
     // dW = T_raw * 2^-(eX + eY) * (s_X s_dY);  canonical T = T_raw << (2(G-1) - eX - eY)
-    const int er = __ldg(p.row_exp + row), ec = __ldg(p.col_exp + col);
+    const int er = ld_here(p.row_exp + row), ec = ld_here(p.col_exp + col);
     *out_y = __fmul_rn(__fmul_rn(__int2float_rn(t), pow2_neg(er + ec)), a_fac);
     *out_t = static_cast<long long>(t) << (2 * (p.G - 1) - er - ec);
   }
 }
 
 __device__ __forceinline__ float epilogue_a_factor(const GemmParams& p) {
-  return p.mode == 0 ? __fmul_rn(__ldg(p.a_scale), pow2_neg(p.G - 1))
-                     : __fmul_rn(__ldg(p.a_scale), __ldg(p.b_scale));
+  return p.mode == 0 ? __fmul_rn(ld_here(p.a_scale), pow2_neg(p.G - 1))
+                     : __fmul_rn(ld_here(p.a_scale), ld_here(p.b_scale));
 }
 
 // value of box element (rr, cc) in a staging buffer written with 128-byte swizzle
@@ -198,12 +198,12 @@ __device__ __noinline__ void write_acc_box(long long* acc, int64_t ld_acc, int64
                                            uint32_t buf, int64_t row0, int64_t col0, int lane) {
   const int64_t col = col0 + lane;
   if (col >= N) return;
-  const int ec = col_exp ? __ldg(col_exp + col) : 0;
+  const int ec = col_exp ? ld_here(col_exp + col) : 0;
   for (int rr = 0; rr < 32; ++rr) {
     const int64_t row = row0 + rr;
     if (row >= M) break;
     const long long t = static_cast<int32_t>(staged(buf, rr, lane));
-    acc[row * ld_acc + col] = row_exp ? t << (2 * (G - 1) - __ldg(row_exp + row) - ec) : t;
+    acc[row * ld_acc + col] = row_exp ? t << (2 * (G - 1) - ld_here(row_exp + row) - ec) : t;
   }
 }
 
@@ -543,8 +543,8 @@ __device__ __noinline__ void factor_warp(const GemmBatch& bt, uint64_t* ufull,
       const int64_t col = n0 + lane + 32 * j;
       f[j] = 0.0f;
       if (col < p.N)
-        f[j] = p.mode == 0 ? __fmul_rn(a_fac, __ldg(p.b_scale + col))
-                           : __fmul_rn(a_fac, pow2_neg(__ldg(p.col_exp + col)));
+        f[j] = p.mode == 0 ? __fmul_rn(a_fac, ld_here(p.b_scale + col))
+                           : __fmul_rn(a_fac, pow2_neg(ld_here(p.col_exp + col)));
     }
     // table it & 1 last held unit it - 2: wait until the epilogue is done with it
     if (it >= 2 &&
@@ -602,11 +602,11 @@ __device__ __noinline__ void plan_chunks(const GemmBatch& bt, volatile int* out,
           uint32_t wd[4] = {0u, 0u, 0u, 0u};
           if (sg < nseg) {
             if (vec && c + 16 <= p.K) {
-              const uint4 v = __ldg(reinterpret_cast<const uint4*>(k_exp + c));
+              const uint4 v = ld_here(reinterpret_cast<const uint4*>(k_exp + c));
               wd[0] = v.x; wd[1] = v.y; wd[2] = v.z; wd[3] = v.w;
             } else {
               for (int i = 0; i < 16 && c + i < p.K; ++i)
-                wd[i >> 2] |= static_cast<uint32_t>(__ldg(k_exp + c + i)) << (8 * (i & 3));
+                wd[i >> 2] |= static_cast<uint32_t>(ld_here(k_exp + c + i)) << (8 * (i & 3));
             }
           }
           unsigned w = 0;
@@ -991,7 +991,7 @@ __global__ void __launch_bounds__(kThreads, 1) shiftmm_kernel(const __grid_const
       volatile int* segkb = reinterpret_cast<volatile int*>(smem + L::seg_offset);
       for (int g = 0; g < bt.count; ++g)
         if (bt.seg[g] != nullptr && lane <= bt.p[g].G)
-          segkb[g * kSegSlots + lane] = __ldg(bt.seg[g] + lane) / kBKElems;
+          segkb[g * kSegSlots + lane] = ld_here(bt.seg[g] + lane) / kBKElems;
       __syncwarp();
       if (lane == 0) mbar_arrive(chunkbar);
     }
@@ -1037,7 +1037,7 @@ __global__ void __launch_bounds__(kThreads, 1) shiftmm_kernel(const __grid_const
       const int64_t row0 = m0 + q * 32;
       const int64_t row = row0 + lane;
       const bool row_ok = row < p.M;
-      const float rfac = pow2_neg((p.mode == 1 && row_ok) ? __ldg(p.row_exp + row) : 0);
+      const float rfac = pow2_neg((p.mode == 1 && row_ok) ? ld_here(p.row_exp + row) : 0);
       if constexpr (!kMulti) {
         // one exact chunk: each TMEM value is already the integer T (as FP32)
         const uint32_t b = c & 1u, tph = (c >> 1) & 1u;
@@ -1215,10 +1215,10 @@ __global__ void __launch_bounds__(256) splitk_finalize_wide_kernel(const GemmPar
     float y;
     long long tc;
     if (p.mode == 0) {
-      y = __fmul_rn(__ll2float_rn(t), __fmul_rn(a_fac, __ldg(p.b_scale + col)));
+      y = __fmul_rn(__ll2float_rn(t), __fmul_rn(a_fac, ld_here(p.b_scale + col)));
       tc = t;
     } else {
-      const int er = __ldg(p.row_exp + row), ec = __ldg(p.col_exp + col);
+      const int er = ld_here(p.row_exp + row), ec = ld_here(p.col_exp + col);
       y = __fmul_rn(__fmul_rn(__ll2float_rn(t), pow2_neg(er + ec)), a_fac);
       tc = t << (2 * (p.G - 1) - er - ec);
     }

@@ -164,8 +164,9 @@ __device__ __forceinline__ void load4(const float* p, int64_t c, int64_t C, bool
 }
 
 // the four codes of a quad at p packed in one word, byte j = column c + j (zeros past C).
-// COH: codes written earlier in the same launch (the single-launch form): coherent loads
-// through L2, not the read-only path, which holds only data no part of the launch writes.
+// COH: codes written earlier in the same launch (the single-launch form) or by a kernel this one
+// is launched behind (the chain): coherent loads through L2, not the read-only path, which holds
+// only data nothing writes while the launch runs.
 template <bool COH = false>
 __device__ __forceinline__ uint32_t load_codes_w(const int8_t* p, int64_t c, int64_t C) {
   if ((C & 3) == 0)
@@ -303,7 +304,6 @@ __global__ void __launch_bounds__(kL1Threads, 3) l1bn_fwd_quant_kernel(const L1b
 
 // Forward pass 2: over the codes, sum |q - m| and sum sign(q - m) per channel, with
 // m = round-half-even(sum q / R).  mean: shared scratch for the block's columns.
-template <bool COH>
 __device__ __forceinline__ void fwd_dev_pass(const L1bnArgs& a, int lg, const Blk& b, RedSmem<2>& sm,
                                              int* mean) {
   const TilePos t = tile_pos(lg, b);
@@ -338,7 +338,7 @@ __device__ __forceinline__ void fwd_dev_pass(const L1bnArgs& a, int lg, const Bl
     for (; w.r < a.R; w.r += U * w.S, pq += U * sq) {
       uint32_t q[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) q[u] = w.r + u * w.S < a.R ? load_codes_w<COH>(pq + u * sq, t.c, a.C) : 0u;
+      for (int u = 0; u < U; ++u) q[u] = w.r + u * w.S < a.R ? load_codes_w<true>(pq + u * sq, t.c, a.C) : 0u;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (w.r + u * w.S >= a.R) break;
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(kL1Threads, 3) l1bn_fwd_dev_kernel(const L1bnA
   griddep_launch_dependents();
   __shared__ RedSmem<2> sm;
   __shared__ int mean[kL1MaxCols];
-  fwd_dev_pass<false>(a, lg, launch_blk(), sm, mean);
+  fwd_dev_pass(a, lg, launch_blk(), sm, mean);
 }
 
 // max over the block of non-negative values given as bit patterns
@@ -474,7 +474,6 @@ __global__ void __launch_bounds__(256) l1bn_zero_kernel(long long* __restrict__ 
 
 // Forward pass 4: y = gamma^q ((x^q - mu^q) / sigma^q) + beta^q, looked up per code from
 // lut, the block's columns' tables in shared memory.
-template <bool COH>
 __device__ __forceinline__ void fwd_out_pass(const L1bnArgs& a, int lg, const Blk& b, const float* lut) {
   const TilePos t = tile_pos(lg, b);
   const int64_t C = a.C;
@@ -488,7 +487,7 @@ __device__ __forceinline__ void fwd_out_pass(const L1bnArgs& a, int lg, const Bl
   for (; w.r < a.R; w.r += U * w.S, pq += U * sq, py += U * sy) {
     uint32_t q[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) q[u] = w.r + u * w.S < a.R ? load_codes_w<COH>(pq + u * sq, t.c, C) : 0u;
+    for (int u = 0; u < U; ++u) q[u] = w.r + u * w.S < a.R ? load_codes_w<true>(pq + u * sq, t.c, C) : 0u;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (w.r + u * w.S >= a.R) break;
@@ -509,7 +508,7 @@ __global__ void __launch_bounds__(kL1Threads, 3) l1bn_fwd_out_kernel(const L1bnA
   for (int i = threadIdx.x; i < ncol * kLutStride; i += kL1Threads)
     lut[i] = a.lut[cbase * kLutStride + i];
   __syncthreads();
-  fwd_out_pass<false>(a, lg, launch_blk(), lut);
+  fwd_out_pass(a, lg, launch_blk(), lut);
 }
 
 // Backward pass 1: dy -> int8 ShiftQuant codes p (stochastic rounding of element r C + c),
@@ -674,8 +673,8 @@ __device__ __forceinline__ void bwd_out_pass(const L1bnArgs& a, int lg, const Bl
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const bool in = w.r + u * w.S < a.R;
-      q[u] = in ? load_codes_w<!FROM_STATE>(pq + u * sc, t.c, C) : 0u;
-      p[u] = in ? load_codes_w<!FROM_STATE>(pp + u * sc, t.c, C) : 0u;
+      q[u] = in ? load_codes_w<true>(pq + u * sc, t.c, C) : 0u;
+      p[u] = in ? load_codes_w<true>(pp + u * sc, t.c, C) : 0u;
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -873,7 +872,7 @@ __global__ void __launch_bounds__(kL1Threads, 3) l1bn_fwd_coop_kernel(const L1bn
   }
   if (!grid_barrier(ctr, 2 * nb, g.status)) return;
   // 3. deviation sums
-  if (red_on) fwd_dev_pass<true>(a, g.lg, b, sm2, mean);
+  if (red_on) fwd_dev_pass(a, g.lg, b, sm2, mean);
   if (!grid_barrier(ctr, 3 * nb, g.status)) return;
   // 4. per-tensor maxima of sigma, |gamma|, |beta| over all channels
   const float Rf = __ll2float_rn(a.R);
@@ -919,7 +918,7 @@ __global__ void __launch_bounds__(kL1Threads, 3) l1bn_fwd_coop_kernel(const L1bn
   float* lut = reinterpret_cast<float*>(dyn);
   for (int i = threadIdx.x; i < ncol * kLutStride; i += kL1Threads) lut[i] = __ldcg(a.lut + cbase * kLutStride + i);
   __syncthreads();
-  fwd_out_pass<true>(a, g.lgo, bo, lut);
+  fwd_out_pass(a, g.lgo, bo, lut);
 }
 
 // The backward as one launch: range pass of dy -> its tau_0, exponents, codes and the sums

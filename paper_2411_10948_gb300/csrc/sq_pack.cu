@@ -166,9 +166,9 @@ __device__ __forceinline__ uint2 pack_chunk(const CodeChunk<CodeT>& ch, bool& ba
 // codes of chunk blockDim.x bx + x of the kPackRowsInFlight rows y, y + blockDim.y, ... of
 // slab by, all loaded before the first is packed.
 template <typename CodeT>
-__global__ void __launch_bounds__(256) pack4_kernel(const CodeT* __restrict__ codes, int64_t R,
-                                                    int64_t C, int64_t ld, uint8_t* __restrict__ out,
-                                                    int64_t ldp, int vec, int* __restrict__ status) {
+__global__ void __launch_bounds__(256) pack4_kernel(const CodeT* codes, int64_t R,
+                                                    int64_t C, int64_t ld, uint8_t* out, int64_t ldp,
+                                                    int vec, int* status) {
   constexpr int U = kPackRowsInFlight;
   const int64_t c0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * kPackCodes;
   if (c0 >= C) return;
@@ -201,8 +201,8 @@ __global__ void __launch_bounds__(256) pack4_kernel(const CodeT* __restrict__ co
 }
 
 template <typename CodeT>
-__global__ void __launch_bounds__(256) unpack4_kernel(const uint8_t* __restrict__ in, int64_t ldp,
-                                                      int64_t R, int64_t C, CodeT* __restrict__ codes,
+__global__ void __launch_bounds__(256) unpack4_kernel(const uint8_t* in, int64_t ldp,
+                                                      int64_t R, int64_t C, CodeT* codes,
                                                       int64_t ld, int vec) {
   constexpr int U = kPackRowsInFlight;
   const int64_t c0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * kPackCodes;

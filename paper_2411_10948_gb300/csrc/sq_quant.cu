@@ -77,7 +77,7 @@ constexpr int kGroupLargeThreads = 1024;
 
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS)
-    group_kernel(const unsigned* __restrict__ range_bits, int64_t C, int G,
+    group_kernel(const unsigned* range_bits, int64_t C, int G,
                  float* __restrict__ tau0_out, uint8_t* __restrict__ exp_out,
                  int* __restrict__ status) {
   __shared__ unsigned wmax[THREADS / 32];
@@ -139,6 +139,8 @@ struct RangeView {
 // passes of 1024 / tc rows from r0 on: four columns -- quad qc, or in strided views columns
 // qc + k 2^lg -- of rows r0 + u rpp, with all eight 16-byte loads in flight together.
 // ROWS: rm[u] becomes the maximum with row u's four values.
+// (x is complete before the kernel ahead of a range pass lets it launch, so single elements may
+// come through the read-only path.)
 template <bool ROWS, int FORM>
 __device__ __forceinline__ void tile_maxima(const RangeView& t, int lg, int64_t cb, int64_t r0, int qc,
                                             unsigned (&m)[4], unsigned (&rm)[8]) {
@@ -512,7 +514,7 @@ __device__ __forceinline__ float channel_inv(float rg, float Qf, bool* zero) {
 
 // the folded shift of inner channel i of the other operand, as a factor
 __device__ __forceinline__ float fold_factor(const QuantArgs& a, float ftau, int64_t i) {
-  const int e = a.fold != nullptr ? static_cast<int>(__ldg(a.fold + i))
+  const int e = a.fold != nullptr ? ld_here(a.fold + i)
                                   : channel_exponent(__ldcg(a.frange + i), ftau, a.G);
   return pow2f(a.G - 1 - e);
 }
@@ -547,7 +549,7 @@ __device__ __forceinline__ ColumnValues column_values(const QuantArgs& a, const 
                                                       float ftau, int64_t c, float Qf, bool write) {
   ColumnValues v = {1.0f, 1.0f, 1.0f, false};
   if (GRAN == SQ_GRAN_SHIFT) {
-    const int e = a.exp != nullptr ? static_cast<int>(__ldg(a.exp + c))
+    const int e = a.exp != nullptr ? ld_here(a.exp + c)
                                    : channel_exponent(__ldcg(a.crange + c), ts.tau, a.G);
     if (write && a.exp_out != nullptr) a.exp_out[c] = static_cast<uint8_t>(e);
     v.scale = pow2f(e);
@@ -700,7 +702,7 @@ __device__ __forceinline__ void store_transposed(const QuantArgs& a, uint32_t ti
     if (r >= a.R) return;
     int lc = threadIdx.x >> lr;
     const int ncol = static_cast<int>(min(a.C - c0, int64_t(4) << lg));
-    CodeT* d = static_cast<CodeT*>(a.codes_t) + (c0 + lc) * a.ldt + __ldg(a.pos_rows + r);
+    CodeT* d = static_cast<CodeT*>(a.codes_t) + (c0 + lc) * a.ldt + ld_here(a.pos_rows + r);
 #pragma unroll 4
     for (; lc < ncol; lc += step) {
       *d = ld_shared_code<CodeT>(chunk_addr<CodeT>(tile_smem, lg, lc, rr >> 3) + (rr & 7) * static_cast<int>(sizeof(CodeT)));
@@ -970,7 +972,7 @@ __device__ __forceinline__ void quantize_registers(const QuantArgs& a, const Qua
     int at[4];
 #pragma unroll
     for (int g = 0; g < 4; ++g)
-      if (g < groups) at[g] = __ldg(a.pos_cols + cb + 32 * g);
+      if (g < groups) at[g] = ld_here(a.pos_cols + cb + 32 * g);
     const int nrows = static_cast<int>(min(a.R - rb, int64_t(64 >> (a.lg - 2))));
     // (column 32 g + lane of the warp's row r)
     uint32_t from = warp_smem + (lane >> 2) * 16 + (lane & 3) * static_cast<int>(sizeof(CodeT));
@@ -1003,7 +1005,7 @@ __device__ __forceinline__ void quantize_rows(const QuantArgs& a, const QuadStat
 #pragma unroll
   for (int j = 0; j < 4; ++j)
     if (a.codes != nullptr && !wide && t.p.c + j < a.C)
-      at[j] = a.pos_cols != nullptr ? __ldg(a.pos_cols + t.p.c + j) : t.p.c + j;
+      at[j] = a.pos_cols != nullptr ? ld_here(a.pos_cols + t.p.c + j) : t.p.c + j;
   CodeT* dst = static_cast<CodeT*>(a.codes) + t.p.r * a.ldc + (wide ? t.p.c : 0);
 #pragma unroll 1
   for (int i = 0; i < 8; ++i) {
