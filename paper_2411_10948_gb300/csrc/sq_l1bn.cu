@@ -1628,10 +1628,30 @@ static int coop_blocks() {
   return slot - 1;
 }
 
+// The errors of a cooperative launch that this stream or device does not take now -- a stream of
+// a context that holds only some of the SMs, for one, cannot have every block resident at once.
+// The context is unharmed and nothing was launched: the call goes on with its next form.
+static bool launch_refused(cudaError_t err) {
+  return err == cudaErrorCooperativeLaunchTooLarge || err == cudaErrorLaunchOutOfResources ||
+         err == cudaErrorNotSupported || err == cudaErrorNotPermitted;
+}
+
+// The outcome of a cooperative launch, the error of a refused one cleared.
+static int coop_outcome(cudaError_t err, const char* what, bool* launched) {
+  if (err == cudaSuccess) err = cudaGetLastError();
+  *launched = err == cudaSuccess;
+  if (err == cudaSuccess) return SQ_OK;
+  if (launch_refused(err)) {
+    cudaGetLastError();
+    return SQ_OK;
+  }
+  return cuda_fail(err, what);
+}
+
 // The single-launch form of a call: the counter and range slots zeroed, then one
-// cooperative launch of `blocks` blocks.
+// cooperative launch of `blocks` blocks.  *launched: false where the launch was refused.
 template <bool FWD>
-static int launch_coop(const L1bnArgs& a, int G, int blocks, int32_t* dev_status, cudaStream_t s) {
+static int launch_coop(const L1bnArgs& a, int G, int blocks, int32_t* dev_status, cudaStream_t s, bool* launched) {
   cudaError_t err = cudaMemsetAsync(a.sync, 0, 256 + kSpread * static_cast<size_t>(a.C) * sizeof(unsigned), s);
   if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync (l1bn sync)");
   CoopGeom g;
@@ -1657,8 +1677,7 @@ static int launch_coop(const L1bnArgs& a, int G, int blocks, int32_t* dev_status
   cfg.numAttrs = 1;
   err = FWD ? cudaLaunchKernelEx(&cfg, l1bn_fwd_coop_kernel, a, g)
             : cudaLaunchKernelEx(&cfg, l1bn_bwd_coop_kernel, a, g);
-  if (err == cudaSuccess) err = cudaGetLastError();
-  return err == cudaSuccess ? SQ_OK : cuda_fail(err, FWD ? "l1bn_fwd_coop_kernel launch" : "l1bn_bwd_coop_kernel launch");
+  return coop_outcome(err, FWD ? "l1bn_fwd_coop_kernel launch" : "l1bn_bwd_coop_kernel launch", launched);
 }
 
 // The resident form's geometry for [R, C] on the current device: of the tile widths 64, 32 and
@@ -1681,8 +1700,10 @@ static bool res_plan(int64_t R, int64_t C, ResGeom* g, bool* fp32) {
                               reinterpret_cast<const void*>(l1bn_fwd_res_kernel<true>),
                               reinterpret_cast<const void*>(l1bn_bwd_res_kernel<false>),
                               reinterpret_cast<const void*>(l1bn_bwd_res_kernel<true>)};
+    int per_sm = 0;
     for (const void* k : kernels)
-      ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kResDyn)) == cudaSuccess;
+      ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kResDyn)) == cudaSuccess &&
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kResThreads, kResDyn) == cudaSuccess && per_sm >= 1;
     cudaGetLastError();
     cached[dev] = ok ? sms + 1 : 1;
   }
@@ -1716,9 +1737,10 @@ static bool res_plan(int64_t R, int64_t C, ResGeom* g, bool* fp32) {
 }
 
 // The resident form of a call: the barrier counter and range slots zeroed, one cooperative
-// launch.
+// launch.  *launched: false where it was refused.
 template <bool FWD>
-static int launch_res(const L1bnArgs& a, int G, ResGeom g, bool fp32, int32_t* dev_status, cudaStream_t s) {
+static int launch_res(const L1bnArgs& a, int G, ResGeom g, bool fp32, int32_t* dev_status, cudaStream_t s,
+                      bool* launched) {
   cudaError_t err = cudaMemsetAsync(a.sync, 0, 256 + kSpread * static_cast<size_t>(a.C) * sizeof(unsigned), s);
   if (err != cudaSuccess) return cuda_fail(err, "cudaMemsetAsync (l1bn sync)");
   g.G = G;
@@ -1736,8 +1758,7 @@ static int launch_res(const L1bnArgs& a, int G, ResGeom g, bool fp32, int32_t* d
   cfg.numAttrs = 1;
   err = cudaLaunchKernelEx(&cfg, FWD ? (fp32 ? l1bn_fwd_res_kernel<true> : l1bn_fwd_res_kernel<false>)
                                      : (fp32 ? l1bn_bwd_res_kernel<true> : l1bn_bwd_res_kernel<false>), a, g);
-  if (err == cudaSuccess) err = cudaGetLastError();
-  return err == cudaSuccess ? SQ_OK : cuda_fail(err, FWD ? "l1bn_fwd_res_kernel launch" : "l1bn_bwd_res_kernel launch");
+  return coop_outcome(err, FWD ? "l1bn_fwd_res_kernel launch" : "l1bn_bwd_res_kernel launch", launched);
 }
 
 // the single-launch form serves this call: few enough channels for every block to form
@@ -1750,6 +1771,20 @@ static int coop_use(int64_t C) {
   const int lgo = tile_lg(C) < kCoopOutLg ? tile_lg(C) : kCoopOutLg;
   const int64_t gxo = (C + (int64_t(4) << lgo) - 1) / (int64_t(4) << lgo);
   return blocks >= gxo && blocks >= 8 ? blocks : 0;
+}
+
+// The first of the single-launch forms that serves the call and is not refused: the resident
+// form, then the cooperative one.  *launched: false where the call is left to the chain.
+template <bool FWD>
+static int launch_single(const L1bnArgs& a, int G, int32_t* dev_status, cudaStream_t s, bool* launched) {
+  *launched = false;
+  ResGeom g;
+  bool fp32 = false;
+  int st = SQ_OK;
+  if (res_plan<FWD>(a.R, a.C, &g, &fp32)) st = launch_res<FWD>(a, G, g, fp32, dev_status, s, launched);
+  if (st != SQ_OK || *launched) return st;
+  if (const int blocks = coop_use<FWD>(a.C)) st = launch_coop<FWD>(a, G, blocks, dev_status, s, launched);
+  return st;
 }
 
 }  // namespace sq
@@ -1816,10 +1851,9 @@ extern "C" sq_status shiftquant_l1bn_forward(const float* x, int64_t rows, int64
   a.beta = beta;
   a.vec_in = (ld_x % 4 == 0) && aligned16(x);
   a.vec_out = (ld_y % 4 == 0) && aligned16(y);
-  ResGeom g;
-  bool fp32 = false;
-  if (res_plan<true>(rows, channels, &g, &fp32)) return launch_res<true>(a, n_groups, g, fp32, dev_status, s);
-  if (const int blocks = coop_use<true>(channels)) return launch_coop<true>(a, n_groups, blocks, dev_status, s);
+  bool single = false;
+  st = launch_single<true>(a, n_groups, dev_status, s, &single);
+  if (st != SQ_OK || single) return st;
   // the channel sums start at zero (a kernel, not a memset, so that the launches after the
   // range pass stay a chain of kernels, each launched behind the one before)
   const int64_t nz = 3 * kSpread * channels;
@@ -1874,10 +1908,9 @@ extern "C" sq_status shiftquant_l1bn_backward(const float* dy, int64_t rows, int
   a.dbeta = dbeta;
   a.vec_in = (ld_dy % 4 == 0) && aligned16(dy);
   a.vec_out = (ld_dx % 4 == 0) && aligned16(dx);
-  ResGeom g;
-  bool fp32 = false;
-  if (res_plan<false>(rows, channels, &g, &fp32)) return launch_res<false>(a, n_groups, g, fp32, dev_status, s);
-  if (const int blocks = coop_use<false>(channels)) return launch_coop<false>(a, n_groups, blocks, dev_status, s);
+  bool single = false;
+  st = launch_single<false>(a, n_groups, dev_status, s, &single);
+  if (st != SQ_OK || single) return st;
   const int64_t nz = 2 * kSpread * channels;
   l1bn_zero_kernel<<<static_cast<unsigned>((nz + 255) / 256 < 1024 ? (nz + 255) / 256 : 1024), 256, 0, s>>>(
       a.st + kStP * kSpread * channels, nz);

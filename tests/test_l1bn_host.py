@@ -1,0 +1,70 @@
+"""Which launches an L1 batch norm call makes, on the host alone (no GPU): the resident form, and
+what follows where the device refuses a cooperative launch."""
+import ctypes
+
+import pytest
+
+import fake_cudart
+from paper_2411_10948_gb300 import native as N
+
+FWD_CHAIN = ["l1bn_zero_kernel", "calib_init_kernel", "colmax_kernel", "group_kernel", "l1bn_fwd_quant_kernel",
+             "l1bn_fwd_dev_kernel", "l1bn_fwd_chan_kernel", "l1bn_fwd_lut_kernel", "l1bn_fwd_out_kernel"]
+BWD_CHAIN = ["l1bn_zero_kernel", "calib_init_kernel", "colmax_kernel", "group_kernel", "l1bn_bwd_quant_kernel",
+             "l1bn_bwd_chan_kernel", "l1bn_bwd_out_kernel"]
+TOO_LARGE, OUT_OF_RESOURCES, ILLEGAL_ADDRESS = 720, 701, 700   # cudaError_t
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return fake_cudart.link(tmp_path_factory.mktemp("fake"))
+
+
+def call(lib, R, C, backward):
+    """(status, kernels launched) of one call; addresses stand for device memory."""
+    p = ctypes.c_void_p
+    state, size = p(1 << 32), lib.shiftquant_l1bn_state_bytes(R, C)
+    lib.fake_log()
+    if backward:
+        st = lib.shiftquant_l1bn_backward(p(1 << 20), R, C, C, 8, 4, 1, state, size, p(1 << 21), C, p(1 << 22),
+                                          p(1 << 23), p(1 << 24), None)
+    else:
+        st = lib.shiftquant_l1bn_forward(p(1 << 20), R, C, C, p(1 << 22), p(1 << 23), 8, 4, p(1 << 21), C, state,
+                                         size, p(1 << 24), None)
+    return st, fake_cudart.launches(lib)
+
+
+@pytest.mark.parametrize("backward", [False, True])
+@pytest.mark.parametrize("C", [64, 2048])
+def test_resident_form_is_one_cooperative_launch(lib, C, backward):
+    st, ran = call(lib, 3136, C, backward)
+    assert st == N.SQ_OK and len(ran) == 1
+    assert ran[0][0] == f"l1bn_{'bwd' if backward else 'fwd'}_res_kernel" and ran[0][2] == "c"
+
+
+@pytest.mark.parametrize("error", [TOO_LARGE, OUT_OF_RESOURCES])
+@pytest.mark.parametrize("backward", [False, True])
+def test_refused_launch_goes_on_with_the_next_form(lib, backward, error):
+    d = "bwd" if backward else "fwd"
+    chain = BWD_CHAIN if backward else FWD_CHAIN
+    # too many channels for the cooperative form: the chain
+    lib.fake_refuse(error, 1)
+    st, ran = call(lib, 3136, 2048, backward)
+    assert st == N.SQ_OK and [k[0] for k in ran] == chain
+    assert lib.fake_last_error() == 0
+    # the resident form's blocks alone do not fit: the cooperative form
+    lib.fake_refuse(error, 1)
+    st, ran = call(lib, 3136, 64, backward)
+    assert st == N.SQ_OK and [k[0] for k in ran] == [f"l1bn_{d}_coop_kernel"]
+    # no cooperative launch at all
+    lib.fake_refuse(error, 2)
+    st, ran = call(lib, 3136, 64, backward)
+    assert st == N.SQ_OK and [k[0] for k in ran] == chain
+    assert lib.fake_last_error() == 0
+
+
+def test_other_errors_are_reported(lib):
+    lib.fake_refuse(ILLEGAL_ADDRESS, 1)
+    st, ran = call(lib, 3136, 2048, False)
+    assert st == N.SQ_ECUDA and ran == []
+    lib.fake_refuse(0, 0)
+    lib.cudaGetLastError()
