@@ -750,8 +750,8 @@ def run_l1bn(args, dev):
         fm, bm = statistics.median(times["fwd"]), statistics.median(times["bwd"])
         fg = L1BN_FWD_BYTES * R * C / (fm * 1e-3) / 1e9
         bg = L1BN_BWD_BYTES * R * C / (bm * 1e-3) / 1e9
-        launches = {"fwd": N.shiftquant_l1bn_kernel_launches(C),
-                    "bwd": N.shiftquant_l1bn_kernel_launches(C, True)}
+        launches = {"fwd": N.shiftquant_l1bn_launches(R, C),
+                    "bwd": N.shiftquant_l1bn_launches(R, C, True)}
         out.append({"shape": name, "rows": R, "channels": C, "fwd_ms": fm, "bwd_ms": bm,
                     "fwd_gbs": fg, "bwd_gbs": bg, "fwd_frac": fg / peaks["hbm_gbs"],
                     "bwd_frac": bg / peaks["hbm_gbs"], "launches": launches})

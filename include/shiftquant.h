@@ -555,13 +555,16 @@ sq_status shiftquant_l1bn_backward(const float *dy, int64_t rows, int64_t channe
                                    float *dgamma, float *dbeta, int32_t *dev_status,
                                    void *stream);
 
-/* The most kernels one shiftquant_l1bn_forward (backward = 0) or _backward (1) call launches
- * on the current device: 1 for at most 1024 channels on a device that runs cooperative
- * launches (the passes then run as phases of one launch, separated by bounded grid barriers,
- * after one memset of the state's counter and range slots), else the chain of 9 (forward) or
- * 7 (backward) kernels -- also 1 where the rows are few enough for the tensor to stay in the
- * SMs' shared memory; 0 for no channels, -1 for a negative count or no device.  Results do
- * not depend on the form. */
+/* Kernels one shiftquant_l1bn_forward (backward = 0) or _backward (1) call on [rows, channels]
+ * launches on the current device: 1 where the tensor fits the SMs' shared memory or has at most
+ * 1024 channels, on a device that runs cooperative launches (the passes then run as phases of
+ * one launch, separated by bounded grid barriers, after one memset of the state's counter and
+ * range slots), else the chain of 9 (forward) or 7 (backward) kernels; 0 for no channels, -1
+ * for a negative count or no device.  A call whose cooperative launch the device refuses goes
+ * on with the chain.  Results do not depend on the form. */
+int shiftquant_l1bn_launches(int64_t rows, int64_t channels, int backward);
+
+/* The same for the most rows a call may have: 1 for at most 1024 channels, else the chain's. */
 int shiftquant_l1bn_kernel_launches(int64_t channels, int backward);
 
 /* Self-test of the single-launch L1 batch normalization's grid barrier (failure path):

@@ -1820,6 +1820,16 @@ extern "C" sq_status shiftquant_selftest_grid_barrier_timeout(void* scratch, int
   return err == cudaSuccess ? SQ_OK : cuda_fail(err, "l1bn_selftest_barrier_kernel launch");
 }
 
+extern "C" int shiftquant_l1bn_launches(int64_t rows, int64_t channels, int backward) {
+  if (rows < 0) return -1;
+  ResGeom g;
+  bool fp32 = false;
+  if (rows > 0 && channels > 0 && channels < (int64_t(1) << 31) &&
+      (backward ? res_plan<false>(rows, channels, &g, &fp32) : res_plan<true>(rows, channels, &g, &fp32)))
+    return 1;
+  return shiftquant_l1bn_kernel_launches(channels, backward);
+}
+
 extern "C" int shiftquant_l1bn_kernel_launches(int64_t channels, int backward) {
   if (channels < 0 || channels >= (int64_t(1) << 31)) return -1;
   if (channels == 0) return 0;

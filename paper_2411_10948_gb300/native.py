@@ -43,7 +43,8 @@ EXPORTS = (
     "shiftquant_layer_step", "shiftquant_layer_step_host", "shiftquant_layer_step_host_split",
     "shiftquant_selftest_wait_timeout",
     "shiftquant_l1bn_state_bytes", "shiftquant_l1bn_forward", "shiftquant_l1bn_backward",
-    "shiftquant_l1bn_kernel_launches", "shiftquant_selftest_grid_barrier_timeout",
+    "shiftquant_l1bn_launches", "shiftquant_l1bn_kernel_launches",
+    "shiftquant_selftest_grid_barrier_timeout",
     "shiftquant_group_order", "shiftquant_group_order_width", "shiftquant_quantize_ordered",
     "shiftquant_pack_codes", "shiftquant_unpack_codes", "shiftquant_packed_groups_bytes",
     "shiftquant_pack_groups", "shiftquant_unpack_groups",
@@ -184,6 +185,8 @@ def load(path: str | None = None) -> ctypes.CDLL:
     lib.shiftquant_selftest_wait_timeout.restype = i32
     lib.shiftquant_l1bn_state_bytes.argtypes = [i64, i64]
     lib.shiftquant_l1bn_state_bytes.restype = sz
+    lib.shiftquant_l1bn_launches.argtypes = [i64, i64, i32]
+    lib.shiftquant_l1bn_launches.restype = i32
     lib.shiftquant_l1bn_kernel_launches.argtypes = [i64, i32]
     lib.shiftquant_l1bn_kernel_launches.restype = i32
     lib.shiftquant_selftest_grid_barrier_timeout.argtypes = [vp, vp, vp]
@@ -521,8 +524,14 @@ def shiftquant_selftest_grid_barrier_timeout(scratch, dev_status, stream=None) -
                                                            _stream(stream)))
 
 
+def shiftquant_l1bn_launches(rows: int, channels: int, backward: bool = False) -> int:
+    """Kernels one L1 batch-norm call on [rows, channels] launches: 1 in a single-launch form,
+    else 9 / 7."""
+    return int(load().shiftquant_l1bn_launches(rows, channels, 1 if backward else 0))
+
+
 def shiftquant_l1bn_kernel_launches(channels: int, backward: bool = False) -> int:
-    """Kernels one L1 batch-norm call launches: 1 in the single-launch form, else 9 / 7."""
+    """The same for the most rows a call may have."""
     return int(load().shiftquant_l1bn_kernel_launches(channels, 1 if backward else 0))
 
 

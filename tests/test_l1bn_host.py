@@ -68,3 +68,21 @@ def test_other_errors_are_reported(lib):
     assert st == N.SQ_ECUDA and ran == []
     lib.fake_refuse(0, 0)
     lib.cudaGetLastError()
+
+
+# a whole tensor and a ring of rows on the SMs, too many rows for that, few channels, and more
+# channel tiles than SMs
+@pytest.mark.parametrize("R,C", [(3136, 2048), (200704, 64), (300000, 64), (300000, 1024), (300000, 1025),
+                                 (40, 9800), (1, 1), (1 << 24, 3000)])
+@pytest.mark.parametrize("backward", [False, True])
+def test_launch_query_is_what_a_call_launches(lib, R, C, backward):
+    st, ran = call(lib, R, C, backward)
+    assert st == N.SQ_OK and lib.shiftquant_l1bn_launches(R, C, int(backward)) == len(ran)
+
+
+def test_launch_query_at_its_edges(lib):
+    assert lib.shiftquant_l1bn_launches(5, 0, 0) == 0
+    assert lib.shiftquant_l1bn_launches(-1, 5, 0) == lib.shiftquant_l1bn_launches(5, -1, 0) == -1
+    # no rows, and any number of rows
+    assert lib.shiftquant_l1bn_launches(0, 64, 0) == lib.shiftquant_l1bn_kernel_launches(64, 0) == 1
+    assert lib.shiftquant_l1bn_kernel_launches(1025, 0) == 9 and lib.shiftquant_l1bn_kernel_launches(1025, 1) == 7
