@@ -40,6 +40,14 @@ __device__ __forceinline__ float4 ld_stream_v4(const float* p) {
   return v;
 }
 
+// The same through L1, for rows that need not start on a sector: a sector in which two threads'
+// or two rows' parts meet is fetched once, where a load past L1 fetches it again.
+__device__ __forceinline__ float4 ld_rows_v4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+
 // One value by a coherent load (through L1, as a plain load), issued where it stands: volatile,
 // so that the compiler neither sinks it to its use nor moves it across a griddep_wait.  With
 // plain loads, a 5003 x 1155 x 1001 layer step (6-bit) took 5 us more; past

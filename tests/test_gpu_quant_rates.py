@@ -1,0 +1,49 @@
+"""Rates of the quantizer that hold between shapes: what a width costs next to one beside it."""
+import pytest
+import torch
+
+from paper_2411_10948_gb300 import layer as L
+from paper_2411_10948_gb300 import native as N
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_2411_10948_gb300 import build
+    build.build_library()
+    N.load()
+
+
+def time_per_element(C, bits, mode):
+    """ps an element: graph replays of calls on three tensors in turn, larger than L2 together."""
+    M, n = 30_000_000 // C, 24
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    sets = []
+    for _ in range(3):
+        x, q = torch.randn(M, C, device="cuda"), L.ShiftTensor.alloc(M, C, bits, 4, "cuda", False)
+        N.shiftquant_calibrate(x, N.SQ_GRAN_SHIFT, 4, q.range, q.tau0, q.exp, st)
+        sets.append((x, q))
+    g = L.CapturedStep(lambda: [N.shiftquant_quantize(x, N.SQ_GRAN_SHIFT, bits, 4, q.tau0, q.exp, None, mode, 5,
+                                                      q.codes, None, q.scale) for x, q in sets * (n // 3)])
+    for _ in range(3):
+        g.replay()
+    ts = []
+    for _ in range(15):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        g.replay()
+        b.record()
+        b.synchronize()
+        ts.append(a.elapsed_time(b) / n * 1e9 / (M * C))
+    return sorted(ts)[len(ts) // 2]
+
+
+# Rows of 292 and 420 fp32 start and end inside a sector, and so do their BF16 codes (the code
+# rows are padded to 16 bytes); rows of 288 and 416 do not.  What the shared sectors cost is at
+# most one more sector of 37 (53) read and one partly written of 19 (27): 4% of the bytes.  Three
+# times that is allowed (read twice in every tile they took 25-30% longer).
+@pytest.mark.parametrize("ragged,whole", [(292, 288), (420, 416)])
+def test_rows_that_share_sectors(ragged, whole):
+    r, w = (time_per_element(C, 8, N.SQ_ROUND_NEAREST_EVEN) for C in (ragged, whole))
+    assert r <= 1.12 * w, (r, w)
