@@ -536,34 +536,59 @@ __device__ __forceinline__ TensorScale tensor_scale(const QuantArgs& a, float Qf
   return t;
 }
 
-// What a thread needs of column c: the multiplier (SHIFT: 2^e Q / tau_0, where
+// What a thread needs of the columns of its quad: the multiplier (SHIFT: 2^e Q / tau_0, where
 // fl(fl(x 2^e) fl(Q / tau_0)) = fl(x (2^e fl(Q / tau_0))) as scaling by 2^e is exact -- or, not
-// merged, Q / tau_0 alone with the 2^e in `scale`; PER_COL: Q / range), whether the column's
-// codes are all 0, and the folded shift (PER_ROW).
-struct ColumnValues {
-  float mul, scale, fold;
-  bool zero;
-};
-
+// merged, Q / tau_0 alone with the 2^e in `pre`; PER_COL: Q / range), the folded shift
+// (PER_ROW), and which columns' codes are all 0 (bits of the result).  c: the quad's first column;
+// columns past the last stand for the last, and their codes are not stored.  write: the
+// quad's exponents or scales are this thread's to store.
 template <int GRAN, bool FOLD>
-__device__ __forceinline__ ColumnValues column_values(const QuantArgs& a, const TensorScale& ts,
-                                                      float ftau, int64_t c, float Qf, bool write) {
-  ColumnValues v = {1.0f, 1.0f, 1.0f, false};
-  if (GRAN == SQ_GRAN_SHIFT) {
-    const int e = a.exp != nullptr ? ld_here(a.exp + c)
-                                   : channel_exponent(__ldcg(a.crange + c), ts.tau, a.G);
-    if (write && a.exp_out != nullptr) a.exp_out[c] = static_cast<uint8_t>(e);
-    v.scale = pow2f(e);
-    v.mul = ts.zero ? 0.0f : (ts.merged ? __fmul_rn(ts.invS, v.scale) : ts.invS);
-    v.zero = ts.zero;
-  } else if (GRAN == SQ_GRAN_PER_COL) {
-    const float rg = __ldcg(a.rt + c);
-    v.mul = channel_inv(rg, Qf, &v.zero);
-    if (write) a.scale_out[c] = v.zero ? 0.0f : __fdiv_rn(rg, Qf);
-  } else if (FOLD) {
-    v.fold = fold_factor(a, ftau, c);
+__device__ __forceinline__ unsigned quad_columns(const QuantArgs& a, const TensorScale& ts, float ftau, int64_t c,
+                                                 float Qf, bool write, float (&mul)[4], float (&pre)[4],
+                                                 float (&cfold)[4]) {
+  const int last = static_cast<int>(min(a.C - 1 - c, int64_t(3)));
+  const int64_t c0 = last < 0 ? a.C - 1 : c;
+  int at[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    at[j] = max(min(j, last), 0);
+    mul[j] = pre[j] = cfold[j] = 1.0f;
   }
-  return v;
+  unsigned zero = 0u;
+  if (GRAN == SQ_GRAN_SHIFT) {
+    int e[4];
+    if (a.exp != nullptr) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) e[j] = ld_here(a.exp + c0 + at[j]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) e[j] = channel_exponent(__ldcg(a.crange + c0 + at[j]), ts.tau, a.G);
+      if (write && a.exp_out != nullptr) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j <= last) a.exp_out[c + j] = static_cast<uint8_t>(e[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      pre[j] = pow2f(e[j]);
+      mul[j] = ts.zero ? 0.0f : (ts.merged ? __fmul_rn(ts.invS, pre[j]) : ts.invS);
+    }
+    zero = ts.zero ? 15u : 0u;
+  } else if (GRAN == SQ_GRAN_PER_COL) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float rg = __ldcg(a.rt + c0 + at[j]);
+      bool z = false;
+      mul[j] = channel_inv(rg, Qf, &z);
+      zero |= z ? 1u << j : 0u;
+      if (write && j <= last) a.scale_out[c + j] = z ? 0.0f : __fdiv_rn(rg, Qf);
+    }
+  } else if (FOLD) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) cfold[j] = fold_factor(a, ftau, c0 + at[j]);
+  }
+  return zero;
 }
 
 // The per-row values of a chunk's eight rows, held one row per lane of each group of eight
@@ -742,7 +767,7 @@ __device__ __forceinline__ void store_transposed(const QuantArgs& a, uint32_t ti
 
 // The values a thread keeps over its rows.
 struct QuadState {
-  float mul[4], pre[4], cfold[4];   // per column (ColumnValues)
+  float mul[4], pre[4], cfold[4];   // per column (quad_columns)
   unsigned czero;                   // bit j: column j's codes are all 0
   bool merged;                      // TensorScale
   bool rare;   // inputs quantize to zero for another reason than their value, or need a second scale
@@ -760,17 +785,7 @@ __device__ __forceinline__ QuadState quad_state(const QuantArgs& a, unsigned bx,
   if (GRAN == SQ_GRAN_SHIFT) ts = tensor_scale(a, Qf);
   const float ftau = FOLD && a.fold == nullptr ? slots_tau(a.ftslots) : 0.0f;
   t.merged = ts.merged;
-  t.czero = 0u;
-  const bool first = by == 0 && t.p.chunk == 0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    ColumnValues v = {1.0f, 1.0f, 1.0f, false};
-    if (t.p.c + j < a.C) v = column_values<GRAN, FOLD>(a, ts, ftau, t.p.c + j, Qf, first);
-    t.mul[j] = v.mul;
-    t.pre[j] = v.scale;
-    t.cfold[j] = v.fold;
-    t.czero |= v.zero ? 1u << j : 0u;
-  }
+  t.czero = quad_columns<GRAN, FOLD>(a, ts, ftau, t.p.c, Qf, by == 0 && t.p.chunk == 0, t.mul, t.pre, t.cfold);
   t.rv = row_values<GRAN, FOLD>(a, ftau, t.p.r, Qf, bx == 0 && t.p.col < 32);
   t.state = 0;   // seed + (idx + 1) gamma
   if (MODE == SQ_ROUND_STOCHASTIC)
@@ -819,10 +834,9 @@ __device__ __forceinline__ void keep_words(uint32_t slot, const uint32_t (&words
 }
 
 // The chunk of each of the quad's columns -- its code of every row, gathered from the thread's
-// slots -- into the staging area.
+// slots (row i's at slot0 + i step) -- into the staging area.
 template <typename CodeT>
-__device__ __forceinline__ void stage_chunks(const TilePos& p, int lg, uint32_t tile_smem) {
-  const uint32_t slot0 = quad_slot(tile_smem + (threadIdx.x >> 5) * kWarpBytes, lg, 0), step = 16u << lg;
+__device__ __forceinline__ void stage_chunks(const TilePos& p, int lg, uint32_t tile_smem, uint32_t slot0, uint32_t step) {
   uint32_t words[8][sizeof(CodeT)];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -869,6 +883,10 @@ enum Form {
   kOrdered    // aligned rows of x, codes in a group order
 };
 
+// Whether a kernel writes a transposed copy: as it is launched for, or as the arguments say.  (As
+// a test in the rows' unrolled body, eight predicated stores more.)
+enum Trans { kNoTrans, kTrans, kTransAny };
+
 template <int FORM>
 __device__ __forceinline__ bool register_tile(const QuantArgs& a, unsigned bx, unsigned by) {
   const int64_t r1 = (static_cast<int64_t>(by) + 1) << (11 - a.lg);
@@ -881,6 +899,15 @@ __device__ __forceinline__ bool register_tile(const QuantArgs& a, unsigned bx, u
   return c1 <= a.C || (FORM == kAligned && (a.C & 3) == 0);
 }
 
+// base + i rows of `bytes` bytes, as one multiply-add (a sum of two words would take two
+// instructions of the pipe that stochastic rounding fills)
+template <typename T>
+__device__ __forceinline__ T* row_at(T* base, uint32_t i, uint32_t bytes) {
+  uint64_t p;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(p) : "r"(i), "r"(bytes), "l"(base));
+  return reinterpret_cast<T*>(p);
+}
+
 template <int FORM>
 __device__ __forceinline__ void load_registers(const QuantArgs& a, unsigned bx, unsigned by, float4 (&x)[8]) {
   const TilePos p = tile_pos(a.lg, bx, by);
@@ -890,12 +917,13 @@ __device__ __forceinline__ void load_registers(const QuantArgs& a, unsigned bx, 
     const float* src = a.x + (p.c < a.C ? p.c : 0);
     if (p.r + 8 <= a.R) {
       src += p.r * a.ld;
+      const uint32_t row = static_cast<uint32_t>(a.ld * 4);
       if (a.sectors) {   // (set_alignment)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = ld_stream_v4(src + i * a.ld);
+        for (int i = 0; i < 8; ++i) x[i] = ld_stream_v4(row_at(src, i, row));
       } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = ld_rows_v4(src + i * a.ld);
+        for (int i = 0; i < 8; ++i) x[i] = ld_rows_v4(row_at(src, i, row));
       }
     } else {
 #pragma unroll
@@ -935,18 +963,22 @@ __device__ __forceinline__ void load_registers(const QuantArgs& a, unsigned bx, 
   }
 }
 
-template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD>
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int TRANS>
 __device__ __forceinline__ void quantize_registers(const QuantArgs& a, const QuadState& t, const float4 (&xin)[8],
                                                    uint32_t tile_smem) {
   const float Qf = static_cast<float>(a.Q);
   const uint64_t row_step = static_cast<uint64_t>(a.C) * kSplitMixGamma;
   const bool ordered = FORM == kOrdered && a.pos_cols != nullptr;
-  CodeT* dst = static_cast<CodeT*>(a.codes) + t.p.r * a.ldc + t.p.c;
+  CodeT* const first = static_cast<CodeT*>(a.codes) + t.p.r * a.ldc + t.p.c;
+  const uint32_t row = static_cast<uint32_t>(a.ldc * static_cast<int64_t>(sizeof(CodeT)));
   // the codes are kept in the thread's slots for the transposed copy and for a group order
-  const bool kept = a.codes_t != nullptr || ordered;
+  const bool trans = TRANS == kTransAny ? a.codes_t != nullptr : TRANS == kTrans;
+  const bool kept = trans || ordered;
   const uint32_t warp_smem = tile_smem + (threadIdx.x >> 5) * kWarpBytes;
   uint64_t state = t.state;
-  const uint32_t keep = quad_slot(warp_smem, a.lg, 0), step = 16u << a.lg;
+  // (slots of four codes each, those of a row side by side: no two lanes' stores share a bank)
+  constexpr uint32_t kSlot = 4 * sizeof(CodeT);
+  const uint32_t keep = warp_smem + (quad_slot(0, a.lg, 0) >> 4) * kSlot, step = kSlot << a.lg;
   // rows of the quad to store
   const int rows = a.codes == nullptr || ordered || t.p.c >= a.C ? 0 : static_cast<int>(min(a.R - t.p.r, int64_t(8)));
 #pragma unroll
@@ -956,6 +988,7 @@ __device__ __forceinline__ void quantize_registers(const QuantArgs& a, const Qua
     quantize_quad<CodeT, GRAN, MODE, FOLD>(t, x, i, state, Qf, words);
     state += row_step;
     if (i < rows) {
+      CodeT* dst = row_at(first, i, row);
       if (FORM == kShifted && t.p.c + 3 >= a.C) {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -966,7 +999,6 @@ __device__ __forceinline__ void quantize_registers(const QuantArgs& a, const Qua
         *reinterpret_cast<uint32_t*>(dst) = words[0];
       }
     }
-    dst += a.ldc;
     if (kept) keep_words<CodeT>(keep + i * step, words);
   }
   if (ordered) {
@@ -981,20 +1013,20 @@ __device__ __forceinline__ void quantize_registers(const QuantArgs& a, const Qua
       if (g < groups) at[g] = ld_here(a.pos_cols + cb + 32 * g);
     const int nrows = static_cast<int>(min(a.R - rb, int64_t(64 >> (a.lg - 2))));
     // (column 32 g + lane of the warp's row r)
-    uint32_t from = warp_smem + (lane >> 2) * 16 + (lane & 3) * static_cast<int>(sizeof(CodeT));
+    uint32_t from = warp_smem + lane * static_cast<int>(sizeof(CodeT));
     CodeT* d = static_cast<CodeT*>(a.codes) + rb * a.ldc;
     __syncwarp();
 #pragma unroll 2
     for (int r = 0; r < nrows; ++r) {
 #pragma unroll
       for (int g = 0; g < 4; ++g)
-        if (g < groups) d[at[g]] = ld_shared_code<CodeT>(from + g * 128);
+        if (g < groups) d[at[g]] = ld_shared_code<CodeT>(from + g * 32 * static_cast<int>(sizeof(CodeT)));
       from += step;
       d += a.ldc;
     }
     __syncwarp();   // the chunks may overwrite the slots
   }
-  if (a.codes_t != nullptr) stage_chunks<CodeT>(t.p, a.lg, tile_smem);
+  if (trans) stage_chunks<CodeT>(t.p, a.lg, tile_smem, keep, step);
 }
 
 // ------------------------------------------------------------ shared-memory path
@@ -1043,13 +1075,13 @@ __device__ __forceinline__ void quantize_rows(const QuantArgs& a, const QuadStat
     }
     if (a.codes_t != nullptr) keep_words<CodeT>(slot, words);
   }
-  if (a.codes_t != nullptr) stage_chunks<CodeT>(t.p, a.lg, tile_smem);
+  if (a.codes_t != nullptr) stage_chunks<CodeT>(t.p, a.lg, tile_smem, slot0, step);
 }
 
 // One tile of a tensor.
 // WAIT: x may be read before the preceding kernel has completed (it did not write x), its
 // results only after the wait.
-template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, bool WAIT = false>
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int TRANS, bool WAIT = false>
 __device__ __forceinline__ void quantize_block(const QuantArgs& a, unsigned bx, unsigned by, uint32_t tile_smem) {
   bool fast = register_tile<FORM>(a, bx, by);
   float4 x[8];
@@ -1058,37 +1090,38 @@ __device__ __forceinline__ void quantize_block(const QuantArgs& a, unsigned bx, 
   const QuadState t = quad_state<GRAN, MODE, FOLD>(a, bx, by);
   fast = fast && !__any_sync(0xFFFFFFFFu, t.rare);   // (each warp by itself: their parts of the tile are their own)
   if (fast) {
-    quantize_registers<CodeT, FORM, GRAN, MODE, FOLD>(a, t, x, tile_smem);
+    quantize_registers<CodeT, FORM, GRAN, MODE, FOLD, TRANS>(a, t, x, tile_smem);
   } else {
     load_tile(a, bx, by, tile_smem + (threadIdx.x >> 5) * kWarpBytes);
     quantize_rows<CodeT, GRAN, MODE, FOLD>(a, t, tile_smem);
   }
-  if (a.codes_t != nullptr) store_transposed<CodeT>(a, tile_smem, bx, by);
+  if (TRANS == kTransAny ? a.codes_t != nullptr : TRANS == kTrans) store_transposed<CodeT>(a, tile_smem, bx, by);
 }
 
-template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD>
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int TRANS>
 __global__ void __launch_bounds__(kQuantThreads, 4) quantize_kernel(const QuantArgs a) {
   __shared__ __align__(128) uint8_t tile[8 * kWarpBytes];
   // launched early behind the range pass: nothing it wrote (nor x) is read before it is done
   if (!a.beside) griddep_wait();
   griddep_launch_dependents();
-  quantize_block<CodeT, FORM, GRAN, MODE, FOLD>(a, blockIdx.x, blockIdx.y, smem_u32(tile));
+  quantize_block<CodeT, FORM, GRAN, MODE, FOLD, TRANS>(a, blockIdx.x, blockIdx.y, smem_u32(tile));
   if (a.beside) griddep_wait();
 }
 
-template <typename CodeT, int FORM, int GRAN, bool FOLD>
+template <typename CodeT, int FORM, int GRAN, bool FOLD, int TRANS = kTransAny>
 static void launch_mode(const QuantArgs& a, int mode, dim3 grid, cudaStream_t s) {
   if (mode == SQ_ROUND_NEAREST_EVEN)
-    launch_pdl(quantize_kernel<CodeT, FORM, GRAN, SQ_ROUND_NEAREST_EVEN, FOLD>, grid, dim3(kQuantThreads), s, a);
+    launch_pdl(quantize_kernel<CodeT, FORM, GRAN, SQ_ROUND_NEAREST_EVEN, FOLD, TRANS>, grid, dim3(kQuantThreads), s, a);
   else
-    launch_pdl(quantize_kernel<CodeT, FORM, GRAN, SQ_ROUND_STOCHASTIC, FOLD>, grid, dim3(kQuantThreads), s, a);
+    launch_pdl(quantize_kernel<CodeT, FORM, GRAN, SQ_ROUND_STOCHASTIC, FOLD, TRANS>, grid, dim3(kQuantThreads), s, a);
 }
 
 template <typename CodeT, int FORM>
 static void launch_gran(const QuantArgs& a, int gran, int mode, dim3 grid, cudaStream_t s) {
   const bool fold = FORM != kOrdered && (a.fold != nullptr || a.frange != nullptr);   // group-ordered codes carry no fold
   if (gran == SQ_GRAN_SHIFT) {
-    launch_mode<CodeT, FORM, SQ_GRAN_SHIFT, false>(a, mode, grid, s);
+    if (a.codes_t != nullptr) launch_mode<CodeT, FORM, SQ_GRAN_SHIFT, false, kTrans>(a, mode, grid, s);
+    else launch_mode<CodeT, FORM, SQ_GRAN_SHIFT, false, kNoTrans>(a, mode, grid, s);
   } else if (gran == SQ_GRAN_PER_COL) {
     if (fold) launch_mode<CodeT, FORM, SQ_GRAN_PER_COL, FORM != kOrdered>(a, mode, grid, s);
     else launch_mode<CodeT, FORM, SQ_GRAN_PER_COL, false>(a, mode, grid, s);
@@ -1125,7 +1158,7 @@ __device__ __forceinline__ void quantize_weight_block(const QuantArgs& af, const
   const QuadState td = quad_state<kRow, kRn, FD>(ad, bx, by);
   fast = fast && !__any_sync(0xFFFFFFFFu, td.rare);
   if (fast) {
-    quantize_registers<CodeT, FORM, kRow, kRn, FD>(ad, td, x, tile_smem);
+    quantize_registers<CodeT, FORM, kRow, kRn, FD, kNoTrans>(ad, td, x, tile_smem);
   } else {   // the per-in-channel role has no transposed copy: it leaves the tile as it is
     load_tile(af, bx, by, tile_smem + (threadIdx.x >> 5) * kWarpBytes);
     quantize_rows<CodeT, kRow, kRn, FD>(ad, td, tile_smem);
@@ -1136,7 +1169,7 @@ __device__ __forceinline__ void quantize_weight_block(const QuantArgs& af, const
     fast = false;
   }
   if (fast)
-    quantize_registers<CodeT, FORM, kCol, kRn, FF>(af, tf, x, tile_smem);
+    quantize_registers<CodeT, FORM, kCol, kRn, FF, kTrans>(af, tf, x, tile_smem);
   else
     quantize_rows<CodeT, kCol, kRn, FF>(af, tf, tile_smem);
   store_transposed<CodeT>(af, tile_smem, bx, by);
@@ -1300,13 +1333,13 @@ __global__ void __launch_bounds__(kQuantThreads, 4) layer_quantize_kernel(const 
   griddep_launch_dependents();
   unsigned b = blockIdx.x;
   if (b < q.xend) {
-    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_NEAREST_EVEN, false, true>(q.x, b % q.xgx, b / q.xgx, smem);
+    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_NEAREST_EVEN, false, kTransAny, true>(q.x, b % q.xgx, b / q.xgx, smem);
   } else if (b < q.wend) {
     b -= q.xend;
     quantize_weight_block<CodeT, FORM, true, true, true>(q.wf, q.wd, b % q.wgx, b / q.wgx, smem);
   } else {
     b -= q.wend;
-    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_STOCHASTIC, false, true>(q.g, b % q.ggx, b / q.ggx, smem);
+    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_STOCHASTIC, false, kTransAny, true>(q.g, b % q.ggx, b / q.ggx, smem);
   }
 }
 
@@ -1499,7 +1532,9 @@ static void set_alignment(QuantArgs* a, int cbytes) {
   const bool ordered = a->pos_cols != nullptr || a->pos_rows != nullptr;
   a->form = ordered ? kOrdered : (a->vec_in ? kAligned : kShifted);
   const bool in = a->form == kShifted ? aligned16(a->x) : a->vec_in != 0;
-  a->fast = in && (a->codes == nullptr || a->vec_out || a->pos_cols != nullptr);
+  // (rows of less than 4 GB: row_at)
+  a->fast = in && (a->codes == nullptr || a->vec_out || a->pos_cols != nullptr) && a->ld < (int64_t(1) << 30) &&
+            a->ldc < (int64_t(1) << 31);
 }
 
 // both roles of a weight (the folds are set by the caller)
