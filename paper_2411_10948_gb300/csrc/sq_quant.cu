@@ -605,7 +605,7 @@ __device__ __forceinline__ RowValues row_values(const QuantArgs& a, float ftau, 
   const int lane = threadIdx.x & 31;
   const int64_t r = r0 + (lane & 7);
   if (GRAN == SQ_GRAN_PER_ROW) {
-    bool z = true;
+    bool z = false;   // (rows past the last: their codes are not stored)
     if (r < a.R) {
       const float rg = __ldcg(a.rt + r);
       v.mul = channel_inv(rg, Qf, &z);
@@ -833,22 +833,11 @@ __device__ __forceinline__ void keep_words(uint32_t slot, const uint32_t (&words
     st_shared_u32(slot, words[0]);
 }
 
-// The chunk of each of the quad's columns -- its code of every row, gathered from the thread's
-// slots (row i's at slot0 + i step) -- into the staging area.
+// The chunk of each of the quad's columns -- its code of every row, words[i] those of row i --
+// into the staging area.
 template <typename CodeT>
-__device__ __forceinline__ void stage_chunks(const TilePos& p, int lg, uint32_t tile_smem, uint32_t slot0, uint32_t step) {
-  uint32_t words[8][sizeof(CodeT)];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    if constexpr (sizeof(CodeT) == 2) {
-      const uint2 v = ld_shared_v2_u32(slot0 + i * step);
-      words[i][0] = v.x;
-      words[i][1] = v.y;
-    } else {
-      words[i][0] = ld_shared_u32(slot0 + i * step);
-    }
-  }
-  __syncwarp();   // every lane's slots have been read: the chunks may overwrite them
+__device__ __forceinline__ void stage_chunks(const TilePos& p, int lg, uint32_t tile_smem,
+                                             const uint32_t (&words)[8][sizeof(CodeT)]) {
   // (the quad's columns differ in the low two bits of the column alone, which chunk_addr
   // exclusive-ors into the low bits of the place)
   constexpr uint32_t kChunkBytes = 8 * sizeof(CodeT);
@@ -875,6 +864,24 @@ __device__ __forceinline__ void stage_chunks(const TilePos& p, int lg, uint32_t 
   }
 }
 
+// The same from the thread's slots (keep_words), row i's at slot0 + i step.
+template <typename CodeT>
+__device__ __forceinline__ void stage_slots(const TilePos& p, int lg, uint32_t tile_smem, uint32_t slot0, uint32_t step) {
+  uint32_t words[8][sizeof(CodeT)];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    if constexpr (sizeof(CodeT) == 2) {
+      const uint2 v = ld_shared_v2_u32(slot0 + i * step);
+      words[i][0] = v.x;
+      words[i][1] = v.y;
+    } else {
+      words[i][0] = ld_shared_u32(slot0 + i * step);
+    }
+  }
+  __syncwarp();   // every lane's slots have been read: the chunks may overwrite them
+  stage_chunks<CodeT>(p, lg, tile_smem, words);
+}
+
 // ---------------------------------------------------------------- register path
 // What a launch's register path expects of its tensor; tiles that differ take the other path.
 enum Form {
@@ -883,9 +890,18 @@ enum Form {
   kOrdered    // aligned rows of x, codes in a group order
 };
 
-// Whether a kernel writes a transposed copy: as it is launched for, or as the arguments say.  (As
-// a test in the rows' unrolled body, eight predicated stores more.)
-enum Trans { kNoTrans, kTrans, kTransAny };
+// Which outputs a kernel writes: the codes, both, the transposed codes alone, or as the arguments
+// say.  (Each test in the rows' unrolled body is eight predicated stores more.)
+enum Outputs { kCodes, kBoth, kTransposed, kAnyOutputs };
+
+template <int OUT>
+__device__ __forceinline__ bool has_codes(const QuantArgs& a) {
+  return OUT == kAnyOutputs ? a.codes != nullptr : OUT != kTransposed;
+}
+template <int OUT>
+__device__ __forceinline__ bool has_transposed(const QuantArgs& a) {
+  return OUT == kAnyOutputs ? a.codes_t != nullptr : OUT != kCodes;
+}
 
 template <int FORM>
 __device__ __forceinline__ bool register_tile(const QuantArgs& a, unsigned bx, unsigned by) {
@@ -963,24 +979,26 @@ __device__ __forceinline__ void load_registers(const QuantArgs& a, unsigned bx, 
   }
 }
 
-template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int TRANS>
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int OUT>
 __device__ __forceinline__ void quantize_registers(const QuantArgs& a, const QuadState& t, const float4 (&xin)[8],
                                                    uint32_t tile_smem) {
   const float Qf = static_cast<float>(a.Q);
   const uint64_t row_step = static_cast<uint64_t>(a.C) * kSplitMixGamma;
-  const bool ordered = FORM == kOrdered && a.pos_cols != nullptr;
+  const bool ordered = FORM == kOrdered && OUT != kTransposed && a.pos_cols != nullptr;
   CodeT* const first = static_cast<CodeT*>(a.codes) + t.p.r * a.ldc + t.p.c;
   const uint32_t row = static_cast<uint32_t>(a.ldc * static_cast<int64_t>(sizeof(CodeT)));
   // the codes are kept in the thread's slots for the transposed copy and for a group order
-  const bool trans = TRANS == kTransAny ? a.codes_t != nullptr : TRANS == kTrans;
-  const bool kept = trans || ordered;
+  const bool trans = has_transposed<OUT>(a);
+  constexpr bool kHeld = OUT == kTransposed;   // nothing else to keep in registers: no slots
+  const bool kept = !kHeld && (trans || ordered);
+  uint32_t held[kHeld ? 8 : 1][sizeof(CodeT)];
   const uint32_t warp_smem = tile_smem + (threadIdx.x >> 5) * kWarpBytes;
   uint64_t state = t.state;
   // (slots of four codes each, those of a row side by side: no two lanes' stores share a bank)
   constexpr uint32_t kSlot = 4 * sizeof(CodeT);
   const uint32_t keep = warp_smem + (quad_slot(0, a.lg, 0) >> 4) * kSlot, step = kSlot << a.lg;
   // rows of the quad to store
-  const int rows = a.codes == nullptr || ordered || t.p.c >= a.C ? 0 : static_cast<int>(min(a.R - t.p.r, int64_t(8)));
+  const int rows = !has_codes<OUT>(a) || ordered || t.p.c >= a.C ? 0 : static_cast<int>(min(a.R - t.p.r, int64_t(8)));
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const float x[4] = {xin[i].x, xin[i].y, xin[i].z, xin[i].w};
@@ -1000,6 +1018,10 @@ __device__ __forceinline__ void quantize_registers(const QuantArgs& a, const Qua
       }
     }
     if (kept) keep_words<CodeT>(keep + i * step, words);
+    if constexpr (kHeld) {
+#pragma unroll
+      for (int k = 0; k < static_cast<int>(sizeof(CodeT)); ++k) held[i][k] = words[k];
+    }
   }
   if (ordered) {
     // The channels of a group keep their order, so 32 consecutive columns go to a few runs of
@@ -1026,7 +1048,10 @@ __device__ __forceinline__ void quantize_registers(const QuantArgs& a, const Qua
     }
     __syncwarp();   // the chunks may overwrite the slots
   }
-  if (trans) stage_chunks<CodeT>(t.p, a.lg, tile_smem, keep, step);
+  if constexpr (kHeld)
+    stage_chunks<CodeT>(t.p, a.lg, tile_smem, held);
+  else if (trans)
+    stage_slots<CodeT>(t.p, a.lg, tile_smem, keep, step);
 }
 
 // ------------------------------------------------------------ shared-memory path
@@ -1075,13 +1100,13 @@ __device__ __forceinline__ void quantize_rows(const QuantArgs& a, const QuadStat
     }
     if (a.codes_t != nullptr) keep_words<CodeT>(slot, words);
   }
-  if (a.codes_t != nullptr) stage_chunks<CodeT>(t.p, a.lg, tile_smem, slot0, step);
+  if (a.codes_t != nullptr) stage_slots<CodeT>(t.p, a.lg, tile_smem, slot0, step);
 }
 
 // One tile of a tensor.
 // WAIT: x may be read before the preceding kernel has completed (it did not write x), its
 // results only after the wait.
-template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int TRANS, bool WAIT = false>
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int OUT, bool WAIT = false>
 __device__ __forceinline__ void quantize_block(const QuantArgs& a, unsigned bx, unsigned by, uint32_t tile_smem) {
   bool fast = register_tile<FORM>(a, bx, by);
   float4 x[8];
@@ -1090,38 +1115,60 @@ __device__ __forceinline__ void quantize_block(const QuantArgs& a, unsigned bx, 
   const QuadState t = quad_state<GRAN, MODE, FOLD>(a, bx, by);
   fast = fast && !__any_sync(0xFFFFFFFFu, t.rare);   // (each warp by itself: their parts of the tile are their own)
   if (fast) {
-    quantize_registers<CodeT, FORM, GRAN, MODE, FOLD, TRANS>(a, t, x, tile_smem);
+    quantize_registers<CodeT, FORM, GRAN, MODE, FOLD, OUT>(a, t, x, tile_smem);
   } else {
     load_tile(a, bx, by, tile_smem + (threadIdx.x >> 5) * kWarpBytes);
     quantize_rows<CodeT, GRAN, MODE, FOLD>(a, t, tile_smem);
   }
-  if (TRANS == kTransAny ? a.codes_t != nullptr : TRANS == kTrans) store_transposed<CodeT>(a, tile_smem, bx, by);
+  if (has_transposed<OUT>(a)) store_transposed<CodeT>(a, tile_smem, bx, by);
 }
 
-template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int TRANS>
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int OUT>
 __global__ void __launch_bounds__(kQuantThreads, 4) quantize_kernel(const QuantArgs a) {
   __shared__ __align__(128) uint8_t tile[8 * kWarpBytes];
   // launched early behind the range pass: nothing it wrote (nor x) is read before it is done
   if (!a.beside) griddep_wait();
   griddep_launch_dependents();
-  quantize_block<CodeT, FORM, GRAN, MODE, FOLD, TRANS>(a, blockIdx.x, blockIdx.y, smem_u32(tile));
+  quantize_block<CodeT, FORM, GRAN, MODE, FOLD, OUT>(a, blockIdx.x, blockIdx.y, smem_u32(tile));
   if (a.beside) griddep_wait();
 }
 
-template <typename CodeT, int FORM, int GRAN, bool FOLD, int TRANS = kTransAny>
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD, int OUT>
+static void launch_outputs(const QuantArgs& a, dim3 grid, cudaStream_t s) {
+  launch_pdl(quantize_kernel<CodeT, FORM, GRAN, MODE, FOLD, OUT>, grid, dim3(kQuantThreads), s, a);
+}
+
+// The outputs that get a kernel of their own: ShiftQuant's codes with and without the copy, and
+// what each role of a weight writes.
+template <typename CodeT, int FORM, int GRAN, int MODE, bool FOLD>
+static void launch_form(const QuantArgs& a, dim3 grid, cudaStream_t s) {
+  constexpr bool kShift = GRAN == SQ_GRAN_SHIFT, kWeight = !kShift && MODE == SQ_ROUND_NEAREST_EVEN;
+  if constexpr (kShift) {
+    if (a.codes != nullptr && a.codes_t != nullptr)
+      return launch_outputs<CodeT, FORM, GRAN, MODE, FOLD, kBoth>(a, grid, s);
+  }
+  if constexpr (kShift || (kWeight && GRAN == SQ_GRAN_PER_ROW)) {
+    if (a.codes_t == nullptr) return launch_outputs<CodeT, FORM, GRAN, MODE, FOLD, kCodes>(a, grid, s);
+  }
+  if constexpr (kWeight && GRAN == SQ_GRAN_PER_COL) {
+    if (a.codes == nullptr) return launch_outputs<CodeT, FORM, GRAN, MODE, FOLD, kTransposed>(a, grid, s);
+  }
+  launch_outputs<CodeT, FORM, GRAN, MODE, FOLD, kAnyOutputs>(a, grid, s);
+}
+
+template <typename CodeT, int FORM, int GRAN, bool FOLD>
 static void launch_mode(const QuantArgs& a, int mode, dim3 grid, cudaStream_t s) {
   if (mode == SQ_ROUND_NEAREST_EVEN)
-    launch_pdl(quantize_kernel<CodeT, FORM, GRAN, SQ_ROUND_NEAREST_EVEN, FOLD, TRANS>, grid, dim3(kQuantThreads), s, a);
+    launch_form<CodeT, FORM, GRAN, SQ_ROUND_NEAREST_EVEN, FOLD>(a, grid, s);
   else
-    launch_pdl(quantize_kernel<CodeT, FORM, GRAN, SQ_ROUND_STOCHASTIC, FOLD, TRANS>, grid, dim3(kQuantThreads), s, a);
+    launch_form<CodeT, FORM, GRAN, SQ_ROUND_STOCHASTIC, FOLD>(a, grid, s);
 }
 
 template <typename CodeT, int FORM>
 static void launch_gran(const QuantArgs& a, int gran, int mode, dim3 grid, cudaStream_t s) {
   const bool fold = FORM != kOrdered && (a.fold != nullptr || a.frange != nullptr);   // group-ordered codes carry no fold
   if (gran == SQ_GRAN_SHIFT) {
-    if (a.codes_t != nullptr) launch_mode<CodeT, FORM, SQ_GRAN_SHIFT, false, kTrans>(a, mode, grid, s);
-    else launch_mode<CodeT, FORM, SQ_GRAN_SHIFT, false, kNoTrans>(a, mode, grid, s);
+    launch_mode<CodeT, FORM, SQ_GRAN_SHIFT, false>(a, mode, grid, s);
   } else if (gran == SQ_GRAN_PER_COL) {
     if (fold) launch_mode<CodeT, FORM, SQ_GRAN_PER_COL, FORM != kOrdered>(a, mode, grid, s);
     else launch_mode<CodeT, FORM, SQ_GRAN_PER_COL, false>(a, mode, grid, s);
@@ -1158,7 +1205,7 @@ __device__ __forceinline__ void quantize_weight_block(const QuantArgs& af, const
   const QuadState td = quad_state<kRow, kRn, FD>(ad, bx, by);
   fast = fast && !__any_sync(0xFFFFFFFFu, td.rare);
   if (fast) {
-    quantize_registers<CodeT, FORM, kRow, kRn, FD, kNoTrans>(ad, td, x, tile_smem);
+    quantize_registers<CodeT, FORM, kRow, kRn, FD, kCodes>(ad, td, x, tile_smem);
   } else {   // the per-in-channel role has no transposed copy: it leaves the tile as it is
     load_tile(af, bx, by, tile_smem + (threadIdx.x >> 5) * kWarpBytes);
     quantize_rows<CodeT, kRow, kRn, FD>(ad, td, tile_smem);
@@ -1169,7 +1216,7 @@ __device__ __forceinline__ void quantize_weight_block(const QuantArgs& af, const
     fast = false;
   }
   if (fast)
-    quantize_registers<CodeT, FORM, kCol, kRn, FF, kTrans>(af, tf, x, tile_smem);
+    quantize_registers<CodeT, FORM, kCol, kRn, FF, kTransposed>(af, tf, x, tile_smem);
   else
     quantize_rows<CodeT, kCol, kRn, FF>(af, tf, tile_smem);
   store_transposed<CodeT>(af, tile_smem, bx, by);
@@ -1333,13 +1380,13 @@ __global__ void __launch_bounds__(kQuantThreads, 4) layer_quantize_kernel(const 
   griddep_launch_dependents();
   unsigned b = blockIdx.x;
   if (b < q.xend) {
-    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_NEAREST_EVEN, false, kTransAny, true>(q.x, b % q.xgx, b / q.xgx, smem);
+    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_NEAREST_EVEN, false, kAnyOutputs, true>(q.x, b % q.xgx, b / q.xgx, smem);
   } else if (b < q.wend) {
     b -= q.xend;
     quantize_weight_block<CodeT, FORM, true, true, true>(q.wf, q.wd, b % q.wgx, b / q.wgx, smem);
   } else {
     b -= q.wend;
-    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_STOCHASTIC, false, kTransAny, true>(q.g, b % q.ggx, b / q.ggx, smem);
+    quantize_block<CodeT, FORM, SQ_GRAN_SHIFT, SQ_ROUND_STOCHASTIC, false, kAnyOutputs, true>(q.g, b % q.ggx, b / q.ggx, smem);
   }
 }
 

@@ -47,3 +47,32 @@ def time_per_element(C, bits, mode):
 def test_rows_that_share_sectors(ragged, whole):
     r, w = (time_per_element(C, 8, N.SQ_ROUND_NEAREST_EVEN) for C in (ragged, whole))
     assert r <= 1.12 * w, (r, w)
+
+
+def time_per_row_codes(K, C):
+    """us a call: a weight's per-in-channel codes, graph replays."""
+    n, st = 48, torch.zeros(1, dtype=torch.int32, device="cuda")
+    w = torch.randn(K, C, device="cuda")
+    d = L.ChannelTensor(L.empty_codes(K, C, 8, 4, "cuda"), torch.zeros(K, device="cuda"), torch.zeros(K, device="cuda"))
+    N.shiftquant_calibrate(w, N.SQ_GRAN_PER_ROW, 4, d.range, None, None, st)
+    g = L.CapturedStep(lambda: [N.shiftquant_quantize(w, N.SQ_GRAN_PER_ROW, 8, 4, d.range, None, None,
+                                                      N.SQ_ROUND_NEAREST_EVEN, 0, d.codes, None, d.scale)
+                                for _ in range(n)])
+    for _ in range(3):
+        g.replay()
+    ts = []
+    for _ in range(15):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        g.replay()
+        b.record()
+        b.synchronize()
+        ts.append(a.elapsed_time(b) / n * 1e3)
+    return sorted(ts)[len(ts) // 2]
+
+
+# 300 rows end inside a tile of 64 rows, 320 do not: the same tiles, the last one partly used (as
+# long as a tile's rows past the tensor's end counted as rows of zeros, it took twice the time)
+def test_last_row_tile_of_a_weight():
+    r, w = time_per_row_codes(300, 256), time_per_row_codes(320, 256)
+    assert r <= 1.3 * w, (r, w)
