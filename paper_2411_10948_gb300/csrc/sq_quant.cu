@@ -378,10 +378,11 @@ __global__ void __launch_bounds__(256)
 // reader takes the largest
 constexpr int kTauSlots = 16;
 
-__device__ __forceinline__ float slots_tau(const unsigned* slots) {   // by a whole warp
+__device__ __forceinline__ unsigned slots_word(const unsigned* slots) {   // the lane's word, of a whole warp
   const int lane = threadIdx.x & 31;
-  return __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, lane < kTauSlots ? __ldcg(slots + lane) : 0u));
+  return __ldcg(slots + (lane < kTauSlots ? lane : 0));
 }
+__device__ __forceinline__ float slots_tau(unsigned word) { return __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, word)); }
 
 struct QuantArgs {
   const float* x;
@@ -513,82 +514,44 @@ __device__ __forceinline__ float channel_inv(float rg, float Qf, bool* zero) {
   return *zero ? 0.0f : inv;
 }
 
-// the folded shift of inner channel i of the other operand, as a factor
-__device__ __forceinline__ float fold_factor(const QuantArgs& a, float ftau, int64_t i) {
-  const int e = a.fold != nullptr ? ld_here(a.fold + i)
-                                  : channel_exponent(__ldcg(a.frange + i), ftau, a.G);
-  return pow2f(a.G - 1 - e);
+// What gives the exponent of channel i: itself where it is given, else the channel's range
+__device__ __forceinline__ uint32_t load_exponent(const uint8_t* exp, const float* range, int64_t i) {
+  return exp != nullptr ? static_cast<uint32_t>(ld_here(exp + i)) : __float_as_uint(__ldcg(range + i));
+}
+__device__ __forceinline__ int exponent_of(uint32_t v, const uint8_t* exp, float tau, int G) {
+  return exp != nullptr ? static_cast<int>(v) : channel_exponent(__uint_as_float(v), tau, G);
 }
 
-// ShiftQuant's per-tensor values
-struct TensorScale {
-  float tau, invS;
-  bool zero;    // tau_0 is 0 or not finite, or Q / tau_0 overflows: every code is 0
-  bool merged;  // 2^e Q / tau_0 is finite for every e: one multiplication per element
-};
-
-__device__ __forceinline__ TensorScale tensor_scale(const QuantArgs& a, float Qf) {
-  TensorScale t;
-  t.tau = a.tslots != nullptr ? slots_tau(a.tslots) : __ldcg(a.rt);
-  t.invS = __fdiv_rn(Qf, t.tau);
-  t.zero = !(t.tau > 0.0f) || !isfinite(t.tau) || !isfinite(t.invS);
-  t.merged = isfinite(__fmul_rn(t.invS, pow2f(a.G - 1)));
-  return t;
+// Four columns' values from p: one load where they are all there (whole) and aligned, else those
+// at the offsets at.  Past L1 a load of one column in four fetches the other three's sectors too:
+// transposed codes of a [3072, 768] weight (4-bit) 4.7 us with four loads, 3.5 us with one.
+__device__ __forceinline__ void load_ranges(const float* p, bool whole, const int (&at)[4], float (&v)[4]) {
+  if (whole && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+    const float4 f = __ldcg(reinterpret_cast<const float4*>(p));
+    v[0] = f.x;
+    v[1] = f.y;
+    v[2] = f.z;
+    v[3] = f.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = __ldcg(p + at[j]);
+  }
 }
-
-// What a thread needs of the columns of its quad: the multiplier (SHIFT: 2^e Q / tau_0, where
-// fl(fl(x 2^e) fl(Q / tau_0)) = fl(x (2^e fl(Q / tau_0))) as scaling by 2^e is exact -- or, not
-// merged, Q / tau_0 alone with the 2^e in `pre`; PER_COL: Q / range), the folded shift
-// (PER_ROW), and which columns' codes are all 0 (bits of the result).  c: the quad's first column;
-// columns past the last stand for the last, and their codes are not stored.  write: the
-// quad's exponents or scales are this thread's to store.
-template <int GRAN, bool FOLD>
-__device__ __forceinline__ unsigned quad_columns(const QuantArgs& a, const TensorScale& ts, float ftau, int64_t c,
-                                                 float Qf, bool write, float (&mul)[4], float (&pre)[4],
-                                                 float (&cfold)[4]) {
-  const int last = static_cast<int>(min(a.C - 1 - c, int64_t(3)));
-  const int64_t c0 = last < 0 ? a.C - 1 : c;
-  int at[4];
+__device__ __forceinline__ void load_exponents(const uint8_t* exp, const float* range, int64_t c0, bool whole,
+                                               const int (&at)[4], uint32_t (&v)[4]) {
+  if (exp == nullptr) {
+    float f[4];
+    load_ranges(range + c0, whole, at, f);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    at[j] = max(min(j, last), 0);
-    mul[j] = pre[j] = cfold[j] = 1.0f;
+    for (int j = 0; j < 4; ++j) v[j] = __float_as_uint(f[j]);
+  } else if (whole && (reinterpret_cast<uintptr_t>(exp + c0) & 3) == 0) {
+    const uint32_t w = static_cast<uint32_t>(ld_here(reinterpret_cast<const int*>(exp + c0)));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = (w >> (8 * j)) & 0xFFu;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = static_cast<uint32_t>(ld_here(exp + c0 + at[j]));
   }
-  unsigned zero = 0u;
-  if (GRAN == SQ_GRAN_SHIFT) {
-    int e[4];
-    if (a.exp != nullptr) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) e[j] = ld_here(a.exp + c0 + at[j]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) e[j] = channel_exponent(__ldcg(a.crange + c0 + at[j]), ts.tau, a.G);
-      if (write && a.exp_out != nullptr) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (j <= last) a.exp_out[c + j] = static_cast<uint8_t>(e[j]);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      pre[j] = pow2f(e[j]);
-      mul[j] = ts.zero ? 0.0f : (ts.merged ? __fmul_rn(ts.invS, pre[j]) : ts.invS);
-    }
-    zero = ts.zero ? 15u : 0u;
-  } else if (GRAN == SQ_GRAN_PER_COL) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float rg = __ldcg(a.rt + c0 + at[j]);
-      bool z = false;
-      mul[j] = channel_inv(rg, Qf, &z);
-      zero |= z ? 1u << j : 0u;
-      if (write && j <= last) a.scale_out[c + j] = z ? 0.0f : __fdiv_rn(rg, Qf);
-    }
-  } else if (FOLD) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) cfold[j] = fold_factor(a, ftau, c0 + at[j]);
-  }
-  return zero;
 }
 
 // The per-row values of a chunk's eight rows, held one row per lane of each group of eight
@@ -598,24 +561,6 @@ struct RowValues {
   float mul, fold;
   unsigned zero;  // bit i: row i of the lane's group quantizes to zero
 };
-
-template <int GRAN, bool FOLD>
-__device__ __forceinline__ RowValues row_values(const QuantArgs& a, float ftau, int64_t r0, float Qf, bool write) {
-  RowValues v = {1.0f, 1.0f, 0u};
-  const int lane = threadIdx.x & 31;
-  const int64_t r = r0 + (lane & 7);
-  if (GRAN == SQ_GRAN_PER_ROW) {
-    bool z = false;   // (rows past the last: their codes are not stored)
-    if (r < a.R) {
-      const float rg = __ldcg(a.rt + r);
-      v.mul = channel_inv(rg, Qf, &z);
-      if (write) a.scale_out[r] = z ? 0.0f : __fdiv_rn(rg, Qf);
-    }
-    v.zero = (__ballot_sync(0xFFFFFFFFu, z) >> (lane & 24)) & 0xFFu;
-  }
-  if (GRAN == SQ_GRAN_PER_COL && FOLD && r < a.R) v.fold = fold_factor(a, ftau, r);
-  return v;
-}
 
 // The thread's place in the tile at (bx, by).
 struct TilePos {
@@ -767,36 +712,105 @@ __device__ __forceinline__ void store_transposed(const QuantArgs& a, uint32_t ti
 
 // The values a thread keeps over its rows.
 struct QuadState {
-  float mul[4], pre[4], cfold[4];   // per column (quad_columns)
+  float mul[4], pre[4], cfold[4];   // per column (quad_state)
   unsigned czero;                   // bit j: column j's codes are all 0
-  bool merged;                      // TensorScale
+  bool merged;                      // (quad_state)
   bool rare;   // inputs quantize to zero for another reason than their value, or need a second scale
   RowValues rv;
   uint64_t state;                   // generator state of element (row, column 0 of the quad)
   TilePos p;
 };
 
+// The values of a thread's quad of columns and chunk of rows.  Per column the multiplier (SHIFT:
+// 2^e Q / tau_0, where fl(fl(x 2^e) fl(Q / tau_0)) = fl(x (2^e fl(Q / tau_0))) as scaling by 2^e
+// is exact -- or, not merged, Q / tau_0 alone with the 2^e in `pre`; PER_COL: Q / range) and the
+// folded shift (PER_ROW).  Columns and rows past the last stand for it: their codes are not
+// stored.  Everything is loaded before any of it is worked on (the divisions branch, and no load
+// moves ahead of a branch): the loads take one latency beside x's, not one after another
+// ([3072, 768] transposed weight codes, 4-bit: 4.9 and 4.4 us).
 template <int GRAN, int MODE, bool FOLD>
 __device__ __forceinline__ QuadState quad_state(const QuantArgs& a, unsigned bx, unsigned by) {
   const float Qf = static_cast<float>(a.Q);
   QuadState t;
   t.p = tile_pos(a.lg, bx, by);
-  TensorScale ts = {};
-  if (GRAN == SQ_GRAN_SHIFT) ts = tensor_scale(a, Qf);
-  const float ftau = FOLD && a.fold == nullptr ? slots_tau(a.ftslots) : 0.0f;
-  t.merged = ts.merged;
-  t.czero = quad_columns<GRAN, FOLD>(a, ts, ftau, t.p.c, Qf, by == 0 && t.p.chunk == 0, t.mul, t.pre, t.cfold);
-  t.rv = row_values<GRAN, FOLD>(a, ftau, t.p.r, Qf, bx == 0 && t.p.col < 32);
+  const int last = static_cast<int>(min(a.C - 1 - t.p.c, int64_t(3)));   // of the quad's columns
+  const int64_t c0 = last < 0 ? a.C - 1 : t.p.c;
+  const int64_t row = t.p.r + (threadIdx.x & 7), r = min(row, a.R - 1);
+  int at[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) at[j] = max(min(j, last), 0);
+  uint32_t cexp[4] = {0u, 0u, 0u, 0u}, rexp = 0u, tword = 0u, ftword = 0u;
+  float crange[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rrange = 0.0f;
+  if (GRAN == SQ_GRAN_SHIFT) {
+    tword = a.tslots != nullptr ? slots_word(a.tslots) : __float_as_uint(__ldcg(a.rt));
+    load_exponents(a.exp, a.crange, c0, last == 3, at, cexp);
+  }
+  if (FOLD && a.fold == nullptr) ftword = slots_word(a.ftslots);
+  if (GRAN == SQ_GRAN_PER_COL) {
+    load_ranges(a.rt + c0, last == 3, at, crange);
+    if (FOLD) rexp = load_exponent(a.fold, a.frange, r);
+  }
+  if (GRAN == SQ_GRAN_PER_ROW) {
+    rrange = __ldcg(a.rt + r);
+    if (FOLD) load_exponents(a.fold, a.frange, c0, last == 3, at, cexp);
+  }
+
+  const float ftau = FOLD && a.fold == nullptr ? slots_tau(ftword) : 0.0f;
+  t.rv = {1.0f, 1.0f, 0u};
+  t.czero = 0u;
+  t.merged = true;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) t.mul[j] = t.pre[j] = t.cfold[j] = 1.0f;
+  const bool write = by == 0 && t.p.chunk == 0;   // the first tiles' columns
+  if (GRAN == SQ_GRAN_SHIFT) {
+    const float tau = a.tslots != nullptr ? slots_tau(tword) : __uint_as_float(tword);
+    const float invS = __fdiv_rn(Qf, tau);
+    // tau_0 is 0 or not finite, or Q / tau_0 overflows: every code is 0
+    const bool zero = !(tau > 0.0f) || !isfinite(tau) || !isfinite(invS);
+    t.merged = isfinite(__fmul_rn(invS, pow2f(a.G - 1)));   // 2^e Q / tau_0 is finite for every e
+    t.czero = zero ? 15u : 0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      cexp[j] = static_cast<uint32_t>(exponent_of(cexp[j], a.exp, tau, a.G));
+      t.pre[j] = pow2f(static_cast<int>(cexp[j]));
+      t.mul[j] = zero ? 0.0f : (t.merged ? __fmul_rn(invS, t.pre[j]) : invS);
+    }
+    if (write && a.exp_out != nullptr) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (j <= last) a.exp_out[t.p.c + j] = static_cast<uint8_t>(cexp[j]);
+    }
+    if (bx == 0 && by == 0 && threadIdx.x == 0) {
+      *a.scale_out = zero ? 0.0f : __fdiv_rn(tau, Qf);
+      if (a.tau_out != nullptr) *a.tau_out = tau;
+    }
+  }
+  if (GRAN == SQ_GRAN_PER_COL) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      bool z = false;
+      t.mul[j] = channel_inv(crange[j], Qf, &z);
+      t.czero |= z ? 1u << j : 0u;
+      if (write && j <= last) a.scale_out[t.p.c + j] = z ? 0.0f : __fdiv_rn(crange[j], Qf);
+    }
+    if (FOLD) t.rv.fold = pow2f(a.G - 1 - exponent_of(rexp, a.fold, ftau, a.G));
+  }
+  if (GRAN == SQ_GRAN_PER_ROW) {
+    bool z = false;
+    t.rv.mul = channel_inv(rrange, Qf, &z);
+    z = z && row < a.R;
+    t.rv.zero = (__ballot_sync(0xFFFFFFFFu, z) >> (threadIdx.x & 24)) & 0xFFu;
+    if (bx == 0 && t.p.col < 32 && row < a.R) a.scale_out[row] = z ? 0.0f : __fdiv_rn(rrange, Qf);
+    if (FOLD) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) t.cfold[j] = pow2f(a.G - 1 - exponent_of(cexp[j], a.fold, ftau, a.G));
+    }
+  }
   t.state = 0;   // seed + (idx + 1) gamma
   if (MODE == SQ_ROUND_STOCHASTIC)
     t.state = a.seed + (static_cast<uint64_t>(a.row0 + t.p.r) * static_cast<uint64_t>(a.C) +
                         static_cast<uint64_t>(t.p.c) + 1ull) * kSplitMixGamma;
-  t.rare = t.czero != 0u || (GRAN == SQ_GRAN_SHIFT && !ts.merged) ||
-           (GRAN == SQ_GRAN_PER_ROW && t.rv.zero != 0u);
-  if (GRAN == SQ_GRAN_SHIFT && bx == 0 && by == 0 && threadIdx.x == 0) {
-    *a.scale_out = ts.zero ? 0.0f : __fdiv_rn(ts.tau, Qf);
-    if (a.tau_out != nullptr) *a.tau_out = ts.tau;
-  }
+  t.rare = t.czero != 0u || !t.merged || (GRAN == SQ_GRAN_PER_ROW && t.rv.zero != 0u);
   return t;
 }
 
