@@ -219,7 +219,7 @@ constexpr int kRangeCluster = 8;
 constexpr int64_t kRangeClusterMaxCols = 512;   // clusters for tensors of at most 512 columns
 
 template <int CL, bool ROWS, int FORM>
-__global__ void __launch_bounds__(kColTx* kColTy, ROWS || FORM == kViewStrided ? 4 : 6)
+__global__ void __launch_bounds__(kColTx* kColTy)
     colmax_kernel(const RangeView v, int lg, unsigned* __restrict__ range_bits,
                   unsigned* __restrict__ row_bits, int* __restrict__ status) {
   __shared__ unsigned red[kColTy * kColTx * 4];
