@@ -207,13 +207,11 @@ __device__ __noinline__ void write_acc_box(long long* acc, int64_t ld_acc, int64
   }
 }
 
-// One 32 x 32 output box of an epilogue warp (see emit_box) of a GEMM whose outputs are fp32
-// values and nothing else: T's integers `vals` times the column factors at `fac`, times the
-// row's factor first where kRow, staged and sent by a TMA store.
+// T's integers `vals` times the column factors at `fac`, times the row's factor first where
+// kRow, into the staging box.
 template <bool kRow>
-__device__ __forceinline__ void emit_plain(const uint32_t (&vals)[32], bool as_float, uint32_t fac, float rfac,
-                                           const CUtensorMap* tma_y, uint32_t buf, int32_t row0, int32_t col0,
-                                           int lane) {
+__device__ __forceinline__ void stage_values(const uint32_t (&vals)[32], bool as_float, uint32_t fac, float rfac,
+                                             uint32_t buf, int lane) {
   const uint32_t line = buf + lane * 128 + ((lane & 7) << 4);
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
@@ -228,6 +226,60 @@ __device__ __forceinline__ void emit_plain(const uint32_t (&vals)[32], bool as_f
     }
     st_shared_v4(line ^ (k << 4), o[0], o[1], o[2], o[3]);
   }
+}
+
+// T's integers as int32 into the staging box.
+__device__ __forceinline__ void stage_sums(const uint32_t (&vals)[32], bool as_float, uint32_t buf, int lane) {
+  const uint32_t line = buf + lane * 128 + ((lane & 7) << 4);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    uint32_t o[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      o[e] = as_float ? static_cast<uint32_t>(__float2int_rn(__uint_as_float(vals[k * 4 + e]))) : vals[k * 4 + e];
+    st_shared_v4(line ^ (k << 4), o[0], o[1], o[2], o[3]);
+  }
+}
+
+// The column maxima of |output| over the rows of a staged box, added to the output range
+// (ordered bit patterns of |y|): lane l reads the four columns 4 (l & 7) .. +3 of the eight rows
+// 8 (l >> 3) .. +7 (16-byte loads), the four row groups combine by two exchanges, and lanes 0-7
+// add each column's maximum.
+__device__ __forceinline__ void box_maxima(const GemmParams& p, uint32_t buf, int64_t row0, int64_t col0, int lane) {
+  const int cq = lane & 7, rg = lane >> 3;
+  uint32_t m[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int rr = rg * 8 + i;
+    if (row0 + rr < p.M) {
+      const uint4 v = ld_shared_v4_u32(buf + rr * 128 + ((cq ^ (rr & 7)) << 4));
+      m[0] = max(m[0], v.x & 0x7FFFFFFFu);
+      m[1] = max(m[1], v.y & 0x7FFFFFFFu);
+      m[2] = max(m[2], v.z & 0x7FFFFFFFu);
+      m[3] = max(m[3], v.w & 0x7FFFFFFFu);
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    m[e] = max(m[e], __shfl_xor_sync(0xFFFFFFFFu, m[e], 8));
+    m[e] = max(m[e], __shfl_xor_sync(0xFFFFFFFFu, m[e], 16));
+  }
+  if (rg == 0) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int64_t col = col0 + cq * 4 + e;
+      if (m[e] != 0u && col < p.N) atomicMax(p.colmax + col, m[e]);
+    }
+  }
+}
+
+// One 32 x 32 output box of an epilogue warp (see emit_box) of a GEMM whose outputs are fp32
+// values, sent by a TMA store.
+template <bool kRow>
+__device__ __forceinline__ void emit_plain(const uint32_t (&vals)[32], bool as_float, uint32_t fac, float rfac,
+                                           const CUtensorMap* tma_y, uint32_t buf, int32_t row0, int32_t col0,
+                                           int lane) {
+  stage_values<kRow>(vals, as_float, fac, rfac, buf, lane);
   fence_proxy_async_smem();
   __syncwarp();
   if (lane == 0) {
@@ -239,15 +291,7 @@ __device__ __forceinline__ void emit_plain(const uint32_t (&vals)[32], bool as_f
 // The box of a split of K: T's integers are added into the int32 workspace by a TMA reduction.
 __device__ __forceinline__ void emit_sums(const uint32_t (&vals)[32], bool as_float, const CUtensorMap* tma_ws,
                                           uint32_t buf, int32_t row0, int32_t col0, int lane) {
-  const uint32_t line = buf + lane * 128 + ((lane & 7) << 4);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    uint32_t o[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      o[e] = as_float ? static_cast<uint32_t>(__float2int_rn(__uint_as_float(vals[k * 4 + e]))) : vals[k * 4 + e];
-    st_shared_v4(line ^ (k << 4), o[0], o[1], o[2], o[3]);
-  }
+  stage_sums(vals, as_float, buf, lane);
   fence_proxy_async_smem();
   __syncwarp();
   if (lane == 0) {
@@ -259,18 +303,20 @@ __device__ __forceinline__ void emit_sums(const uint32_t (&vals)[32], bool as_fl
 // One 32 x 32 output box of an epilogue warp: lane = row, vals = the lane's 32 columns as
 // exact integers (FP32 patterns when `as_float`, else int32); fac = shared-memory address
 // of the box's 32 column factors (16-byte aligned), rfac the row's factor (weight gradient
-// only: the forward and loss-propagation outputs take the column factor alone).  The box is staged in shared
-// memory (128-byte swizzle) and leaves either as dequantized fp32 values (a TMA store, or a
-// lane a column where rows are not 16-byte aligned), as int32 partial sums through a TMA reduce-add into the split-K workspace, or -- past the
-// int32 range -- as int64 additions (64-bit atomics, a row of 32 columns per instruction)
-// into the int64 workspace.  The exactness-check integers are written when asked.
-// Two warps per scheduler drain a tile, so a box costs its instructions and their latency:
-// the two usual ways out (emit_plain, emit_sums) are straight-line code of their own, without
-// a test of the way out per element.  Layer launches with the tests inside / with pairs
-// storing 32-byte sectors from registers / so: 12544 x 2304 x 256 (4-bit) 52.3 / - / 46.8 us,
-// 12608 x 768 x 3072 (6-bit) 165 / 155 / 143 us, 4096 x 11008 x 4096 (8-bit) 715 / 700 / 674 us.
-// (The rarer ways out as functions shared with these cost the kernels with several chunks a unit
-// registers: 149, 698 us.)
+// only: the forward and loss-propagation outputs take the column factor alone).  The box is
+// staged in shared memory (128-byte swizzle) and leaves as dequantized fp32 values (a TMA store,
+// or a lane a column where rows are not 16-byte aligned), as int32 partial sums through a TMA
+// reduce-add into the split-K workspace, or -- past the int32 range -- as int64 additions (64-bit
+// atomics, a row of 32 columns per instruction) into the int64 workspace.  The exactness-check
+// integers and the column maxima are formed when asked.
+// Two warps per scheduler drain a tile, so a box costs its instructions and their latency: each
+// way out is straight-line code, without a test of the way out per element, and the column maxima
+// are taken from the staged box.  Layer launches with the tests inside / with pairs storing
+// 32-byte sectors from registers / so: 12544 x 2304 x 256 (4-bit) 52.3 / - / 46.8 us,
+// 12608 x 768 x 3072 (6-bit) 165 / 155 / 138 us, 4096 x 11008 x 4096 (8-bit) 715 / 700 / 674 us;
+// with the column maxima, tests inside / so: 12608 x 768 x 3072 (6-bit) 186 / 161 us,
+// 12544 x 2304 x 256 (8-bit) 139 / 129 us.  (One tail for all fp32 outputs, reached by tests of
+// the box: 144 us where the plain box by itself takes 138.)
 __device__ __forceinline__ void emit_box(const GemmParams& p, const CUtensorMap* tma_y,
                                          const CUtensorMap* tma_ws, const uint32_t (&vals)[32],
                                          bool as_float, uint32_t fac, float rfac, uint32_t buf,
@@ -283,88 +329,22 @@ __device__ __forceinline__ void emit_box(const GemmParams& p, const CUtensorMap*
   }
   __syncwarp();
   const int32_t r32 = static_cast<int32_t>(row0), c32 = static_cast<int32_t>(col0);
-  if (p.ws == nullptr && p.acc == nullptr && p.colmax == nullptr && tma_out) {
+  if (p.ws == nullptr && p.acc == nullptr && tma_out) {
     if (p.mode == 1)
       emit_plain<true>(vals, as_float, fac, rfac, tma_y, buf, r32, c32, lane);
     else
       emit_plain<false>(vals, as_float, fac, rfac, tma_y, buf, r32, c32, lane);
+    if (p.colmax != nullptr) box_maxima(p, buf, row0, col0, lane);
     return;
   }
   if (p.ws != nullptr && !p.wide) {
     emit_sums(vals, as_float, tma_ws, buf, r32, c32, lane);
     return;
   }
-  if (p.acc != nullptr && p.ws == nullptr) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      uint32_t o[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const uint32_t a = vals[k * 4 + e];
-        o[e] = as_float ? static_cast<uint32_t>(__float2int_rn(__uint_as_float(a))) : a;
-      }
-      st_shared_v4(buf + lane * 128 + ((k ^ (lane & 7)) << 4), o[0], o[1], o[2], o[3]);
-    }
-    __syncwarp();
-    write_acc_box(p.acc, p.ld_acc, p.M, p.N, p.mode == 1 ? p.row_exp : nullptr,
-                  p.mode == 1 ? p.col_exp : nullptr, p.G, buf, row0, col0, lane);
-    __syncwarp();
-  }
-  const bool row_scaled = p.mode == 1;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    uint32_t o[4];
-    const float4 f4 = p.ws != nullptr ? make_float4(0.f, 0.f, 0.f, 0.f) : ld_shared_v4_f32(fac + k * 16);
-    const float f[4] = {f4.x, f4.y, f4.z, f4.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const uint32_t a = vals[k * 4 + e];
-      if (p.ws != nullptr) {
-        o[e] = as_float ? static_cast<uint32_t>(__float2int_rn(__uint_as_float(a))) : a;
-      } else {
-        const float val = as_float ? __uint_as_float(a) : __int2float_rn(static_cast<int32_t>(a));
-        // x * 1 is x exactly, so skipping the row factor of 1 changes no result
-        o[e] = __float_as_uint(__fmul_rn(row_scaled ? __fmul_rn(val, rfac) : val, f[e]));
-      }
-    }
-    st_shared_v4(buf + lane * 128 + ((k ^ (lane & 7)) << 4), o[0], o[1], o[2], o[3]);
-  }
-  if (p.colmax != nullptr && p.ws == nullptr) {
-    // The column maxima of |output| over the box's 32 rows, from the staged box: lane l
-    // reads the four columns 4 (l & 7) .. +3 of the eight rows 8 (l >> 3) .. +7 (16-byte
-    // loads), the four row groups combine by two exchanges, and lanes 0-7 add each column's
-    // maximum to the output range (ordered bit patterns of |y|).
-    __syncwarp();
-    const int cq = lane & 7, rg = lane >> 3;
-    uint32_t m[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int rr = rg * 8 + i;
-      if (row0 + rr < p.M) {
-        uint32_t v[4];
-        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                     : "r"(buf + rr * 128 + ((cq ^ (rr & 7)) << 4)));
-#pragma unroll
-        for (int e = 0; e < 4; ++e) m[e] = max(m[e], v[e] & 0x7FFFFFFFu);
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      m[e] = max(m[e], __shfl_xor_sync(0xFFFFFFFFu, m[e], 8));
-      m[e] = max(m[e], __shfl_xor_sync(0xFFFFFFFFu, m[e], 16));
-    }
-    if (rg == 0) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int64_t col = col0 + cq * 4 + e;
-        if (m[e] != 0u && col < p.N) atomicMax(p.colmax + col, m[e]);
-      }
-    }
-  }
-  if (p.ws != nullptr && p.wide) {
+  if (p.ws != nullptr) {
     // a split of a K loop beyond the int32 range: its exact int32 sums are added into the
     // int64 workspace, row by row (the lanes cover 32 consecutive columns of a row)
+    stage_sums(vals, as_float, buf, lane);
     __syncwarp();
     unsigned long long* w64 = reinterpret_cast<unsigned long long*>(p.ws);
     const int64_t col = col0 + lane;
@@ -379,9 +359,21 @@ __device__ __forceinline__ void emit_box(const GemmParams& p, const CUtensorMap*
     __syncwarp();  // the staging box is free for the next one
     return;
   }
-  if (tma_out) {
-    fence_proxy_async_smem();
+  if (p.acc != nullptr) {
+    stage_sums(vals, as_float, buf, lane);
     __syncwarp();
+    write_acc_box(p.acc, p.ld_acc, p.M, p.N, p.mode == 1 ? p.row_exp : nullptr,
+                  p.mode == 1 ? p.col_exp : nullptr, p.G, buf, row0, col0, lane);
+    __syncwarp();
+  }
+  if (p.mode == 1)
+    stage_values<true>(vals, as_float, fac, rfac, buf, lane);
+  else
+    stage_values<false>(vals, as_float, fac, rfac, buf, lane);
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (p.colmax != nullptr) box_maxima(p, buf, row0, col0, lane);
+  if (tma_out) {
     if (lane == 0) {
       tma_store_2d(tma_y, buf, c32, r32);
       bulk_commit();
@@ -390,7 +382,6 @@ __device__ __forceinline__ void emit_box(const GemmParams& p, const CUtensorMap*
   }
   // rows that start anywhere: a lane a column, so that each store is one run of 128 bytes
   // (5003 x 1155 x 1001, 6-bit: the launch 67 us with four columns a lane, 52 us so)
-  __syncwarp();
   const int64_t col = col0 + lane;
   const int rows = p.M - row0 < 32 ? static_cast<int>(p.M - row0) : 32;
   float* dst = p.y + row0 * p.ldy + col;

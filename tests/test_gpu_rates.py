@@ -1,4 +1,5 @@
-"""Rates of the quantizer that hold between shapes: what a width costs next to one beside it."""
+"""Rates that hold between shapes and between calls: what a width costs next to one beside it, and
+what an output costs on top of a launch."""
 import pytest
 import torch
 
@@ -76,3 +77,35 @@ def time_per_row_codes(K, C):
 def test_last_row_tile_of_a_weight():
     r, w = time_per_row_codes(300, 256), time_per_row_codes(320, 256)
     assert r <= 1.3 * w, (r, w)
+
+
+# The column maxima of Y and dX are one more pass over boxes that are staged anyway: the launch
+# may take half as long again, not twice (as with a test of each box's way out per element)
+def test_layer_launch_with_ranges():
+    M, K, C, bits = 12544, 2304, 256, 6
+    lay = L.QuantLinear(M, K, C, bits, 4)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    for q, n in ((lay.x, K), (lay.g, C)):
+        L.shift_quantize(torch.randn((M, n), generator=g, device="cuda"), q, bits, 4, 0, 0, lay.status)
+    ws = torch.zeros(N.shiftquant_gemm_layer_workspace_bytes(M, K, C, bits, 4), dtype=torch.uint8, device="cuda")
+    yr, dr = torch.zeros(C, device="cuda"), torch.zeros(K, device="cuda")
+
+    def launch(**ranges):
+        N.shiftquant_gemm_layer(lay.x.codes, lay.x.codes_t, lay.x.scale, lay.x.exp, lay.g.codes, lay.g.codes_t,
+                                lay.g.scale, lay.g.exp, lay.wf.codes, lay.wf.scale, lay.wd.codes, lay.wd.scale,
+                                M, K, C, bits, 4, lay.y, lay.dx, lay.dw, workspace=ws, dev_status=lay.status, **ranges)
+
+    times = []
+    for kw in ({}, {"y_range": yr, "dx_range": dr}):
+        run = L.CapturedStep(lambda: [launch(**kw) for _ in range(8)])
+        ts = []
+        for _ in range(15):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            run.replay()
+            b.record()
+            b.synchronize()
+            ts.append(a.elapsed_time(b))
+        times.append(sorted(ts)[len(ts) // 2])
+    assert lay.status.item() == 0
+    assert times[1] <= 1.5 * times[0], times
