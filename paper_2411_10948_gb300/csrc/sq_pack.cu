@@ -8,10 +8,10 @@
 // the operand format before the GEMM that reads it.  Both directions are streaming HBM
 // passes: sixteen codes per thread and row, 16-byte loads and 8-byte stores where rows allow.
 // Bound by HBM and by how fast a launch of a few microseconds gets its loads out: a thread has
-// eight rows in flight, a block takes each row slab once, and a launch's blocks are resident
-// before the kernel ahead of them ends.  [12544, 2304] codes packed and unpacked: 23.9 us with
-// 4 rows in flight in one wave of blocks that walked the rows, 17.1 us so (20.9 with 4 rows,
-// 19.1 with 6; 18.0 with dense rows taken as one run of 4 KB pieces).
+// up to eight rows in flight (pack_shape), a block takes each row slab once, and a launch's
+// blocks are resident before the kernel ahead of them ends.  [12544, 2304] codes packed and
+// unpacked: 23.9 us with 4 rows in flight in one wave of blocks that walked the rows, 17.1 us so
+// (18.0 with dense rows taken as one run of 4 KB pieces).
 //
 // Layout: element c of a row in byte c / 2 of the packed row, the low nibble for even c,
 // as a 4-bit two's complement; map field of channel c at bit (c mod (8 / w)) w of byte
@@ -96,8 +96,6 @@ __device__ __forceinline__ uint2 e4m3_of_nibbles(uint32_t w) {
   return out;
 }
 
-constexpr int kPackRowsInFlight = 8;   // rows a thread loads before working on them
-
 // The 16 codes of a chunk as words (two BF16 or four E4M3 codes a word, low code first).
 template <typename CodeT>
 struct CodeChunk {
@@ -163,13 +161,12 @@ __device__ __forceinline__ uint2 pack_chunk(const CodeChunk<CodeT>& ch, bool& ba
 
 // codes [R, ld] -> packed [R, ldp]; a code outside [-8, 7] (not a 4-bit code) is packed as
 // its low nibble and flags SQ_DEV_INTERNAL.  Thread (x, y) of block (bx, by) packs the 16
-// codes of chunk blockDim.x bx + x of the kPackRowsInFlight rows y, y + blockDim.y, ... of
-// slab by, all loaded before the first is packed.
-template <typename CodeT>
+// codes of chunk blockDim.x bx + x of the U rows y, y + blockDim.y, ... of slab by, all loaded
+// before the first is packed.
+template <typename CodeT, int U>
 __global__ void __launch_bounds__(256) pack4_kernel(const CodeT* codes, int64_t R,
                                                     int64_t C, int64_t ld, uint8_t* out, int64_t ldp,
                                                     int vec, int* status) {
-  constexpr int U = kPackRowsInFlight;
   const int64_t c0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * kPackCodes;
   if (c0 >= C) return;
   const bool full = vec && c0 + kPackCodes <= C;
@@ -200,11 +197,10 @@ __global__ void __launch_bounds__(256) pack4_kernel(const CodeT* codes, int64_t 
   if (bad) atomicOr(status, kDevInternal);
 }
 
-template <typename CodeT>
+template <typename CodeT, int U>
 __global__ void __launch_bounds__(256) unpack4_kernel(const uint8_t* in, int64_t ldp,
                                                       int64_t R, int64_t C, CodeT* codes,
                                                       int64_t ld, int vec) {
-  constexpr int U = kPackRowsInFlight;
   const int64_t c0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * kPackCodes;
   if (c0 >= C) return;
   const bool full = vec && c0 + kPackCodes <= C;
@@ -265,19 +261,57 @@ __global__ void __launch_bounds__(256) unpack4_kernel(const uint8_t* in, int64_t
 }
 
 // A pack / unpack launch: blocks of 256 threads, bx chunks of 16 codes across by 256 / bx
-// rows, each thread taking kPackRowsInFlight rows of its column.  bx is the widest of 32, 16
-// and 8 that leaves the fewest threads past the row's end (2304 codes are 4.5 times 32 chunks
-// and 9 times 16).
-static void pack_shape(int64_t R, int64_t C, dim3* grid, dim3* block) {
+// rows, each thread taking `u` rows of its column.  bx is the widest of 32, 16 and 8 that leaves
+// the fewest threads past the row's end (2304 codes are 4.5 times 32 chunks and 9 times 16).
+// u is the largest of 1, 2, 4 and `most` that leaves two blocks for every SM: few blocks of many
+// rows each are a chain of loads on part of the chip, the more so where a row's last chunk goes
+// code by code.  Pack and unpack, E4M3, 1 / 2 / 4 / 8 rows: [1000, 300] 1.8 + 2.0, 2.2 + 2.4,
+// 3.1 + 3.6, 6.2 + 6.3 us; [12544, 256] 2.5 + 2.1, 1.9 + 2.1, 2.2 + 2.3, 3.2 + 2.7 us;
+// [12544, 2304] 12.1 + 12.6, 12.8 + 10.8, 12.3 + 9.8, 9.9 + 8.4 us.
+struct PackShape {
+  dim3 grid, block;
+  int u;
+};
+
+static int device_sms_or(int n) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return n;
+  return sms;
+}
+
+static PackShape pack_shape(int64_t R, int64_t C, int most) {
   const int64_t chunks = (C + kPackCodes - 1) / kPackCodes;
   int bx = 32;
   for (int b = 16; b >= 8; b /= 2)
     if ((chunks + b - 1) / b * b < (chunks + bx - 1) / bx * bx) bx = b;
-  const int64_t by = 256 / bx, slab = by * kPackRowsInFlight;
-  int64_t gy = (R + slab - 1) / slab;
+  const int64_t by = 256 / bx, gx = (chunks + bx - 1) / bx, want = 2 * device_sms_or(152);
+  int u = most;
+  while (u > 1 && gx * ((R + by * u - 1) / (by * u)) < want) u /= 2;
+  int64_t gy = (R + by * u - 1) / (by * u);
   if (gy > 65535) gy = 65535;   // the blocks then walk the rows
-  *grid = dim3(static_cast<unsigned>((chunks + bx - 1) / bx), static_cast<unsigned>(gy));
-  *block = dim3(static_cast<unsigned>(bx), static_cast<unsigned>(by));
+  return {dim3(static_cast<unsigned>(gx), static_cast<unsigned>(gy)),
+          dim3(static_cast<unsigned>(bx), static_cast<unsigned>(by)), u};
+}
+
+template <typename CodeT>
+static cudaError_t launch_pack(const void* codes, int64_t R, int64_t C, int64_t ld, uint8_t* packed, int64_t ldp,
+                               int vec, int* status, cudaStream_t s) {
+  // (BF16 codes: eight rows' words leave one block an SM; [12608, 3072] 20.5 us with 8, 18.6 with 4)
+  const PackShape p = pack_shape(R, C, sizeof(CodeT) == 1 ? 8 : 4);
+  auto kernel = p.u == 8 ? pack4_kernel<CodeT, sizeof(CodeT) == 1 ? 8 : 4> : p.u == 4 ? pack4_kernel<CodeT, 4>
+                : p.u == 2 ? pack4_kernel<CodeT, 2> : pack4_kernel<CodeT, 1>;
+  return launch_pdl(kernel, p.grid, p.block, s, static_cast<const CodeT*>(codes), R, C, ld, packed, ldp, vec, status);
+}
+
+template <typename CodeT>
+static cudaError_t launch_unpack(const uint8_t* packed, int64_t ldp, int64_t R, int64_t C, void* codes, int64_t ld,
+                                 int vec, cudaStream_t s) {
+  const PackShape p = pack_shape(R, C, 8);
+  auto kernel = p.u == 8 ? unpack4_kernel<CodeT, 8> : p.u == 4 ? unpack4_kernel<CodeT, 4>
+                : p.u == 2 ? unpack4_kernel<CodeT, 2> : unpack4_kernel<CodeT, 1>;
+  return launch_pdl(kernel, p.grid, p.block, s, packed, ldp, R, C, static_cast<CodeT*>(codes), ld, vec);
 }
 
 __device__ __forceinline__ int map_bits(int G) { return G <= 2 ? 1 : (G <= 4 ? 2 : 4); }
@@ -305,10 +339,7 @@ __global__ void __launch_bounds__(256) unpack_groups_kernel(const uint8_t* __res
 }
 
 static unsigned grid_for(int64_t items) {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    sms = 0;
+  const int sms = device_sms_or(0);
   int64_t b = (items + 255) / 256;
   const int64_t cap = sms > 0 ? static_cast<int64_t>(sms) * 16 : 65535;
   if (b > cap) b = cap;
@@ -339,15 +370,9 @@ extern "C" sq_status shiftquant_pack_codes(const void* codes, int64_t rows, int6
   const int vec = aligned16(codes) && (ld * cb) % 16 == 0 &&
                   (reinterpret_cast<uintptr_t>(packed) & 7u) == 0 && ld_packed % 8 == 0;
   cudaStream_t s = as_stream(stream);
-  dim3 grid, block;
-  pack_shape(rows, cols, &grid, &block);
-  cudaError_t err;
-  if (cb == 1)
-    err = launch_pdl(pack4_kernel<uint8_t>, grid, block, s, static_cast<const uint8_t*>(codes), rows, cols, ld,
-                     packed, ld_packed, vec, dev_status);
-  else
-    err = launch_pdl(pack4_kernel<uint16_t>, grid, block, s, static_cast<const uint16_t*>(codes), rows, cols, ld,
-                     packed, ld_packed, vec, dev_status);
+  const cudaError_t err =
+      cb == 1 ? launch_pack<uint8_t>(codes, rows, cols, ld, packed, ld_packed, vec, dev_status, s)
+              : launch_pack<uint16_t>(codes, rows, cols, ld, packed, ld_packed, vec, dev_status, s);
   return err == cudaSuccess ? SQ_OK : cuda_fail(err, "pack4_kernel launch");
 }
 
@@ -365,15 +390,8 @@ extern "C" sq_status shiftquant_unpack_codes(const uint8_t* packed, int64_t ld_p
   const int vec = aligned16(codes) && (ld * cb) % 16 == 0 &&
                   (reinterpret_cast<uintptr_t>(packed) & 7u) == 0 && ld_packed % 8 == 0;
   cudaStream_t s = as_stream(stream);
-  dim3 grid, block;
-  pack_shape(rows, cols, &grid, &block);
-  cudaError_t err;
-  if (cb == 1)
-    err = launch_pdl(unpack4_kernel<uint8_t>, grid, block, s, packed, ld_packed, rows, cols,
-                     static_cast<uint8_t*>(codes), ld, vec);
-  else
-    err = launch_pdl(unpack4_kernel<uint16_t>, grid, block, s, packed, ld_packed, rows, cols,
-                     static_cast<uint16_t*>(codes), ld, vec);
+  const cudaError_t err = cb == 1 ? launch_unpack<uint8_t>(packed, ld_packed, rows, cols, codes, ld, vec, s)
+                                  : launch_unpack<uint16_t>(packed, ld_packed, rows, cols, codes, ld, vec, s);
   return err == cudaSuccess ? SQ_OK : cuda_fail(err, "unpack4_kernel launch");
 }
 

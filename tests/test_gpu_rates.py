@@ -109,3 +109,26 @@ def test_layer_launch_with_ranges():
         times.append(sorted(ts)[len(ts) // 2])
     assert lay.status.item() == 0
     assert times[1] <= 1.5 * times[0], times
+
+
+# Rows of 300 codes end inside a chunk of sixteen, which goes code by code; with few rows of them a
+# thread must not take eight, one after another (three times as long as rows of whole chunks)
+def test_few_ragged_rows_pack_and_unpack():
+    def calls(C):
+        M, n, st = 1000, 48, torch.zeros(1, dtype=torch.int32, device="cuda")
+        codes, back = (L.empty_codes(M, C, 4, 4, "cuda").zero_() for _ in range(2))
+        packed = torch.zeros((M, (C + 1) // 2 + 15 & ~15), dtype=torch.uint8, device="cuda")
+        g = L.CapturedStep(lambda: [(N.shiftquant_pack_codes(codes, 4, 4, packed, st),
+                                     N.shiftquant_unpack_codes(packed, C, 4, 4, back)) for _ in range(n)])
+        ts = []
+        for _ in range(15):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            g.replay()
+            b.record()
+            b.synchronize()
+            ts.append(a.elapsed_time(b) / n * 1e3)
+        return sorted(ts)[len(ts) // 2]
+
+    ragged, whole = calls(300), calls(304)
+    assert ragged <= 2.2 * whole, (ragged, whole)
