@@ -1773,6 +1773,19 @@ static int coop_use(int64_t C) {
   return blocks >= gxo && blocks >= 8 ? blocks : 0;
 }
 
+// Where the cooperative form is the faster of the two that could serve a call (8-bit, cooperative
+// / resident): the backward of less than a million elements, whose few rows leave most of a
+// 1024-thread block idle -- [1000, 256] 12.0 / 13.9 us, [2000, 100] 14.9 / 16.5, [3136, 256]
+// 14.1 / 14.7, but [12544, 64] 16.6 / 16.6, [3136, 512] 17.0 / 16.7 -- except very few rows, which
+// need no sums across blocks ([100, 1000] 14.5 / 12.4); and the forward through the ring where rows
+// of x are not aligned or rows of codes not whole words ([200704, 61] 85 / 87, [200704, 64] from an
+// unaligned base 57.7 / 60.3).
+template <bool FWD>
+static bool coop_better(const L1bnArgs& a, bool fp32) {
+  if (FWD) return !fp32 && (!a.vec_in || (a.C & 3) != 0);
+  return a.R >= 256 && a.R * a.C < (int64_t(1) << 20);
+}
+
 // The first of the single-launch forms that serves the call and is not refused: the resident
 // form, then the cooperative one.  *launched: false where the call is left to the chain.
 template <bool FWD>
@@ -1781,9 +1794,11 @@ static int launch_single(const L1bnArgs& a, int G, int32_t* dev_status, cudaStre
   ResGeom g;
   bool fp32 = false;
   int st = SQ_OK;
-  if (res_plan<FWD>(a.R, a.C, &g, &fp32)) st = launch_res<FWD>(a, G, g, fp32, dev_status, s, launched);
+  const int blocks = coop_use<FWD>(a.C);
+  if (res_plan<FWD>(a.R, a.C, &g, &fp32) && !(blocks > 0 && coop_better<FWD>(a, fp32)))
+    st = launch_res<FWD>(a, G, g, fp32, dev_status, s, launched);
   if (st != SQ_OK || *launched) return st;
-  if (const int blocks = coop_use<FWD>(a.C)) st = launch_coop<FWD>(a, G, blocks, dev_status, s, launched);
+  if (blocks > 0) st = launch_coop<FWD>(a, G, blocks, dev_status, s, launched);
   return st;
 }
 

@@ -36,7 +36,7 @@ def call(lib, R, C, backward):
 @pytest.mark.parametrize("backward", [False, True])
 @pytest.mark.parametrize("C", [64, 2048])
 def test_resident_form_is_one_cooperative_launch(lib, C, backward):
-    st, ran = call(lib, 3136, C, backward)
+    st, ran = call(lib, 20000, C, backward) if C == 64 else call(lib, 3136, C, backward)
     assert st == N.SQ_OK and len(ran) == 1
     assert ran[0][0] == f"l1bn_{'bwd' if backward else 'fwd'}_res_kernel" and ran[0][2] == "c"
 
@@ -53,11 +53,11 @@ def test_refused_launch_goes_on_with_the_next_form(lib, backward, error):
     assert lib.fake_last_error() == 0
     # the resident form's blocks alone do not fit: the cooperative form
     lib.fake_refuse(error, 1)
-    st, ran = call(lib, 3136, 64, backward)
+    st, ran = call(lib, 20000, 64, backward)
     assert st == N.SQ_OK and [k[0] for k in ran] == [f"l1bn_{d}_coop_kernel"]
     # no cooperative launch at all
     lib.fake_refuse(error, 2)
-    st, ran = call(lib, 3136, 64, backward)
+    st, ran = call(lib, 20000, 64, backward)
     assert st == N.SQ_OK and [k[0] for k in ran] == chain
     assert lib.fake_last_error() == 0
 
@@ -68,6 +68,18 @@ def test_other_errors_are_reported(lib):
     assert st == N.SQ_ECUDA and ran == []
     lib.fake_refuse(0, 0)
     lib.cudaGetLastError()
+
+
+# few rows of a backward, and a forward whose rows of codes are not whole words: the cooperative form
+@pytest.mark.parametrize("R,C,backward,form", [(1000, 256, True, "l1bn_bwd_coop_kernel"),
+                                               (255, 256, True, "l1bn_bwd_res_kernel"),
+                                               (1000, 256, False, "l1bn_fwd_res_kernel"),
+                                               (200704, 61, False, "l1bn_fwd_coop_kernel"),
+                                               (200704, 61, True, "l1bn_bwd_res_kernel"),
+                                               (3136, 1025, True, "l1bn_bwd_res_kernel")])
+def test_form_of_a_shape(lib, R, C, backward, form):
+    st, ran = call(lib, R, C, backward)
+    assert st == N.SQ_OK and [k[0] for k in ran] == [form]
 
 
 # a whole tensor and a ring of rows on the SMs, too many rows for that, few channels, and more
