@@ -1777,13 +1777,14 @@ static int coop_use(int64_t C) {
 // / resident): the backward of less than a million elements, whose few rows leave most of a
 // 1024-thread block idle -- [1000, 256] 12.0 / 13.9 us, [2000, 100] 14.9 / 16.5, [3136, 256]
 // 14.1 / 14.7, but [12544, 64] 16.6 / 16.6, [3136, 512] 17.0 / 16.7 -- except very few rows, which
-// need no sums across blocks ([100, 1000] 14.5 / 12.4); and the forward through the ring where rows
-// of x are not aligned or rows of codes not whole words ([200704, 61] 85 / 87, [200704, 64] from an
-// unaligned base 57.7 / 60.3).
+// need few sums across blocks ([100, 1000] 14.5 / 12.4), and rows of codes that are not whole
+// words ([12544, 61] 20.7 / 18.7); and the forward through the ring where rows of x are not aligned
+// or rows of codes not whole words ([200704, 61] 85 / 87, [200704, 64] from an unaligned base
+// 57.7 / 60.3).
 template <bool FWD>
 static bool coop_better(const L1bnArgs& a, bool fp32) {
   if (FWD) return !fp32 && (!a.vec_in || (a.C & 3) != 0);
-  return a.R >= 256 && a.R * a.C < (int64_t(1) << 20);
+  return a.R >= 256 && (a.C & 3) == 0 && a.R * a.C < (int64_t(1) << 20);
 }
 
 // The first of the single-launch forms that serves the call and is not refused: the resident

@@ -73,6 +73,7 @@ def test_other_errors_are_reported(lib):
 # few rows of a backward, and a forward whose rows of codes are not whole words: the cooperative form
 @pytest.mark.parametrize("R,C,backward,form", [(1000, 256, True, "l1bn_bwd_coop_kernel"),
                                                (255, 256, True, "l1bn_bwd_res_kernel"),
+                                               (12544, 61, True, "l1bn_bwd_res_kernel"),
                                                (1000, 256, False, "l1bn_fwd_res_kernel"),
                                                (200704, 61, False, "l1bn_fwd_coop_kernel"),
                                                (200704, 61, True, "l1bn_bwd_res_kernel"),
