@@ -27,6 +27,7 @@
 // before it (programmatic stream serialization).
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstring>
 
 #include "sq_device.cuh"
@@ -1608,10 +1609,10 @@ static int launched(const char* what) {
 // block of a cooperative launch must be resident at once), 0 where it cannot run.
 template <bool FWD>
 static int coop_blocks() {
-  static int cached[64][2];   // [device][fwd]: blocks + 1, 0 = not asked yet
+  static std::atomic<int> cached[64][2];   // [device][fwd]: blocks + 1, 0 = not asked yet (any thread may ask)
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  int& slot = cached[dev][FWD ? 1 : 0];
+  int slot = cached[dev][FWD ? 1 : 0].load(std::memory_order_acquire);
   if (slot == 0) {
     int coop = 0, sms = 0, per_sm = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
@@ -1624,6 +1625,7 @@ static int coop_blocks() {
     else
       slot = 1;
     cudaGetLastError();
+    cached[dev][FWD ? 1 : 0].store(slot, std::memory_order_release);
   }
   return slot - 1;
 }
@@ -1687,10 +1689,11 @@ static int launch_coop(const L1bnArgs& a, int G, int blocks, int32_t* dev_status
 // device runs no cooperative launches.
 template <bool FWD>
 static bool res_plan(int64_t R, int64_t C, ResGeom* g, bool* fp32) {
-  static int cached[64];   // [device]: SMs + 1, 0 = not asked yet
+  static std::atomic<int> cached[64];   // [device]: SMs + 1, 0 = not asked yet (any thread may ask)
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
-  if (cached[dev] == 0) {
+  int known = cached[dev].load(std::memory_order_acquire);
+  if (known == 0) {
     int coop = 0, sms = 0, smem = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1705,9 +1708,10 @@ static bool res_plan(int64_t R, int64_t C, ResGeom* g, bool* fp32) {
       ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kResDyn)) == cudaSuccess &&
            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kResThreads, kResDyn) == cudaSuccess && per_sm >= 1;
     cudaGetLastError();
-    cached[dev] = ok ? sms + 1 : 1;
+    known = ok ? sms + 1 : 1;
+    cached[dev].store(known, std::memory_order_release);   // after the kernels' attributes are set
   }
-  const int sms = cached[dev] - 1;
+  const int sms = known - 1;
   double best = 0.0;
   const int widest = tile_lg(C) < 4 ? tile_lg(C) : 4;
   for (int lgq = widest; lgq >= (widest < 2 ? widest : 2); --lgq) {

@@ -1,6 +1,7 @@
 """Which launches an L1 batch norm call makes, on the host alone (no GPU): the resident form, and
 what follows where the device refuses a cooperative launch."""
 import ctypes
+from concurrent.futures import ThreadPoolExecutor
 
 import pytest
 
@@ -99,3 +100,12 @@ def test_launch_query_at_its_edges(lib):
     # no rows, and any number of rows
     assert lib.shiftquant_l1bn_launches(0, 64, 0) == lib.shiftquant_l1bn_kernel_launches(64, 0) == 1
     assert lib.shiftquant_l1bn_kernel_launches(1025, 0) == 9 and lib.shiftquant_l1bn_kernel_launches(1025, 1) == 7
+
+
+def test_threads_ask_for_the_plan_together(tmp_path):
+    # a library nobody has called yet, from sixteen threads at once
+    lib = fake_cudart.link(tmp_path)
+    with ThreadPoolExecutor(16) as ex:
+        got = list(ex.map(lambda i: lib.shiftquant_l1bn_launches(300000 if i % 2 else 3136, 1025, i // 2 % 2),
+                          range(64)))
+    assert got == [(1, 9, 1, 7)[i % 4] for i in range(64)]
