@@ -354,8 +354,9 @@ typedef struct {
 
 /* workspace: optional int32 scratch of shiftquant_gemm_layer_workspace_bytes() bytes,
  * 16-byte aligned.  Its first 256 bytes hold the counter through which the CTAs take their
- * work units as they free up (the units of the three GEMMs differ in length); without a
- * workspace each CTA strides over the unit list.  After it, each GEMM with too few output
+ * work units as they free up (the units of the three GEMMs differ in length) and, in a layer
+ * step, the largest magnitudes of X and dY; without a workspace each CTA strides over the unit
+ * list.  After it, each GEMM with too few output
  * tiles for the SMs splits its K loop into its own region -- into fewer parts than alone,
  * as the other GEMMs of the launch keep the SMs busy. */
 sq_status shiftquant_gemm_layer(const sq_layer_gemms *args, void *workspace,
@@ -406,8 +407,7 @@ int shiftquant_gemm_layer_wgrad_in_place(int64_t M, int64_t K, int64_t N, int bi
  *          likewise);
  *   3. W per out-channel (forward role): codes written transposed [N, K] with X's group
  *      shifts folded in; W per in-channel (loss-propagation role): codes [K, N] with dY's
- *      shifts folded in -- both roles by shiftquant_calibrate_weight and
- *      shiftquant_quantize_weight;
+ *      shifts folded in -- both roles from one read of W for the ranges and one for the codes;
  *   4. the forward, loss-propagation and weight-gradient GEMMs as one launch
  *      (shiftquant_gemm_layer).
  * Every buffer is a caller-owned DEVICE buffer; the layouts are those of the calls above:
@@ -419,10 +419,13 @@ int shiftquant_gemm_layer_wgrad_in_place(int64_t M, int64_t K, int64_t N, int bi
  *     g_scale; wf_codes [N, ld_wf], wf_range[N], wf_scale[N]; wd_codes [K, ld_wd],
  *     wd_range[K], wd_scale[K].  Codes in the type of shiftquant_code_type(bits, n_groups),
  *     rows 16-byte aligned (ld * code bytes a multiple of 16, pointers 16-byte aligned).
- *   workspace: optional, as for shiftquant_gemm_layer (shiftquant_gemm_layer_workspace_bytes).
+ *   workspace: optional, as for shiftquant_gemm_layer (shiftquant_gemm_layer_workspace_bytes);
+ *     written from the step's first launch on.  With at least its 256 bytes the quantizer passes
+ *     of the three tensors run together -- one launch for every range, one launch or three
+ *     beside one another for the codes -- else one library call after another (the same results).
  *   dev_status: the device status word (see the conventions above).
- * The struct lives in host memory and is read during the call only.  The quantizer and GEMM
- * launches run one after the other on `stream`; M, K or N == 0 does nothing. */
+ * The struct lives in host memory and is read during the call only.  Everything is launched on
+ * `stream`: later work on it sees the whole step done; M, K or N == 0 does nothing. */
 typedef struct {
   int64_t M, K, N;
   int bits, n_groups;

@@ -29,8 +29,8 @@
 //               tile, ahead of the epilogue
 //   warps 4-11  epilogue: tcgen05.ld, int32 accumulation across chunks, dequantizing
 //               multiply, TMA stores of 32 x 32 boxes (or int32 TMA reductions into a
-//               split-K workspace; plain stores where
-//               the output rows are not 16-byte aligned)
+//               split-K workspace; plain stores where the output rows are not 16-byte
+//               aligned)
 // Work units reach the roles through a small shared-memory ring that the producer of the
 // CTA (a pair's leader) fills: with a scheduling counter it takes each next unit from it
 // (units are handed out in list order as CTAs free up), without one it strides over the
@@ -1295,7 +1295,7 @@ static int make_output_map(CUtensorMap* map, void* base, int64_t rows, int64_t c
   return SQ_OK;
 }
 
-static int device_sms(int* dev_out) {
+int device_sms(int* dev_out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   int n = 0;
@@ -1695,7 +1695,7 @@ struct JobPlan {
 // CTAs take their units as they free up -- for batches whose units differ in length.
 // Without one each CTA strides over the unit list.
 // counter_zeroed: the caller clears the counter word itself, it is not among the regions.
-// *live is false when there is nothing to launch.
+// *have is false when there is nothing to launch.
 static int plan_jobs(GemmJob* jobs, int njobs, int bits, int G, int32_t* dev_status, cudaStream_t s,
                      int* sched, int max_ctas, bool no_copies, bool counter_zeroed, JobPlan* jp, bool* have) {
   *have = false;

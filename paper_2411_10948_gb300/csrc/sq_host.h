@@ -35,6 +35,9 @@ inline int code_bytes(int type) { return type == SQ_CODE_E4M3 ? 1 : 2; }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// SMs of the current device (its index to *dev_out unless null), -1 without one
+int device_sms(int* dev_out);
+
 inline cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 
 // ------------------------------------------------------------ one layer step's parts
@@ -48,9 +51,10 @@ struct ZeroRegion {
 int check_layer_quant(const sq_layer_step* L);
 // whether the passes of quantize_layer can index the layer's tiles
 bool layer_quant_fits(const sq_layer_step* L);
-// The quantizer passes of a checked layer step in three launches, and the zero regions
-// cleared.  words: 256 bytes of device memory, of which the first 64 are left zero and the
-// rest is the passes' own.
+// The quantizer passes of a checked layer step -- zeroed accumulators, ranges, codes: three
+// launches, five where the codes of a large layer are three -- and the zero regions cleared.
+// words: 256 bytes of device memory, of which the first 64 are left zero and the rest is the
+// passes' own.
 int quantize_layer(const sq_layer_step* L, uint64_t seed, unsigned* words, const ZeroRegion* zero, int nzero,
                    cudaStream_t s);
 

@@ -273,20 +273,12 @@ struct PackShape {
   int u;
 };
 
-static int device_sms_or(int n) {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-    return n;
-  return sms;
-}
-
 static PackShape pack_shape(int64_t R, int64_t C, int most) {
   const int64_t chunks = (C + kPackCodes - 1) / kPackCodes;
   int bx = 32;
   for (int b = 16; b >= 8; b /= 2)
     if ((chunks + b - 1) / b * b < (chunks + bx - 1) / bx * bx) bx = b;
-  const int64_t by = 256 / bx, gx = (chunks + bx - 1) / bx, want = 2 * device_sms_or(152);
+  const int64_t by = 256 / bx, gx = (chunks + bx - 1) / bx, want = 2 * static_cast<int64_t>(device_sms(nullptr));
   int u = most;
   while (u > 1 && gx * ((R + by * u - 1) / (by * u)) < want) u /= 2;
   int64_t gy = (R + by * u - 1) / (by * u);
@@ -339,7 +331,7 @@ __global__ void __launch_bounds__(256) unpack_groups_kernel(const uint8_t* __res
 }
 
 static unsigned grid_for(int64_t items) {
-  const int sms = device_sms_or(0);
+  const int sms = device_sms(nullptr);
   int64_t b = (items + 255) / 256;
   const int64_t cap = sms > 0 ? static_cast<int64_t>(sms) * 16 : 65535;
   if (b > cap) b = cap;

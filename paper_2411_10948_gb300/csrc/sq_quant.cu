@@ -455,21 +455,6 @@ static int tile_lg(int64_t C) {
   return 3;
 }
 
-template <typename CodeT>
-__device__ __forceinline__ CodeT encode_code(float v);
-
-template <>
-__device__ __forceinline__ uint16_t encode_code<uint16_t>(float v) {
-  // v is an integer with at most 8 significant bits: the top half of its binary32
-  // pattern is its exact BF16 pattern
-  return static_cast<uint16_t>(__float_as_uint(v) >> 16);
-}
-
-template <>
-__device__ __forceinline__ uint8_t encode_code<uint8_t>(float v) {
-  return static_cast<uint8_t>(__nv_cvt_float_to_fp8(v, __NV_SATFINITE, __NV_E4M3));
-}
-
 // n codes as 32-bit words, the first code in the low bits
 template <typename CodeT, int N>
 __device__ __forceinline__ void encode_words(const float (&q)[N], uint32_t (&w)[N * sizeof(CodeT) / 4]) {
@@ -1204,9 +1189,9 @@ static void launch_quantize(const QuantArgs& a, int gran, int mode, dim3 grid, c
 // Both roles of a weight from one pass over it (Sec. 5.1): the forward GEMM's
 // per-out-channel codes (gran PER_COL, written transposed, the fold indexed by row) and loss
 // propagation's per-in-channel codes (gran PER_ROW, natural layout, the fold indexed by
-// column), both from the one load of the block's tile into shared memory.  Re-reading the
-// tile for the second role (from L2) put a second load latency in every block: 87 us for
-// large_linear's [4096, 11008] weight against 76 us with the tile kept.
+// column), both from one load of the block's tile, held in registers (in shared memory on the
+// general path).  Bound by HBM with four blocks an SM: a [4096, 11008] weight, 8-bit, takes 63.5
+// us, of which 42.8 for the transposed codes alone and 40.2 for the others.
 template <typename CodeT, int FORM, bool FF, bool FD, bool WAIT = false>
 __device__ __forceinline__ void quantize_weight_block(const QuantArgs& af, const QuantArgs& ad, unsigned bx,
                                                       unsigned by, uint32_t tile_smem) {
@@ -1265,11 +1250,26 @@ static void launch_quantize_weight(const QuantArgs& af, const QuantArgs& ad, dim
 
 // ============================================================= a layer's quantizer passes
 // The quantizer passes of a layer step (X, dY and W: three tensors, eleven launches one by
-// one, each short next to its launch gap and its last wave) as three launches: the
-// accumulators zeroed, every tensor's range pass, every tensor's quantization.  The grouping
-// needs no launch of its own: the range pass also keeps tau_0 (kTauSlots words per tensor),
-// and a quantizer block forms the exponents of its own columns, and the shifts it folds into
-// weight codes, from the ranges and tau_0.
+// one, each short next to its launch gap and its last wave) as one launch each: the
+// accumulators zeroed, every tensor's range pass, every tensor's codes (three launches beside one
+// another for large layers).  The grouping needs no launch of its own: the range pass also keeps
+// tau_0 (kTauSlots words per tensor), and a quantizer block forms the exponents of its own
+// columns, and the shifts it folds into weight codes, from the ranges and tau_0.
+//
+// What a launch of this chain may rely on.  Each is launched behind the one before it and starts
+// when every block of that one has let it (griddep_launch_dependents) or has ended:
+//   layer_init     waits for whatever precedes it, only then lets the range pass start -- so x,
+//                  dy and w are complete when that starts, and it reads them before its own wait;
+//   layer_range    waits (for the zeroed accumulators) before its first atomic, and lets the codes
+//                  start after that wait;
+//   codes, first   layer_quantize loads x early and waits before anything the range pass wrote;
+//                  quantize_kernel of X waits first, and only then lets the next one start;
+//   codes, beside  those of W and dY read x, ranges and tau_0 (past L1) without a wait: the launch
+//                  before them was let go by one that had waited for the range pass.  Their wait
+//                  comes last, so that whoever waits for dY's launch has waited for all three;
+//   GEMM           waits before everything.
+// A kernel put between two of these must wait before it lets the next one start, and a launch
+// that writes x, dy, w or the ranges must not come after layer_init.
 struct LayerInit {
   unsigned* p[5];
   int64_t n[5];
@@ -1660,17 +1660,17 @@ bool layer_quant_fits(const sq_layer_step* L) {
 }
 
 // The codes of a layer's tensors: one launch while its blocks stay within two resident waves
-// (four blocks on each of 152 SMs), where launches and their tails are what counts; above, one
-// launch per tensor, each running beside the tail of the one before it, each body with the
-// instruction cache and the registers to itself.  Whole steps, one launch against three:
+// (four blocks on each SM), where launches and their tails are what counts; above, one launch per
+// tensor, each running beside the tail of the one before it, each body with the instruction cache
+// and the registers to itself.  Whole steps when the line was drawn, one launch against three:
 // 256 x 512 x 512 (4-bit) 24.7 / 26.6 us; 12608 x 768 x 3072 (6-bit) 271 / 261 us,
 // 4096 x 11008 x 4096 (8-bit) 957 / 939 us (with the three one after another 123 us where
 // beside one another take 115 us: 12544 x 2304 x 256, 4-bit).
-constexpr unsigned kLayerQuantMaxBlocks = 8 * 152;
+constexpr int kLayerQuantWaveBlocks = 8;   // an SM's, in two waves
 
 template <typename CodeT>
-static cudaError_t launch_layer_quantize(const LayerQuant& q, unsigned blocks, cudaStream_t s) {
-  if (blocks > kLayerQuantMaxBlocks) {
+static cudaError_t launch_layer_quantize(const LayerQuant& q, unsigned blocks, int sms, cudaStream_t s) {
+  if (blocks > static_cast<unsigned>(kLayerQuantWaveBlocks * sms)) {
     QuantArgs g = q.g, wf = q.wf;
     g.beside = wf.beside = 1;
     launch_quantize<CodeT>(q.x, SQ_GRAN_SHIFT, SQ_ROUND_NEAREST_EVEN, quant_grid(q.x), s);
@@ -1687,6 +1687,8 @@ int quantize_layer(const sq_layer_step* L, uint64_t seed, unsigned* words, const
                    cudaStream_t s) {
   const int64_t M = L->M, K = L->K, N = L->N;
   const int cbytes = code_bytes(code_type(L->bits, L->n_groups));
+  const int sms = device_sms(nullptr);
+  if (sms <= 0) return fail(SQ_ECUDA, "layer_step: no current CUDA device");
   unsigned* xtau = words + kTauSlots;
   unsigned* gtau = words + 2 * kTauSlots;
   auto bits = [](float* p) { return reinterpret_cast<unsigned*>(p); };
@@ -1695,7 +1697,7 @@ int quantize_layer(const sq_layer_step* L, uint64_t seed, unsigned* words, const
                  {K, N, N, K, 3 * kTauSlots}};
   const int64_t widest = K > N ? K : N;
   const int64_t ib = (widest + 255) / 256;
-  cudaError_t err = launch_pdl(layer_init_kernel, dim3(static_cast<unsigned>(ib < 152 ? ib : 152)), dim3(256), s, z);
+  cudaError_t err = launch_pdl(layer_init_kernel, dim3(static_cast<unsigned>(ib < sms ? ib : sms)), dim3(256), s, z);
   if (err != cudaSuccess) return cuda_fail(err, "layer_init_kernel launch");
   // 2. ranges
   LayerRange r;
@@ -1769,8 +1771,8 @@ int quantize_layer(const sq_layer_step* L, uint64_t seed, unsigned* words, const
   q.xend = xg.x * xg.y;
   q.wend = q.xend + wg.x * wg.y;
   const unsigned nb = q.wend + gg.x * gg.y;
-  err = code_type(L->bits, L->n_groups) == SQ_CODE_E4M3 ? launch_layer_quantize<uint8_t>(q, nb, s)
-                                                        : launch_layer_quantize<uint16_t>(q, nb, s);
+  err = code_type(L->bits, L->n_groups) == SQ_CODE_E4M3 ? launch_layer_quantize<uint8_t>(q, nb, sms, s)
+                                                        : launch_layer_quantize<uint16_t>(q, nb, sms, s);
   return err == cudaSuccess ? SQ_OK : cuda_fail(err, "layer_quantize_kernel launch");
 }
 
