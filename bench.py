@@ -702,10 +702,9 @@ def run_chain(args, dev, flush_steps=None):
 
 
 L1BN_SHAPES = (("resnet_stage1", 64 * 56 * 56, 64), ("resnet_stage3", 64 * 14 * 14, 256))
-# HBM bytes per element of the passes (fp32 in / out, 1-byte codes): forward = range pass 4,
-# quantize + code sums 4 + 1, deviation sums 1, output 1 + 4; backward = range pass 4,
-# quantize + sums 4 + 1 (x codes) + 1 (gradient codes), output 1 + 1 + 4
-L1BN_FWD_BYTES, L1BN_BWD_BYTES = 15, 16
+# HBM bytes per element that a call cannot do without: x (dy) read once and y (dx) written once,
+# fp32.  What a form moves beyond that (1-byte codes, a second read of the input) is its own cost.
+L1BN_FWD_BYTES, L1BN_BWD_BYTES = 8, 8
 
 
 def run_l1bn(args, dev):
@@ -757,6 +756,7 @@ def run_l1bn(args, dev):
                     "bwd_frac": bg / peaks["hbm_gbs"], "launches": launches})
     return {"bits": 8, "n_groups": 4, "bytes_per_element": {"fwd": L1BN_FWD_BYTES,
                                                            "bwd": L1BN_BWD_BYTES},
+            "bytes_basis": "input read once, output written once (fp32)",
             "peak": peaks["hbm_gbs"], "peak_source": f"{src} copy bandwidth",
             "statistic": "median over graph replays after an L2 flush", "shapes": out}
 

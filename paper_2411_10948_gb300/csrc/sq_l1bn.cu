@@ -972,9 +972,10 @@ __global__ void __launch_bounds__(kL1Threads, 2) l1bn_bwd_coop_kernel(const L1bn
 // results are the same bit for bit.
 // Bound by instruction issue on top of its traffic: about 55 instructions an element in the
 // forward and 89 in the backward (two 64-bit multiplies of the generator among them), on one
-// block per SM whose phases wait at 2-4 grid barriers of about 1.5 us.  Forward and backward
-// together, 8-bit, the cooperative form (or, above 1024 channels, the chain) before and this
-// form now: [200704, 64] 129 and 109 us (ring), [3136, 2048] 115 and 80 us (whole).
+// block per SM whose phases wait at 2-4 grid barriers (forward) and 1-2 (backward) of about 1.5
+// us.  Forward and backward together, 8-bit, the cooperative form (or, above 1024 channels, the
+// chain) before and this form now: [200704, 64] 129 and 109 us (ring), [3136, 2048] 115 and 82 us
+// (whole).
 constexpr int kResThreads = 1024;
 constexpr int kResWarps = kResThreads / 32;
 constexpr int kResRing = 6;   // 96 KB a block in flight or resident

@@ -52,9 +52,10 @@ static sq_layer_gemms step_gemms(const sq_layer_step* L) {
 // The device part of the step, in stream order on s, with a usable workspace: the quantizer
 // passes of the three tensors together (quantize_layer), which also zero what the GEMMs need,
 // then the GEMM launch behind them.  Against one library call after another (fourteen
-// launches): 256 x 512 x 512 (4-bit) 59.3 -> 24.2 us a step, 12544 x 2304 x 256 (4-bit)
-// 139 -> 114 us, 5003 x 1155 x 1001 (6-bit) 138 -> 105 us, 12608 x 768 x 3072 (6-bit)
-// 286 -> 259 us, 4096 x 11008 x 4096 (8-bit) 967 -> 938 us.
+// launches), when the passes were put together: 256 x 512 x 512 (4-bit) 59.3 -> 24.2 us a step,
+// 12544 x 2304 x 256 (4-bit) 139 -> 114 us, 5003 x 1155 x 1001 (6-bit) 138 -> 105 us,
+// 12608 x 768 x 3072 (6-bit) 286 -> 259 us, 4096 x 11008 x 4096 (8-bit) 967 -> 938 us; now 21.3,
+// 105, 89, 242 and 901 us.
 static int run_step_fused(const sq_layer_step* L, uint64_t seed, void* s) {
   int st = check_layer_quant(L);
   if (st != SQ_OK) return st;
